@@ -22,9 +22,12 @@ struct Cfg {
   static constexpr int kStages = M == 4 ? 3 : 2;  // 192 KB (M = 4), 96 KB + 72 KB step history (M = 8)
   static constexpr int kMinBlocks = 1;
   static constexpr int kTile = 2 * kPairs * kThreads * M;  // elements
-  // groups out of the fast path's range, queued per warp (DeferredGroups): at most
-  // 64 kPairs a tile on top of fewer than 32 left from earlier tiles
-  static constexpr int kDeferCap = 32 + 64 * kPairs;
+  // Groups out of the fast path's range: queued per warp (DeferredGroups) at M = 4, where
+  // it measured 2.7 % faster at tau = 1 on the 7B-shaped set, in place at M = 8 (at
+  // tau = 0.5 the queue's code measured 3 % slower).  The queue holds at most 64 kPairs a
+  // tile on top of fewer than 32 left from earlier tiles.
+  static constexpr bool kDefer = M == 4;
+  static constexpr int kDeferCap = kDefer ? 32 + 64 * kPairs : 0;
 };
 // Tensors of one multi-tensor launch, at most (its parameter block holds them all).
 constexpr int kMultiMaxBwd = 192;
@@ -201,8 +204,7 @@ __device__ __forceinline__ void bwd_inputs(const float* const* phi_g, const uint
 // whole history stays in registers.  With HIST (M = 8) registers are tight:
 // the keys die after the forward relaxation (a flagged group re-forms them) and
 // the upstream gradients are formed only for the sweep.
-template <int N, int M, bool TAU1, class V, bool HIST = false, bool ST = false, bool OPT = false,
-          bool NARROW = false, bool DEFER = false>
+template <int N, int M, bool TAU1, class V, bool HIST, bool ST, bool OPT, bool NARROW, bool DEFER, bool WIDE>
 __device__ __forceinline__ uint32_t bwd_groups(const float* const* phi_g, const uint16_t* const* W_g,
                                            const uint16_t* const* dWm_g, const int64_t* e0, const uint32_t* q0,
                                            const BwdArgs& a, const BwdOptArgs& o, V* hist = nullptr) {
@@ -253,7 +255,7 @@ __device__ __forceinline__ uint32_t bwd_groups(const float* const* phi_g, const 
       }
   }
   using Steps = typename std::conditional<HIST, SmemSteps<N, M, V, Cfg<M>::kThreads>, RegSteps<N, M, V>>::type;
-  FastGroup<N, M, TAU1, true, V, Steps> fg;
+  FastGroup<N, M, TAU1, true, V, Steps, WIDE> fg;
   if constexpr (HIST) fg.st.at = hist;
   V kap[HIST ? 1 : M], c[M], dkv[M];
   if constexpr (HIST) {
@@ -327,7 +329,7 @@ __device__ __forceinline__ uint32_t bwd_groups(const float* const* phi_g, const 
       }
 #pragma unroll
       for (int l = 0; l < M; ++l) cc[l] = lane_of(c[l], h);
-      if (!TAU1 && all_finite(k)) {
+      if (!TAU1 && !WIDE && all_finite(k)) {
         RobustGroup<N, M> rg;  // finite keys spread beyond the fast path's float range (as roi_fwd.cu)
         rg.forward(k, a.inv_tau, S);
         rg.backward(cc, a.inv_tau, dk);
@@ -379,10 +381,10 @@ __device__ __forceinline__ uint32_t bwd_groups(const float* const* phi_g, const 
 }
 
 // The exact routine for one group out of the fast path's range (first element g0,
-// call-flat), from global memory (as fwd_exact_group): dphi, the fused AdamW step
+// call-flat), from global memory: dphi, the fused AdamW step
 // (the fast path left this group's logits and moments untouched) and, unless
 // straight-through, dW = bf16(dWm * S).
-template <int N, int M, bool TAU1, bool ST, bool OPT>
+template <int N, int M, bool ST, bool OPT>
 __device__ __forceinline__ void bwd_exact_group(int64_t g0, const BwdArgs& a, const BwdOptArgs& o) {
   // keys and upstream gradients as the tiles' packed code forms them (the group in
   // both halves)
@@ -396,17 +398,11 @@ __device__ __forceinline__ void bwd_exact_group(int64_t g0, const BwdArgs& a, co
   float k[M], cc[M], S[M], dk[M];
 #pragma unroll
   for (int l = 0; l < M; ++l) k[l] = lo(k2[l]), cc[l] = lo(c2[l]);
-  if (!TAU1 && all_finite(k)) {
-    RobustGroup<N, M> rg;
-    rg.forward(k, a.inv_tau, S);
-    rg.backward(cc, a.inv_tau, dk);
-  } else {
 #pragma unroll
-    for (int l = 0; l < M; ++l) k[l] *= kLn2;  // natural-log keys
-    ExactGroup<N, M> ex;
-    ex.forward(k, N, M, a.tau, S);
-    ex.backward(cc, N, M, a.tau, dk);
-  }
+  for (int l = 0; l < M; ++l) k[l] *= kLn2;  // natural-log keys
+  ExactGroup<N, M> ex;
+  ex.forward(k, N, M, a.tau, S);
+  ex.backward(cc, N, M, a.tau, dk);
 #pragma unroll
   for (int l = 0; l < M; ++l) dk[l] = __fmul_rn(dk[l], a.np.inv_lam);
 #pragma unroll
@@ -430,7 +426,7 @@ __device__ __forceinline__ void bwd_exact_group(int64_t g0, const BwdArgs& a, co
 // memory.  NARROW: the call's counters are below 2^32 (a.np.narrow).
 // `tag` (the tensor's index in a multi-tensor launch, shifted to bit 48) is or-ed into
 // the queued entries.
-template <int N, int M, bool TAU1, bool ST, bool OPT, bool NARROW, bool DEFER, class Defer, class Exact>
+template <int N, int M, bool TAU1, bool ST, bool OPT, bool NARROW, bool WIDE, class Defer, class Exact>
 __device__ __forceinline__ void bwd_tile(const uint8_t* const* stage, int64_t tile, const BwdArgs& a,
                                          const BwdOptArgs& o, uint8_t* smem, Defer& dg, int64_t tag,
                                          const Exact& exact) {
@@ -451,24 +447,24 @@ __device__ __forceinline__ void bwd_tile(const uint8_t* const* stage, int64_t ti
     const uint32_t q0[2] = {qt + uint32_t(g0 * (M / 4)), qt + uint32_t(g1 * (M / 4))};
     uint32_t flag;
     if constexpr (M == 4) {
-      flag = bwd_groups<N, M, TAU1, F2, false, ST, OPT, NARROW, DEFER>(pp, pw, pd, e0, q0, a, o);
+      flag = bwd_groups<N, M, TAU1, F2, false, ST, OPT, NARROW, C::kDefer, WIDE>(pp, pw, pd, e0, q0, a, o);
     } else {
       // M = 8: the paired step history does not fit the register file; steps
       // 0 .. N-2 go to shared memory behind the tile ring
       F2* hist = reinterpret_cast<F2*>(smem + kHistOffset<M>) + threadIdx.x;
-      flag = bwd_groups<N, M, TAU1, F2, true, ST, OPT, NARROW, DEFER>(pp, pw, pd, e0, q0, a, o, hist);
+      flag = bwd_groups<N, M, TAU1, F2, true, ST, OPT, NARROW, C::kDefer, WIDE>(pp, pw, pd, e0, q0, a, o, hist);
     }
-    if constexpr (DEFER) {
+    if constexpr (C::kDefer) {
       dg.push((flag & 1u) != 0u, tag | e0[0]);
       dg.push((flag & 2u) != 0u, tag | e0[1]);
     }
   }
-  if constexpr (DEFER) dg.drain(false, exact);
+  if constexpr (C::kDefer) dg.drain(false, exact);
 }
 
 // The ragged tail of a tensor (fewer than one tile after its full tiles), by one
 // CTA, straight from global memory.
-template <int N, int M, bool TAU1, bool ST, bool OPT>
+template <int N, int M, bool TAU1, bool ST, bool OPT, bool WIDE>
 __device__ __forceinline__ void bwd_tail(const BwdArgs& a, const BwdOptArgs& o) {
   using C = Cfg<M>;
   const int64_t t0 = a.full_tiles * C::kTile;
@@ -478,7 +474,7 @@ __device__ __forceinline__ void bwd_tail(const BwdArgs& a, const BwdOptArgs& o) 
     const uint16_t* pw[1] = {a.W + t0 + gi * M};
     const uint16_t* pd[1] = {a.dWm + t0 + gi * M};
     const int64_t e0[1] = {t0 + gi * M};
-    bwd_groups<N, M, TAU1, float, false, ST, OPT>(pp, pw, pd, e0, nullptr, a, o);
+    bwd_groups<N, M, TAU1, float, false, ST, OPT, false, false, WIDE>(pp, pw, pd, e0, nullptr, a, o);
   }
 }
 
@@ -488,7 +484,7 @@ __device__ __forceinline__ void bwd_tail(const BwdArgs& a, const BwdOptArgs& o) 
 // counters): every M = 4 variant, and the 4:8 tau = 1 backward fused with AdamW (at
 // 4:8 the narrow plain backward spilled, 225 against 192 us per 18944 x 3584
 // tensor, while the fused one gained, 386 against 418 us)
-template <int N, int M, bool TAU1, bool ST, bool OPT, bool NARROW_ONLY, bool DEFER>
+template <int N, int M, bool TAU1, bool ST, bool OPT, bool NARROW_ONLY, bool WIDE>
 __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks) roi_bwd_kernel(BwdArgs a, BwdOptArgs o) {
   uint8_t* smem = roi_bwd_smem;
   using C = Cfg<M>;
@@ -501,18 +497,18 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks) roi_bwd_
   src.esize[2] = 2;
   DeferredGroups<C::kDeferCap> dg;
   dg.init(smem + kDeferOffset<N, M, OPT>);
-  const auto exact = [&](int64_t g0) { bwd_exact_group<N, M, TAU1, ST, OPT>(g0, a, o); };
+  const auto exact = [&](int64_t g0) { bwd_exact_group<N, M, ST, OPT>(g0, a, o); };
   // a batch's next tensor may start on the SMs this launch frees (no-op otherwise)
   pdl_launch_dependents();
   const bool ok = run_tiles<C::kThreads, C::kTile, C::kStages, 3>(
       smem, src, a.full_tiles, a.status,
       [&](const uint8_t* const* stage, int64_t tile) {
-        bwd_tile<N, M, TAU1, ST, OPT, NARROW_ONLY, DEFER>(stage, tile, a, o, smem, dg, 0, exact);
+        bwd_tile<N, M, TAU1, ST, OPT, NARROW_ONLY, WIDE>(stage, tile, a, o, smem, dg, 0, exact);
       });
-  if constexpr (DEFER) {
+  if constexpr (C::kDefer) {
     if (ok) dg.drain(true, exact);
   }
-  if (ok && blockIdx.x == gridDim.x - 1) bwd_tail<N, M, TAU1, ST, OPT>(a, o);
+  if (ok && blockIdx.x == gridDim.x - 1) bwd_tail<N, M, TAU1, ST, OPT, WIDE>(a, o);
   // the launch completes only after the batch's previous one (stream order)
   if (blockIdx.x == 0) pdl_wait();
 }
@@ -570,7 +566,7 @@ __device__ __forceinline__ BwdOptArgs multi_opt(const BwdMulti& mm, int i) {
 }
 // roi_bwd_kernel over many small tensors at once, walked as roi_fwd_multi_kernel
 // walks them.
-template <int N, int M, bool TAU1, bool ST, bool OPT, bool NARROW_ONLY, bool DEFER>
+template <int N, int M, bool TAU1, bool ST, bool OPT, bool NARROW_ONLY, bool WIDE>
 __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
     roi_bwd_multi_kernel(const __grid_constant__ BwdMulti mm) {
   uint8_t* smem = roi_bwd_smem;
@@ -596,7 +592,7 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
   dg.init(smem + kDeferOffset<N, M, OPT>);
   const auto exact = [&](int64_t e) {
     const int i = int(e >> 48);
-    bwd_exact_group<N, M, TAU1, ST, OPT>(e & kLow, multi_args<M>(mm, i), multi_opt(mm, i));
+    bwd_exact_group<N, M, ST, OPT>(e & kLow, multi_args<M>(mm, i), multi_opt(mm, i));
   };
   int cur = -1, src_cur = -1;
   int64_t lo = 0, hi = 0, src_lo = 0, src_hi = 0;
@@ -625,15 +621,15 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
           a = multi_args<M>(mm, cur);
           o = multi_opt(mm, cur);
         }
-        bwd_tile<N, M, TAU1, ST, OPT, NARROW_ONLY, DEFER>(stage, t - lo, a, o, smem, dg, int64_t(cur) << 48, exact);
+        bwd_tile<N, M, TAU1, ST, OPT, NARROW_ONLY, WIDE>(stage, t - lo, a, o, smem, dg, int64_t(cur) << 48, exact);
       });
-  if constexpr (DEFER) {
+  if constexpr (C::kDefer) {
     if (ok) dg.drain(true, exact);
   }
   if (ok) {
     for (int i = blockIdx.x; i < mm.count; i += gridDim.x) {
       const BwdArgs ai = multi_args<M>(mm, i);
-      if (ai.full_tiles * C::kTile < ai.E) bwd_tail<N, M, TAU1, ST, OPT>(ai, multi_opt(mm, i));
+      if (ai.full_tiles * C::kTile < ai.E) bwd_tail<N, M, TAU1, ST, OPT, WIDE>(ai, multi_opt(mm, i));
     }
   }
   if (blockIdx.x == 0) pdl_wait();
@@ -679,10 +675,10 @@ struct LaunchCache {
   int per_sm[64] = {0};
 };
 
-template <int N, int M, bool TAU1, bool ST, bool OPT, bool NARROW_ONLY, bool DEFER>
+template <int N, int M, bool TAU1, bool ST, bool OPT, bool NARROW_ONLY, bool WIDE>
 int launch_tiles(const BwdArgs& a, const BwdOptArgs& o, cudaStream_t stream, bool pdl = false) {
   using C = Cfg<M>;
-  auto kern = roi_bwd_kernel<N, M, TAU1, ST, OPT, NARROW_ONLY, DEFER>;
+  auto kern = roi_bwd_kernel<N, M, TAU1, ST, OPT, NARROW_ONLY, WIDE>;
   const size_t smem = kBwdSmem<N, M, OPT>;
   static_assert(kBwdSmem<N, M, OPT> <= 232448, "shared memory per CTA");
   static LaunchCache cache;
@@ -700,22 +696,13 @@ int launch_tiles(const BwdArgs& a, const BwdOptArgs& o, cudaStream_t stream, boo
   return launch_maybe_pdl(kern, grid, C::kThreads, smem, stream, pdl, a, o);
 }
 
-// Groups out of the fast path's range: the exact routine in place, or through the
-// deferred queue (32 at a time) for every 2:4 backward (measured 2.7 % faster at
-// tau = 1 on the 7B-shaped set) and for the others below tau = 0.075 (at tau = 0.05
-// some 4-5 % of the groups leave the range and the queue makes the 7B-shaped 4:8
-// backward 3.5x faster; at tau = 0.5 the 4:8 queue code measured 3 % slower).
-constexpr float kDeferBelowTau = 0.075f;
-
 template <int N, int M, bool ST, bool OPT, bool NARROW_ONLY = false>
 int launch_tau(const BwdArgs& a, const BwdOptArgs& o, cudaStream_t stream, bool pdl) {
-  if (a.tau == 1.0f) return launch_tiles<N, M, true, ST, OPT, NARROW_ONLY, M == 4>(a, o, stream, pdl);
-  if constexpr (M == 4) {
-    return launch_tiles<N, M, false, ST, OPT, NARROW_ONLY, true>(a, o, stream, pdl);
-  } else {
-    return a.tau < kDeferBelowTau ? launch_tiles<N, M, false, ST, OPT, NARROW_ONLY, true>(a, o, stream, pdl)
-                                  : launch_tiles<N, M, false, ST, OPT, NARROW_ONLY, false>(a, o, stream, pdl);
+  if (a.tau == 1.0f) return launch_tiles<N, M, true, ST, OPT, NARROW_ONLY, false>(a, o, stream, pdl);
+  if constexpr (!kAlwaysWide<N>) {
+    if (!wide_range<N>(a.tau, a.np)) return launch_tiles<N, M, false, ST, OPT, NARROW_ONLY, false>(a, o, stream, pdl);
   }
+  return launch_tiles<N, M, false, ST, OPT, NARROW_ONLY, true>(a, o, stream, pdl);
 }
 
 template <int N, int M>
@@ -736,10 +723,10 @@ int launch_nm(const BwdArgs& a, const BwdOptArgs& o, cudaStream_t stream, bool p
   return launch_tau<N, M, false, false>(a, o, stream, pdl);
 }
 
-template <int N, int M, bool TAU1, bool ST, bool OPT, bool NARROW_ONLY, bool DEFER>
+template <int N, int M, bool TAU1, bool ST, bool OPT, bool NARROW_ONLY, bool WIDE>
 int launch_multi_kern(const BwdMulti& mm, cudaStream_t stream, bool pdl) {
   using C = Cfg<M>;
-  auto kern = roi_bwd_multi_kernel<N, M, TAU1, ST, OPT, NARROW_ONLY, DEFER>;
+  auto kern = roi_bwd_multi_kernel<N, M, TAU1, ST, OPT, NARROW_ONLY, WIDE>;
   constexpr size_t smem = kBwdMultiSmem<N, M, OPT>;
   static_assert(smem <= 232448, "shared memory per CTA");
   static LaunchCache cache;
@@ -760,13 +747,12 @@ int launch_multi_kern(const BwdMulti& mm, cudaStream_t stream, bool pdl) {
 
 template <int N, int M, bool ST, bool OPT, bool NARROW_ONLY = false>
 int launch_multi_tau(const BwdMulti& mm, cudaStream_t stream, bool pdl) {
-  if (mm.tau == 1.0f) return launch_multi_kern<N, M, true, ST, OPT, NARROW_ONLY, M == 4>(mm, stream, pdl);
-  if constexpr (M == 4) {
-    return launch_multi_kern<N, M, false, ST, OPT, NARROW_ONLY, true>(mm, stream, pdl);
-  } else {
-    return mm.tau < kDeferBelowTau ? launch_multi_kern<N, M, false, ST, OPT, NARROW_ONLY, true>(mm, stream, pdl)
-                                   : launch_multi_kern<N, M, false, ST, OPT, NARROW_ONLY, false>(mm, stream, pdl);
+  if (mm.tau == 1.0f) return launch_multi_kern<N, M, true, ST, OPT, NARROW_ONLY, false>(mm, stream, pdl);
+  if constexpr (!kAlwaysWide<N>) {
+    if (!wide_range<N>(mm.tau, mm.it[0].np))
+      return launch_multi_kern<N, M, false, ST, OPT, NARROW_ONLY, false>(mm, stream, pdl);
   }
+  return launch_multi_kern<N, M, false, ST, OPT, NARROW_ONLY, true>(mm, stream, pdl);
 }
 
 // The backward variant a call needs, in launch_nm's order: 2 fused AdamW,
@@ -878,10 +864,10 @@ int launch_bwd_batch(const BwdCall* calls, int count) {
       const bool narrow = counters_narrow(c.np, c.E);
       int n = 0;
       while (i + n < count && n < kMultiMaxBwd && calls[i + n].N == c.N && calls[i + n].M == c.M &&
-             bwd_kind(calls[i + n]) == kind && counters_narrow(calls[i + n].np, calls[i + n].E) == narrow &&
+             bwd_kind(calls[i + n]) == kind && same_range(c.N, c.tau, c.np, calls[i + n].np) && counters_narrow(calls[i + n].np, calls[i + n].E) == narrow &&
              multi_small(calls[i + n].E, tile))
         ++n;
-      if (n >= multi_min_run(kind == 0 && c.tau >= kDeferBelowTau)) {
+      if (n >= multi_min_run(kind == 0)) {
         int r = -1;
         if (c.N == 2 && c.M == 4) r = launch_multi<2, 4>(calls + i, n, prev_tiled);
         if (c.N == 4 && c.M == 8) r = launch_multi<4, 8>(calls + i, n, prev_tiled);

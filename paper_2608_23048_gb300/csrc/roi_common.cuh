@@ -27,6 +27,14 @@ constexpr float kLn2 = 0.6931471805599453f;
 // fast path's float range and the group is recomputed by the exact routine.
 constexpr float kTinyExcl = 7.888609052210118e-31f;  // 2^-100
 
+// FastGroup's WIDE relaxation: the largest lead of a group's first member over its second,
+// in log2 units, and the patterns that always take it.  With one correction (N = 2) the
+// second maximum costs what the range checks it replaces did; at N = 4 it is formed three
+// times, and wide_range() in roi_launch.h decides.
+constexpr float kLeadCap = 100.0f;
+template <int N>
+constexpr bool kAlwaysWide = N <= 2;
+
 // The device status record (defined in roi_api.cu, one per device, passed to the
 // kernels by address): word 0 holds the status bits, words 2-3 (a 64-bit value,
 // 8-byte aligned) the wall-time limit in ns of a wait for a stage of a copy ring.
@@ -870,6 +878,29 @@ __device__ __forceinline__ V min_of(const V (&x)[M]) {
   return m;
 }
 
+// The second largest of a group's members (ties count twice): M - 1 of them lie at or
+// below it.  Pairs give (larger, smaller); the second of two merged runs is the largest
+// of min(largest, largest) and the two seconds.
+template <int M, class V>
+__device__ __forceinline__ V second_of(const V (&x)[M]) {
+  static_assert(M == 4 || M == 8, "second of 4 or 8");
+  V h[M / 2], s[M / 2];
+#pragma unroll
+  for (int i = 0; i < M / 2; ++i) {
+    h[i] = vmax(x[2 * i], x[2 * i + 1]);
+    s[i] = vmin(x[2 * i], x[2 * i + 1]);
+  }
+#pragma unroll
+  for (int w = M / 2; w > 1; w >>= 1) {
+#pragma unroll
+    for (int i = 0; i < w / 2; ++i) {
+      s[i] = vmax(vmin(h[2 * i], h[2 * i + 1]), vmax(s[2 * i], s[2 * i + 1]));
+      if (w > 2) h[i] = vmax(h[2 * i], h[2 * i + 1]);
+    }
+  }
+  return s[0];
+}
+
 // Step history mu(k), k = 0 .. N-1, of a relaxation kept for the backward sweep:
 // in registers ...
 template <int N, int M, class V>
@@ -899,8 +930,16 @@ struct SmemSteps {
   }
 };
 
+// WIDE (tau != 1): finite keys never leave the float range, whatever their spread.  The
+// weights are taken relative to the group's second largest offset, and the largest one's
+// lead is capped at 2^100.  With a lead that large the others' complements are 1 to the
+// last bit either way; the leader's own complement is a sum of weights of the others,
+// which contains 2^0 and cannot underflow, and the ratios mu_l / om_leader that the
+// backward forms do not contain the leader's weight.  What the cap took from the lead
+// (excess) re-enters the leader's next offset, where log2 of its complement is short by
+// that much.  Only non-finite keys are flagged then.
 template <int N, int M, bool TAU1, bool KEEP, class V = float,
-          class Steps = RegSteps<KEEP ? N : 1, KEEP ? M : 1, V>>
+          class Steps = RegSteps<KEEP ? N : 1, KEEP ? M : 1, V>, bool WIDE = kAlwaysWide<N>>
 struct FastGroup {
   // KEEP: store mu of every step for a backward sweep.  S is then not
   // accumulated: soft() re-sums it from the history on demand (in the order
@@ -974,6 +1013,55 @@ struct FastGroup {
 #pragma unroll
             for (int l = 0; l < M; ++l) cur[l] = vmul(v[l], rt);
           }
+        }
+      }
+    } else if constexpr (WIDE) {
+      const V itau = vconst<V>(inv_tau);
+      // flagged: a non-finite key, or one beyond 2^63, whose offsets could overflow below
+      V sq = vmul(kap[0], kap[0]);
+#pragma unroll
+      for (int l = 1; l < M; ++l) sq = vfma(kap[l], kap[l], sq);
+      flag = vbelow(vsub(sq, sq), 0.0f);
+      V x[M];
+      {
+        const V ref = N > 1 ? second_of(kap) : max_of(kap);
+#pragma unroll
+        for (int l = 0; l < M; ++l) x[l] = vmul(vsub(kap[l], ref), itau);
+      }
+#pragma unroll
+      for (int k = 0; k < N; ++k) {
+        const bool last = k + 1 == N;
+        if (k > 0) {
+          const V ref = last ? max_of(x) : second_of(x);
+#pragma unroll
+          for (int l = 0; l < M; ++l) x[l] = vsub(x[l], ref);
+        }
+        V c[M], e[M];
+#pragma unroll
+        for (int l = 0; l < M; ++l) {
+          c[l] = last ? x[l] : vmin(x[l], vconst<V>(kLeadCap));
+          e[l] = vmap(c[l], ex2_approx);
+        }
+        const V r = vmap(sum_of(e), rcp_approx);
+        if (!KEEP && k > 0 && last) {
+          // last step without KEEP: added into S as it is formed (one fma)
+#pragma unroll
+          for (int l = 0; l < M; ++l) S[l] = vfma(e[l], r, S[l]);
+        } else {
+#pragma unroll
+          for (int l = 0; l < M; ++l) {
+            cur[l] = vmul(e[l], r);
+            if constexpr (KEEP) st.put(k, l, cur[l]);
+            if constexpr (kSumS) S[l] = k == 0 ? cur[l] : vadd(S[l], cur[l]);
+          }
+        }
+        if (!last) {
+          // offset + (log2(1 - mu) - excess) / tau
+          V ex[M];
+          exclusive_sums(e, ex);
+#pragma unroll
+          for (int l = 0; l < M; ++l)
+            x[l] = vfma(vsub(vmap(vmul(ex[l], r), lg2_approx), vsub(x[l], c[l])), itau, x[l]);
         }
       }
     } else {

@@ -24,12 +24,8 @@ struct Cfg {
   static constexpr int kStages = 2;  // 144 KB (M = 4) or 96 KB (M = 8)
   static constexpr int kMinBlocks = 1;
   static constexpr int kTile = 2 * kPairs * kThreads * M;  // elements
-  // groups out of the fast path's range, queued per warp (DeferredGroups): at most
-  // 64 kPairs a tile on top of fewer than 32 left from earlier tiles
-  static constexpr int kDeferCap = 32 + 64 * kPairs;
-  static constexpr size_t kDeferOffset = (tile_smem_bytes<kTile, kStages>(6) + 15) & ~size_t(15);
-  static constexpr size_t kSmem = kDeferOffset + size_t(kDeferCap) * 8 * (kThreads / 32);
-  // multi-tensor launches: the tensors' first tiles behind the queues
+  static constexpr size_t kSmem = tile_smem_bytes<kTile, kStages>(6);
+  // multi-tensor launches: the tensors' first tiles behind the ring
   static constexpr size_t kMultiOffset = (kSmem + 15) & ~size_t(15);
   static constexpr size_t kMultiSmem = kMultiOffset + size_t(kMultiMax + 1) * 8;
 };
@@ -130,11 +126,11 @@ __device__ __forceinline__ void fwd_keys(const float* const* phi_g, const int64_
 }
 
 // Relaxation, hard bits and outputs of L groups whose keys are `kap`.
-template <int N, int M, bool TAU1, class V, bool ST = false, bool DEFER = false>
-__device__ __forceinline__ uint32_t fwd_finish(const V (&kap)[M], const uint16_t* const* W_g, const int64_t* e0,
+template <int N, int M, bool TAU1, class V, bool ST, bool WIDE>
+__device__ __forceinline__ void fwd_finish(const V (&kap)[M], const uint16_t* const* W_g, const int64_t* e0,
                                                const FwdArgs& a, uint32_t* bits) {
   constexpr int L = vlanes<V>();
-  FastGroup<N, M, TAU1, false, V> fg;
+  FastGroup<N, M, TAU1, false, V, RegSteps<1, 1, V>, WIDE> fg;
   fg.forward(kap, a.inv_tau);
   float S[L][M];
 #pragma unroll
@@ -176,52 +172,34 @@ __device__ __forceinline__ uint32_t fwd_finish(const V (&kap)[M], const uint16_t
       }
     }
   }
-  // groups out of the fast path's range: ranked by comparison, and either relaxed
-  // here by the exact routine (DEFER off) or (DEFER) left to fwd_exact_group, which
-  // the caller runs for them from the deferred queue and which writes their soft
-  // mask and Wm again
-  if constexpr (!DEFER) {
-    if (fg.flag != 0u) {
-#pragma unroll
-      for (int h = 0; h < L; ++h) {
-        if ((fg.flag >> h) & 1u) {
-          float k[M], kn[M];
-#pragma unroll
-          for (int l = 0; l < M; ++l) {
-            k[l] = lane_of(kap[l], h);
-            kn[l] = k[l] * kLn2;  // natural-log keys
-          }
-          if constexpr (kFastTopn) {
-            if constexpr (M == 4) {
-              bits[h] = topn_bits4(k, N);
-            } else {
-              bits[h] = topn_bits<M>(k, N);
-            }
-          }
-          // finite keys spread beyond the fast path's float range (tau != 1: at tau = 1
-          // that takes a key gap of ~69 natural-log units, and the tau = 1 kernels keep
-          // their code to the exact routine)
-          if (!TAU1 && all_finite(k)) {
-            RobustGroup<N, M> rg;
-            rg.forward(k, a.inv_tau, S[h]);
-          } else {
-            ExactGroup<N, M> ex;
-            ex.forward(kn, N, M, a.tau, S[h]);
-          }
-        }
-      }
-    }
-  } else if (kFastTopn && fg.flag != 0u) {
+  // groups out of the fast path's range: ranked by comparison and relaxed by an exact
+  // routine
+  if (fg.flag != 0u) {
 #pragma unroll
     for (int h = 0; h < L; ++h) {
       if ((fg.flag >> h) & 1u) {
-        float k[M];
+        float k[M], kn[M];
 #pragma unroll
-        for (int l = 0; l < M; ++l) k[l] = lane_of(kap[l], h);
-        if constexpr (M == 4) {
-          bits[h] = topn_bits4(k, N);
+        for (int l = 0; l < M; ++l) {
+          k[l] = lane_of(kap[l], h);
+          kn[l] = k[l] * kLn2;  // natural-log keys
+        }
+        if constexpr (kFastTopn) {
+          if constexpr (M == 4) {
+            bits[h] = topn_bits4(k, N);
+          } else {
+            bits[h] = topn_bits<M>(k, N);
+          }
+        }
+        // finite keys spread beyond the plain relaxation's float range (at tau = 1 that
+        // takes a key gap of ~69 natural-log units, and the tau = 1 kernels keep their
+        // code to the exact routine)
+        if (!TAU1 && !WIDE && all_finite(k)) {
+          RobustGroup<N, M> rg;
+          rg.forward(k, a.inv_tau, S[h]);
         } else {
-          bits[h] = topn_bits<M>(k, N);
+          ExactGroup<N, M> ex;
+          ex.forward(kn, N, M, a.tau, S[h]);
         }
       }
     }
@@ -265,58 +243,15 @@ __device__ __forceinline__ uint32_t fwd_finish(const V (&kap)[M], const uint16_t
       }
     }
   }
-  return DEFER ? fg.flag : 0u;
-}
-
-// The exact routine for one group out of the fast path's range (first element g0,
-// call-flat), from global memory: the log2-domain routine for finite keys spread
-// beyond the float range (tau != 1; at tau = 1 that takes a key gap of ~69
-// natural-log units and the tau = 1 kernels keep only the general routine), the
-// exact one otherwise.  Writes soft and (unless straight-through) Wm.
-template <int N, int M, bool TAU1, bool ST>
-__device__ __forceinline__ void fwd_exact_group(int64_t g0, const FwdArgs& a) {
-  if (ST && a.soft == nullptr) return;
-  // the keys as the tiles' packed code forms them (the group in both halves), so they
-  // equal, bit for bit, those the fast path and the masked linear's prologue see
-  const float* pp[2] = {a.phi + g0, a.phi + g0};
-  const int64_t e0[2] = {g0, g0};
-  F2 k2[M];
-  fwd_keys<M, F2>(pp, e0, nullptr, a, k2);
-  float k[M], S[M];
-#pragma unroll
-  for (int l = 0; l < M; ++l) k[l] = lo(k2[l]);
-  if (!TAU1 && all_finite(k)) {
-    RobustGroup<N, M> rg;
-    rg.forward(k, a.inv_tau, S);
-  } else {
-#pragma unroll
-    for (int l = 0; l < M; ++l) k[l] *= kLn2;  // natural-log keys
-    ExactGroup<N, M> ex;
-    ex.forward(k, N, M, a.tau, S);
-  }
-#pragma unroll
-  for (int s = 0; s < M / 4; ++s) {
-    if constexpr (!ST) {
-      const uint2 q = reinterpret_cast<const uint2*>(a.W + g0)[s];
-      uint2 o;
-      o.x = pack_bf16x2(__fmul_rn(bf16_bits_to_float(q.x & 0xffffu), S[4 * s]),
-                        __fmul_rn(bf16_bits_to_float(q.x >> 16), S[4 * s + 1]));
-      o.y = pack_bf16x2(__fmul_rn(bf16_bits_to_float(q.y & 0xffffu), S[4 * s + 2]),
-                        __fmul_rn(bf16_bits_to_float(q.y >> 16), S[4 * s + 3]));
-      reinterpret_cast<uint2*>(a.Wm + g0)[s] = o;
-    }
-    if (a.soft != nullptr)
-      reinterpret_cast<float4*>(a.soft + g0)[s] = make_float4(S[4 * s], S[4 * s + 1], S[4 * s + 2], S[4 * s + 3]);
-  }
 }
 
 // One group straight from global memory (the ragged tail; the exact routine in place).
-template <int N, int M, bool TAU1, bool ST = false>
+template <int N, int M, bool TAU1, bool ST, bool WIDE>
 __device__ __forceinline__ void fwd_groups(const float* const* phi_g, const uint16_t* const* W_g, const int64_t* e0,
                                            const FwdArgs& a, uint32_t* bits) {
   float kap[M];
   fwd_keys<M, float>(phi_g, e0, nullptr, a, kap);
-  fwd_finish<N, M, TAU1, float, ST>(kap, W_g, e0, a, bits);
+  fwd_finish<N, M, TAU1, float, ST, WIDE>(kap, W_g, e0, a, bits);
 }
 
 // Combine the M-bit masks of 32 / M consecutive lanes into words and store.
@@ -355,9 +290,8 @@ __device__ __forceinline__ void store_hard_pair(uint32_t* hard, int64_t e0a, int
 
 // One full tile of a tensor (local tile index `tile`), inputs staged in shared
 // memory.  NARROW: the call's counters are below 2^32 (a.np.narrow).
-template <int N, int M, bool TAU1, bool ST, bool NARROW, bool DEFER, class Defer, class Exact>
-__device__ __forceinline__ void fwd_tile(const uint8_t* const* stage, int64_t tile, const FwdArgs& a, Defer& dg,
-                                         int64_t tag, const Exact& exact) {
+template <int N, int M, bool TAU1, bool ST, bool NARROW, bool WIDE>
+__device__ __forceinline__ void fwd_tile(const uint8_t* const* stage, int64_t tile, const FwdArgs& a) {
   using C = Cfg<M>;
   constexpr int kT = C::kTile;
   const float* sphi = reinterpret_cast<const float*>(stage[0]);
@@ -390,19 +324,14 @@ __device__ __forceinline__ void fwd_tile(const uint8_t* const* stage, int64_t ti
     const uint16_t* pw[2] = {sW + g0 * M, sW + g1 * M};
     const int64_t e0[2] = {base + g0 * M, base + g1 * M};
     uint32_t bits[2];
-    const uint32_t flag = fwd_finish<N, M, TAU1, F2, ST, DEFER>(kap[p & 1], pw, e0, a, bits);
+    fwd_finish<N, M, TAU1, F2, ST, WIDE>(kap[p & 1], pw, e0, a, bits);
     if (a.hard != nullptr) store_hard_pair<M>(a.hard, e0[0], e0[1], bits[0], bits[1]);
-    if constexpr (DEFER) {
-      dg.push((flag & 1u) != 0u, tag | e0[0]);
-      dg.push((flag & 2u) != 0u, tag | e0[1]);
-    }
   }
-  if constexpr (DEFER) dg.drain(false, exact);
 }
 
 // The ragged tail of a tensor (fewer than one tile after its full tiles), by one
 // CTA, straight from global memory.
-template <int N, int M, bool TAU1, bool ST>
+template <int N, int M, bool TAU1, bool ST, bool WIDE>
 __device__ __forceinline__ void fwd_tail(const FwdArgs& a) {
   using C = Cfg<M>;
   const int64_t t0 = a.full_tiles * C::kTile;
@@ -416,14 +345,14 @@ __device__ __forceinline__ void fwd_tail(const FwdArgs& a) {
       const float* pp[1] = {a.phi + t0 + gi * M};
       const uint16_t* pw[1] = {a.W + t0 + gi * M};
       const int64_t e0[1] = {t0 + gi * M};
-      fwd_groups<N, M, TAU1, ST>(pp, pw, e0, a, &bits);
+      fwd_groups<N, M, TAU1, ST, WIDE>(pp, pw, e0, a, &bits);
     }
     if (a.hard != nullptr) store_hard<M>(a.hard, t0 + gi * M, bits, active);
   }
 }
 
 // ST: straight-through Wm (a separate instantiation)
-template <int N, int M, bool TAU1, bool ST, bool DEFER>
+template <int N, int M, bool TAU1, bool ST, bool WIDE>
 __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks) roi_fwd_kernel(FwdArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   using C = Cfg<M>;
@@ -432,9 +361,6 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks) roi_fwd_
   src.esize[0] = 4;
   src.ptr[1] = reinterpret_cast<const uint8_t*>(a.W);
   src.esize[1] = 2;
-  DeferredGroups<C::kDeferCap> dg;
-  dg.init(smem + C::kDeferOffset);
-  const auto exact = [&](int64_t g0) { fwd_exact_group<N, M, TAU1, ST>(g0, a); };
   // a batch's next tensor may start on the SMs this launch frees (no-op otherwise)
   pdl_launch_dependents();
   const bool ok = run_tiles<C::kThreads, C::kTile, C::kStages, 2>(
@@ -444,16 +370,13 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks) roi_fwd_
         // body measured slower (register allocation), so those keep one
         if constexpr (M == 4) {
           if (a.np.narrow) {
-            fwd_tile<N, M, TAU1, ST, true, DEFER>(stage, tile, a, dg, 0, exact);
+            fwd_tile<N, M, TAU1, ST, true, WIDE>(stage, tile, a);
             return;
           }
         }
-        fwd_tile<N, M, TAU1, ST, false, DEFER>(stage, tile, a, dg, 0, exact);
+        fwd_tile<N, M, TAU1, ST, false, WIDE>(stage, tile, a);
       });
-  if constexpr (DEFER) {
-    if (ok) dg.drain(true, exact);
-  }
-  if (ok && blockIdx.x == gridDim.x - 1) fwd_tail<N, M, TAU1, ST>(a);
+  if (ok && blockIdx.x == gridDim.x - 1) fwd_tail<N, M, TAU1, ST, WIDE>(a);
   // the launch completes only after the batch's previous one (stream order)
   if (blockIdx.x == 0) pdl_wait();
 }
@@ -500,15 +423,13 @@ __device__ __forceinline__ FwdArgs multi_args(const FwdMulti& mm, int i) {
 // The tile kernel over many small tensors at once: the persistent CTAs walk the
 // concatenation of the tensors' full tiles, finding a tile's tensor by binary
 // search over tile0 (in shared memory) only when a tile leaves the current one.
-// Deferred groups carry their tensor's index above bit 48; each tensor's ragged
-// tail goes to one CTA after the tiles.
-template <int N, int M, bool TAU1, bool ST, bool DEFER>
+// Each tensor's ragged tail goes to one CTA after the tiles.
+template <int N, int M, bool TAU1, bool ST, bool WIDE>
 __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
     roi_fwd_multi_kernel(const __grid_constant__ FwdMulti mm) {
   extern __shared__ __align__(128) uint8_t smem[];
   using C = Cfg<M>;
   const uint32_t esize[2] = {4, 2};
-  constexpr int64_t kLow = (int64_t(1) << 48) - 1;
   // the tensors' first tiles, in shared memory for the searches
   int64_t* tile0 = reinterpret_cast<int64_t*>(smem + C::kMultiOffset);
   for (int i = threadIdx.x; i <= mm.count; i += C::kThreads) tile0[i] = i < mm.count ? mm.it[i].tile0 : mm.total_tiles;
@@ -525,9 +446,6 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
     }
     return lo;
   };
-  DeferredGroups<C::kDeferCap> dg;
-  dg.init(smem + C::kDeferOffset);
-  const auto exact = [&](int64_t e) { fwd_exact_group<N, M, TAU1, ST>(e & kLow, multi_args<M>(mm, int(e >> 48))); };
   // the current tensor of this warp's tiles (and of the copies thread 0 issues),
   // looked up again only when a tile falls outside it
   int cur = -1, src_cur = -1;
@@ -557,22 +475,18 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
           a = multi_args<M>(mm, cur);
         }
         const int64_t local = t - lo;
-        const int64_t tag = int64_t(cur) << 48;
         if constexpr (M == 4) {
           if (a.np.narrow) {
-            fwd_tile<N, M, TAU1, ST, true, DEFER>(stage, local, a, dg, tag, exact);
+            fwd_tile<N, M, TAU1, ST, true, WIDE>(stage, local, a);
             return;
           }
         }
-        fwd_tile<N, M, TAU1, ST, false, DEFER>(stage, local, a, dg, tag, exact);
+        fwd_tile<N, M, TAU1, ST, false, WIDE>(stage, local, a);
       });
-  if constexpr (DEFER) {
-    if (ok) dg.drain(true, exact);
-  }
   if (ok) {
     for (int i = blockIdx.x; i < mm.count; i += gridDim.x) {
       const FwdArgs ai = multi_args<M>(mm, i);
-      if (ai.full_tiles * C::kTile < ai.E) fwd_tail<N, M, TAU1, ST>(ai);
+      if (ai.full_tiles * C::kTile < ai.E) fwd_tail<N, M, TAU1, ST, WIDE>(ai);
     }
   }
   if (blockIdx.x == 0) pdl_wait();
@@ -613,10 +527,10 @@ struct LaunchCache {
   int per_sm[64] = {0};
 };
 
-template <int N, int M, bool TAU1, bool ST, bool DEFER>
+template <int N, int M, bool TAU1, bool ST, bool WIDE>
 int launch_tiles(const FwdArgs& a, cudaStream_t stream, bool pdl) {
   using C = Cfg<M>;
-  auto kern = roi_fwd_kernel<N, M, TAU1, ST, DEFER>;
+  auto kern = roi_fwd_kernel<N, M, TAU1, ST, WIDE>;
   const size_t smem = C::kSmem;
   static_assert(C::kSmem <= 232448, "shared memory per CTA");
   static LaunchCache cache;  // per instantiation and device; racing writers store the same value
@@ -634,18 +548,13 @@ int launch_tiles(const FwdArgs& a, cudaStream_t stream, bool pdl) {
   return launch_maybe_pdl(kern, grid, C::kThreads, smem, stream, pdl, a);
 }
 
-// Groups out of the fast path's range go to the exact routine in place (one thread,
-// the rest of its warp waiting) or, below tau = 0.075, through the deferred queue
-// (32 at a time).  At tau = 0.05 (the end of the paper's schedule) some 4-5 % of
-// the groups leave the range and the queue makes the 7B-shaped 4:8 forward 2.1x
-// faster; at tau >= 0.1 (under 0.2 % of them) the queue's code measured 2-9 % slower.
-constexpr float kDeferBelowTau = 0.075f;
-
 template <int N, int M, bool ST>
 int launch_st(const FwdArgs& a, cudaStream_t stream, bool pdl) {
   if (a.tau == 1.0f) return launch_tiles<N, M, true, ST, false>(a, stream, pdl);
-  return a.tau < kDeferBelowTau ? launch_tiles<N, M, false, ST, true>(a, stream, pdl)
-                                : launch_tiles<N, M, false, ST, false>(a, stream, pdl);
+  if constexpr (!kAlwaysWide<N>) {
+    if (!wide_range<N>(a.tau, a.np)) return launch_tiles<N, M, false, ST, false>(a, stream, pdl);
+  }
+  return launch_tiles<N, M, false, ST, true>(a, stream, pdl);
 }
 
 template <int N, int M>
@@ -653,10 +562,10 @@ int launch_nm(const FwdArgs& a, cudaStream_t stream, bool pdl = false) {
   return a.st ? launch_st<N, M, true>(a, stream, pdl) : launch_st<N, M, false>(a, stream, pdl);
 }
 
-template <int N, int M, bool TAU1, bool ST, bool DEFER>
+template <int N, int M, bool TAU1, bool ST, bool WIDE>
 int launch_multi_kern(const FwdMulti& mm, cudaStream_t stream, bool pdl) {
   using C = Cfg<M>;
-  auto kern = roi_fwd_multi_kernel<N, M, TAU1, ST, DEFER>;
+  auto kern = roi_fwd_multi_kernel<N, M, TAU1, ST, WIDE>;
   static LaunchCache cache;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
@@ -675,10 +584,12 @@ int launch_multi_kern(const FwdMulti& mm, cudaStream_t stream, bool pdl) {
 }
 
 template <int N, int M, bool ST>
-int launch_multi_st(const FwdMulti& mm, cudaStream_t stream, bool pdl) {
+int launch_multi_st(const FwdMulti& mm, bool wide, cudaStream_t stream, bool pdl) {
   if (mm.tau == 1.0f) return launch_multi_kern<N, M, true, ST, false>(mm, stream, pdl);
-  return mm.tau < kDeferBelowTau ? launch_multi_kern<N, M, false, ST, true>(mm, stream, pdl)
-                                 : launch_multi_kern<N, M, false, ST, false>(mm, stream, pdl);
+  if constexpr (!kAlwaysWide<N>) {
+    if (!wide) return launch_multi_kern<N, M, false, ST, false>(mm, stream, pdl);
+  }
+  return launch_multi_kern<N, M, false, ST, true>(mm, stream, pdl);
 }
 
 // One launch over calls[0 .. count), with launch_st's choice of variant.
@@ -708,7 +619,9 @@ int launch_multi(const FwdCall* calls, int count, bool pdl) {
   }
   mm.total_tiles = tiles;
   const cudaStream_t stream = calls[0].stream;
-  return mm.st ? launch_multi_st<N, M, true>(mm, stream, pdl) : launch_multi_st<N, M, false>(mm, stream, pdl);
+  const bool wide = wide_range<N>(mm.tau, mm.it[0].np);
+  return mm.st ? launch_multi_st<N, M, true>(mm, wide, stream, pdl)
+               : launch_multi_st<N, M, false>(mm, wide, stream, pdl);
 }
 
 }  // namespace
@@ -767,7 +680,7 @@ int launch_fwd_batch(const FwdCall* calls, int count) {
       const int64_t tile = c.M == 8 ? Cfg<8>::kTile : Cfg<4>::kTile;
       int n = 0;
       while (i + n < count && n < kMultiMax && calls[i + n].N == c.N && calls[i + n].M == c.M &&
-             multi_small(calls[i + n].E, tile))
+             same_range(c.N, c.tau, c.np, calls[i + n].np) && multi_small(calls[i + n].E, tile))
         ++n;
       if (n >= multi_min_run(false)) {
         int r = -1;

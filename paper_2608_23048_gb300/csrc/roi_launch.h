@@ -15,6 +15,26 @@ inline bool counters_narrow(const NoiseParams& np, int64_t E) {
   return np.e_base <= lim && uint64_t(E) <= lim - np.e_base;
 }
 
+// The relaxation of a tau != 1 tile kernel (FastGroup, M = 4, 8).  WIDE always where it
+// costs nothing (kAlwaysWide; 0.5B-shaped 2:4 step at tau = 0.1 1848 -> 1813 us).  4:8 at
+// tau = 0.5 pays 2.7 % for it (one 1.5B-shaped block, forward and backward, 335 -> 344 us)
+// and takes the plain one unless groups are likely to leave that one's range, which are
+// then relaxed by a slow routine.  The range is ~69 tau in natural-log units of the keys:
+// the Gumbel noise alone exceeds it below tau = 0.2 (same block, plain / WIDE: 347 / 343 us
+// at tau = 0.2, 519 / 344 at 0.1, 1338 / 344 at 0.06), logits of unit spread do where
+// 69 tau is a few times 1 / lambda (986 / 349 us at tau = 0.22, lambda = 0.045, while
+// tau lambda = 0.1 still measured 336 plain).
+constexpr float kWideTau = 0.2f;
+constexpr float kWideTauLambda = 0.09f;
+template <int N>
+inline bool wide_range(float tau, const NoiseParams& np) {
+  return kAlwaysWide<N> || tau <= kWideTau || tau < kWideTauLambda * np.inv_lam;
+}
+// Whether two calls of a batch take the same relaxation (lambda is each item's own).
+inline bool same_range(int N, float tau, const NoiseParams& a, const NoiseParams& b) {
+  return N != 4 || tau == 1.0f || wide_range<4>(tau, a) == wide_range<4>(tau, b);
+}
+
 struct FwdCall {
   const float* phi;
   const uint16_t* W;
@@ -143,10 +163,7 @@ int sm_count();
 // gains from runs of 2 (the q, k, v, o tensors of a 7B-shaped layer), while the
 // forward and the backward fused with AdamW lost on those runs (7B-shaped 2:4 step,
 // forward 11.72 -> 11.80 ms, fused backward 28.8 -> 29.0 ms) and gain only over long
-// ones.  So does the plain backward where many groups go through the deferred
-// queue (tau below the deferral threshold): each drained group reads its tensor's
-// arguments from the parameter block by a per-lane index (tau = 0.05, 1.5B-shaped
-// 4:8 backward 7.01 -> 7.24 ms with short runs shared).  A fwd + bwd step over a
+// ones.  A fwd + bwd step over a
 // Qwen2.5-shaped layer set went from 1.90 to 1.57 ms (0.5B-shaped, 2:4: one launch
 // per direction), 8.92 to 8.78 ms (1.5B-shaped, 4:8) and 24.31 to 24.19 ms
 // (7B-shaped, 2:4).

@@ -119,7 +119,7 @@ __device__ __forceinline__ void issue_chunk(const CUtensorMap* tm_phi, const CUt
 
 // Relax this thread's pair of chunk kc from the staged logits and write
 // bf16(W * S) into the chunk's A tile (core-matrix layout).
-template <int N, int M, bool TAU1>
+template <int N, int M, bool TAU1, bool WIDE>
 __device__ __forceinline__ void chunk_masked_weights(const LinArgs& a, uint8_t* smem, const LinSmem& L, int stage,
                                                      int64_t row0, int kc) {
   int r, gk;
@@ -174,7 +174,7 @@ __device__ __forceinline__ void chunk_masked_weights(const LinArgs& a, uint8_t* 
       kap[l] = key_log2(f2(ph[0][l], ph[1][l]), u, a.np.l2e_inv_lam);
     }
   }
-  FastGroup<N, M, TAU1, false, F2> fg;
+  FastGroup<N, M, TAU1, false, F2, RegSteps<1, 1, F2>, WIDE> fg;
   fg.forward(kap, a.inv_tau);
   float S[2][M];
 #pragma unroll
@@ -192,7 +192,7 @@ __device__ __forceinline__ void chunk_masked_weights(const LinArgs& a, uint8_t* 
           k[l] = lane_of(kap[l], h);
           kn[l] = k[l] * kLn2;  // natural-log keys
         }
-        if (!TAU1 && all_finite(k)) {
+        if (!TAU1 && !WIDE && all_finite(k)) {
           RobustGroup<N, M> rg;
           rg.forward(k, a.inv_tau, S[h]);
         } else {
@@ -224,7 +224,7 @@ __device__ __forceinline__ void chunk_masked_weights(const LinArgs& a, uint8_t* 
   }
 }
 
-template <int N, int M, bool TAU1>
+template <int N, int M, bool TAU1, bool WIDE>
 __global__ void __launch_bounds__(LinCfg<M>::kThreads + 32, 1)
     roi_masked_linear_kernel(const __grid_constant__ CUtensorMap tm_phi, const __grid_constant__ CUtensorMap tm_w,
                              const __grid_constant__ CUtensorMap tm_x, LinArgs a) {
@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(LinCfg<M>::kThreads + 32, 1)
     for (int c = 0; c < nc; ++c) {
       if (ok) ok = mbar_wait_ring(full + s, phase, lim);
       if (!ok) break;
-      chunk_masked_weights<N, M, TAU1>(a, smem, L, s, row0, c_begin + c);
+      chunk_masked_weights<N, M, TAU1, WIDE>(a, smem, L, s, row0, c_begin + c);
       fence_proxy_async_smem();
       mbar_arrive(ready + s);
       if (s == kStages - 1) {
@@ -446,12 +446,20 @@ int launch_nm(const LinearCall& c, const LinArgs& a) {
     return -1;
   const LinSmem L = lin_smem(a.T_pad);
   const size_t smem = size_t(L.total) + 1024;  // + alignment slack
-  auto kern = a.tau == 1.0f ? roi_masked_linear_kernel<N, M, true> : roi_masked_linear_kernel<N, M, false>;
+  // the mask forward's choice of relaxation, so Wm is its bit for bit
+  int variant = a.tau == 1.0f ? 0 : 1;
+  auto kern = a.tau == 1.0f ? roi_masked_linear_kernel<N, M, true, false> : roi_masked_linear_kernel<N, M, false, true>;
+  if constexpr (!kAlwaysWide<N>) {
+    if (variant == 1 && !wide_range<N>(a.tau, a.np)) {
+      variant = 2;
+      kern = roi_masked_linear_kernel<N, M, false, false>;
+    }
+  }
   // the shared-memory limit is set once per device and kernel, to the largest size
-  static int set_to[2][64] = {{0}};
+  static int set_to[3][64] = {{0}};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
-  int& cur = set_to[a.tau == 1.0f ? 1 : 0][dev];
+  int& cur = set_to[variant][dev];
   if (cur < int(smem)) {
     const int want = int(lin_smem(256).total) + 1024;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, want) != cudaSuccess) return -1;

@@ -89,8 +89,6 @@ def assert_same(a, b):
 SHAPES = [(37, 1000), (3, 64), (64, 3584), (512, 256), (1, 32), (129, 2048), (8, 8), (300, 520), (16, 24576)]
 
 
-# tau = 0.05: many groups leave the fast path's range and go through the deferred
-# queues, whose entries name their tensor in a launch shared by several
 @pytest.mark.parametrize("N,M,tau", [(2, 4, 1.0), (2, 4, 0.5), (2, 4, 0.05), (4, 8, 1.0), (4, 8, 0.3), (4, 8, 0.05),
                                      (2, 8, 1.0), (3, 4, 0.8), (8, 16, 0.2), (16, 32, 1.0)])
 def test_batch_equals_single_calls(roi, N, M, tau):
@@ -100,6 +98,17 @@ def test_batch_equals_single_calls(roi, N, M, tau):
     single = run_single(roi, ts, N, M, tau, flags)
     batch = run_batch(roi, ts, N, M, tau, flags)
     for a, b in zip(single, batch):
+        assert_same(a, b)
+
+
+def test_batch_mixes_relaxations(roi):
+    """lambda is each item's own, and at 4:8 it decides which relaxation an item takes: a
+    run of small tensors on both sides of the rule is split there."""
+    ts = make_set([(37, 1000), (3, 64), (64, 512), (512, 256)] * 6, 61)
+    for k, t in enumerate(ts):
+        t["st"] = t["st"][:3] + ((0.29 if k // 9 == 1 else 0.31), 0)  # tau lambda = 0.087 / 0.093
+    flags = [(True, True, k % 2 == 0) for k in range(len(ts))]
+    for a, b in zip(run_single(roi, ts, 4, 8, 0.3, flags), run_batch(roi, ts, 4, 8, 0.3, flags)):
         assert_same(a, b)
 
 

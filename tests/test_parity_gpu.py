@@ -298,6 +298,20 @@ def test_every_group_out_of_range(roi, N, M):
     check_against_oracle(got, phi.numpy(), WL.bf16_bits(W), WL.bf16_bits(dWm), N, M, 0.05, 9, 4, 3, 1.0, 0)
 
 
+# The spread of the keys over the range of the plain tau != 1 relaxation grows as
+# 1 / (tau lambda): the temperatures of the annealing schedule, on both sides of the rule
+# that picks the relaxation for 4:8 (tau = 0.2, tau lambda = 0.09), and tau > 1.  24600 or
+# 24576 + a ragged tail of elements: full tiles of every tile kernel and a remainder.
+@pytest.mark.parametrize("N,M", [(2, 4), (4, 8), (2, 8)])
+@pytest.mark.parametrize("tau,lam", [(0.2236, 0.0447), (0.05, 0.002), (0.21, 0.43), (0.21, 0.42), (0.2, 1.0),
+                                     (0.201, 1.0), (1.5, 0.01)])
+def test_schedule_temperatures(roi, N, M, tau, lam):
+    W, phi, dWm, ph, Wb, dWb = make(41, 600, "normal", data_seed=M + N)
+    st = roi.NoiseState(123456789, 5, 2, lam, 0)
+    got = gpu_run(roi, phi, W, dWm, N, M, tau, st)
+    check_against_oracle(got, ph, Wb, dWb, N, M, tau, 123456789, 5, 2, lam, 0)
+
+
 @pytest.mark.parametrize("rows,cols", [(4, 64), (8, 2112)])
 def test_non_finite_logits_propagate(roi, rows, cols):
     """NaN / +inf logits make their group's outputs NaN (for N = 1 a +inf member
