@@ -502,8 +502,9 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks) roi_bwd_
   pdl_launch_dependents();
   const bool ok = run_tiles<C::kThreads, C::kTile, C::kStages, 3>(
       smem, src, a.full_tiles, a.status,
-      [&](const uint8_t* const* stage, int64_t tile) {
+      [&](const uint8_t* const* stage, int64_t tile, const auto& release) {
         bwd_tile<N, M, TAU1, ST, OPT, NARROW_ONLY, WIDE>(stage, tile, a, o, smem, dg, 0, exact);
+        release();
       });
   if constexpr (C::kDefer) {
     if (ok) dg.drain(true, exact);
@@ -613,7 +614,7 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
         }
         return src_ptr[arr] + size_t(t - src_lo) * C::kTile * esize[arr];
       },
-      [&](const uint8_t* const* stage, int64_t t) {
+      [&](const uint8_t* const* stage, int64_t t, const auto& release) {
         if (t < lo || t >= hi) {
           cur = find(t);
           lo = tile0[cur];
@@ -622,6 +623,7 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
           o = multi_opt(mm, cur);
         }
         bwd_tile<N, M, TAU1, ST, OPT, NARROW_ONLY, WIDE>(stage, t - lo, a, o, smem, dg, int64_t(cur) << 48, exact);
+        release();
       });
   if constexpr (C::kDefer) {
     if (ok) dg.drain(true, exact);

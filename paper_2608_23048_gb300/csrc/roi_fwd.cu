@@ -365,16 +365,18 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks) roi_fwd_
   pdl_launch_dependents();
   const bool ok = run_tiles<C::kThreads, C::kTile, C::kStages, 2>(
       smem, src, a.full_tiles, a.status,
-      [&](const uint8_t* const* stage, int64_t tile) {
+      [&](const uint8_t* const* stage, int64_t tile, const auto& release) {
         // 32-bit counters for M = 4 only: at M = 8 the second copy of the tile
         // body measured slower (register allocation), so those keep one
         if constexpr (M == 4) {
           if (a.np.narrow) {
             fwd_tile<N, M, TAU1, ST, true, WIDE>(stage, tile, a);
+            release();
             return;
           }
         }
         fwd_tile<N, M, TAU1, ST, false, WIDE>(stage, tile, a);
+        release();
       });
   if (ok && blockIdx.x == gridDim.x - 1) fwd_tail<N, M, TAU1, ST, WIDE>(a);
   // the launch completes only after the batch's previous one (stream order)
@@ -467,7 +469,7 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
         const size_t off = size_t(t - src_lo) * C::kTile;
         return arr == 0 ? reinterpret_cast<const uint8_t*>(src_phi + off) : reinterpret_cast<const uint8_t*>(src_W + off);
       },
-      [&](const uint8_t* const* stage, int64_t t) {
+      [&](const uint8_t* const* stage, int64_t t, const auto& release) {
         if (t < lo || t >= hi) {
           cur = find(t);
           lo = tile0[cur];
@@ -478,10 +480,12 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
         if constexpr (M == 4) {
           if (a.np.narrow) {
             fwd_tile<N, M, TAU1, ST, true, WIDE>(stage, local, a);
+            release();
             return;
           }
         }
         fwd_tile<N, M, TAU1, ST, false, WIDE>(stage, local, a);
+        release();
       });
   if (ok) {
     for (int i = blockIdx.x; i < mm.count; i += gridDim.x) {

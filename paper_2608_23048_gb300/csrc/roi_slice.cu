@@ -1,12 +1,11 @@
 // Wide groups (M = 16, 32: the 8:16 and 16:32 patterns) on warp slices: the
-// SL = M / 4 consecutive lanes of a slice hold one group, four members each.  Same method as the
-// one-thread-per-group kernels (Sec. 4.2.2 Eq. 10-12, Algorithm 1; Eq. 5;
-// backward through the relaxation), with the per-group sums, maxima and "sum of
-// the other members" formed across the slice by a shuffle butterfly that never
-// subtracts.  A thread holds the slots t and t + 256 of a tile; where registers
-// allow, the two groups of those slots are relaxed in lockstep on packed FP32
-// (V = F2, one group per half), otherwise one after the other (V = float).
-// Groups whose keys leave the fast path's range are queued by the slice's first
+// SL = M / P consecutive lanes of a slice hold one group, P = 8 or 16 members each, as
+// packed pairs of neighbouring members (F2).  Same method as the one-thread-per-group
+// kernels (Sec. 4.2.2 Eq. 10-12, Algorithm 1; Eq. 5; backward through the relaxation),
+// with the per-group sums and "sum of the other members" formed in the thread and then
+// across the slice's lanes by a shuffle butterfly that never subtracts.  The step loops
+// are rolled: the history of the relaxation that the backward sweeps is indexed in shared
+// memory.  Groups whose keys leave the fast path's range are queued by the slice's first
 // lane (DeferredGroups) and handled 32 at a time, one per lane, by WideRobustGroup
 // (ExactGroup for non-finite keys).
 #include "roi_launch.h"
@@ -15,117 +14,151 @@
 namespace roi {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kTile = 2048;  // 512 four-member slots: slots t and t + 256 per thread
-constexpr int kStagesFwd = 4;
-// backward ring stages: two at 8:16, whose two CTAs per SM also hold their step
-// histories in shared memory, three at 16:32 (one CTA per SM)
+// Launch shapes: threads per CTA (one CTA per SM in either direction), ring stages.
+// The backward keeps steps 0 .. N-3 of the relaxation in shared memory behind the ring
+// (4 P bytes a thread and step) and the last two in registers.
 template <int M>
-constexpr int kStagesBwd = M == 16 ? 2 : 3;
-// Both directions relax the two slots of a thread in lockstep on packed FP32; the
-// backward keeps its step history in shared memory behind the tile ring.  CTAs per
-// SM the registers are sized for (measured on the 3B-shaped set, tau = 0.2):
-// forward two; backward two at 8:16 (128 registers) and one at 16:32, whose paired
-// sixteen steps take 255 registers (at two CTAs it spills: 86.4 against 65.3 ms).
+struct FwdShape {
+  static constexpr int kP = 16;  // members of a group per lane
+  static constexpr int kThreads = 512;
+  static constexpr int kStages = 2;
+};
 template <int M>
-constexpr bool kPairedFwd = true;
-template <int M>
-constexpr bool kPairedBwd = true;
-constexpr int kMinBlocksFwd = 2;
-template <int M>
-constexpr int kMinBlocksBwd = M == 32 ? 1 : 2;
-// The backward's step history: steps 0 .. N-2 of one slot, or of the two slots of
-// a pair (four floats or F2 a step), per thread, thread-strided so a warp touches
-// consecutive words; the last step stays in registers.  Behind it, per step, the
-// sum of mu over the slice's other lanes, which the sweep needs for 1 - mu.
-template <int M>
-constexpr size_t kSliceHistOffset = (tile_smem_bytes<kTile, kStagesBwd<M>>(8) + 15) & ~size_t(15);
-template <int M>
-constexpr bool kReloadHist = M == 16;
-// Deferred exact-routine groups (DeferredGroups): a warp queues at most 64 / SL
-// groups per tile (or per round of the ragged tail) and drains once 32 are queued.
-constexpr int kDeferCap = 48;
-// The kernels queue flagged groups (DeferredGroups) and run the exact routine for
-// them 32 at a time.  Measured on the 3B-shaped set: at tau = 0.2 (no group flagged)
-// the 16:32 step takes 87.3 ms with the queue against 94.3 ms with the exact routine
-// in place; at tau = 0.05 (~4 % flagged) 8:16 takes 52.8 ms against 2424 ms and
-// 16:32 135 ms against 14.7 s.
-constexpr size_t kDeferBytes = size_t(kDeferCap) * 8 * (kThreads / 32);
-constexpr size_t kFwdDeferOffset = (tile_smem_bytes<kTile, kStagesFwd>(6) + 15) & ~size_t(15);
+struct BwdShape {
+  static constexpr int kP = 16;
+  static constexpr int kThreads = M == 16 ? 384 : 256;
+  static constexpr int kStages = 1;
+  static constexpr int kRegSteps = M == 16 ? 2 : 4;  // last steps of the history kept in registers
+};
+template <class Shape>
+constexpr int kTileOf = Shape::kThreads * Shape::kP;  // elements
 template <int N, int M>
-constexpr size_t kSliceHistBytes = size_t(N - 1) * 5 * (kPairedBwd<M> ? 8 : 4) * kThreads;
+constexpr size_t kHistOffset = (tile_smem_bytes<kTileOf<BwdShape<M>>, BwdShape<M>::kStages>(8) + 15) & ~size_t(15);
 template <int N, int M>
-constexpr size_t kSliceDeferOffset = (kSliceHistOffset<M> + kSliceHistBytes<N, M> + 15) & ~size_t(15);
+constexpr size_t kHistBytes = size_t(N - BwdShape<M>::kRegSteps) * BwdShape<M>::kP * sizeof(float) * BwdShape<M>::kThreads;
+// Deferred groups: a warp queues at most 32 / SL of them at a time and drains once 32
+// are queued.  (3B-shaped set, tau = 0.05, ~4 % of the groups: 8:16 52.8 ms a step with
+// the queue against 2424 ms with the routine in place.)
+template <int M, class Shape>
+constexpr int kDeferCap = 31 + 32 * Shape::kP / M;
+template <int M, class Shape>
+constexpr size_t kDeferBytes = size_t(kDeferCap<M, Shape>) * 8 * (Shape::kThreads / 32);
+
+template <int M>
+constexpr size_t kFwdDeferOffset = (tile_smem_bytes<kTileOf<FwdShape<M>>, FwdShape<M>::kStages>(6) + 15) & ~size_t(15);
+template <int N, int M>
+constexpr size_t kBwdDeferOffset = (kHistOffset<N, M> + kHistBytes<N, M> + 15) & ~size_t(15);
+
+// The tau != 1 kernels' relaxation: the plain one costs 10 to 15 % less while few groups
+// leave its range (8:16, one 11008 x 2048 tensor, forward + backward, plain / WIDE: 254 /
+// 291 us at tau = 0.2, 288 / 292 at 0.08, 294 / 292 at 0.06; 16:32: 484 / 562 at 0.2,
+// 576 / 560 at 0.1), and at small tau lambda nearly all groups of spread logits do.
+constexpr float kSliceWideTau = 0.1f;
+constexpr float kSliceWideTauLambda = 0.05f;
+constexpr float kLeastRange = -98.0f;  // of the plain tau != 1 relaxation (SliceRelax::forward)
 
 __device__ __forceinline__ float shfl_xor(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
-__device__ __forceinline__ F2 shfl_xor(F2 v, int o) {
-  return f2(__shfl_xor_sync(0xffffffffu, lo(v), o), __shfl_xor_sync(0xffffffffu, hi(v), o));
-}
-__device__ __forceinline__ float shfl_idx(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-__device__ __forceinline__ F2 shfl_idx(F2 v, int src) {
-  return f2(__shfl_sync(0xffffffffu, lo(v), src), __shfl_sync(0xffffffffu, hi(v), src));
-}
+__device__ __forceinline__ F2 swap(F2 v) { return f2(hi(v), lo(v)); }
 
-template <int SL, class V>
-struct Slice {
-  static_assert(SL == 4 || SL == 8, "slices of 4 or 8 lanes");
-  // Sum over the slice's other lanes (never total minus own) and the total,
-  // identical on every lane of the slice.
-  __device__ __forceinline__ static V others(V p, V& tot) {
-    V oth = shfl_xor(p, 1), acc = vadd(p, oth);
+// Sum of v over the slice's other lanes (never total minus own).
+template <int SL>
+__device__ __forceinline__ float sum_others(float v) {
+  float oth = 0.0f;
 #pragma unroll
-    for (int o = 2; o < SL; o <<= 1) {
-      const V sib = shfl_xor(acc, o);
-      oth = vadd(oth, sib);
-      acc = vadd(acc, sib);
-    }
-    tot = acc;
-    return oth;
+  for (int o = 1; o < SL; o <<= 1) {
+    const float sib = shfl_xor(v, o);
+    oth = o == 1 ? sib : __fadd_rn(oth, sib);
+    v = __fadd_rn(v, sib);
   }
-  __device__ __forceinline__ static V total(V p) {
-    V t;
-    others(p, t);
-    return t;
-  }
-  __device__ __forceinline__ static V max(V v) {
+  return oth;
+}
+// Sum over the group of a packed per-lane partial.
+template <int SL>
+__device__ __forceinline__ float group_sum(F2 p) {
+  float v = __fadd_rn(lo(p), hi(p));
 #pragma unroll
-    for (int o = 1; o < SL; o <<= 1) v = vmax(v, shfl_xor(v, o));
-    return v;
-  }
-  __device__ __forceinline__ static uint32_t any(uint32_t f) {
+  for (int o = 1; o < SL; o <<= 1) v = __fadd_rn(v, shfl_xor(v, o));
+  return v;
+}
+template <int H>
+__device__ __forceinline__ F2 sum_pk(const F2 (&x)[H]) {
+  F2 t[H / 2];
 #pragma unroll
-    for (int o = 1; o < SL; o <<= 1) f |= __shfl_xor_sync(0xffffffffu, f, o);
-    return f;
-  }
-};
-
-template <class V>
-__device__ __forceinline__ V sum4(const V (&x)[4]) {
-  return vadd(vadd(x[0], x[1]), vadd(x[2], x[3]));
-}
-template <class V>
-__device__ __forceinline__ void excl4(const V (&x)[4], V oth, V (&ex)[4]) {
-  const V p01 = vadd(x[0], x[1]), p23 = vadd(x[2], x[3]);
-  ex[0] = vadd(vadd(x[1], p23), oth);
-  ex[1] = vadd(vadd(x[0], p23), oth);
-  ex[2] = vadd(vadd(p01, x[3]), oth);
-  ex[3] = vadd(vadd(p01, x[2]), oth);
-}
-template <class V>
-__device__ __forceinline__ V max4(const V (&x)[4]) {
-  return vmax(vmax(x[0], x[1]), vmax(x[2], x[3]));
-}
-template <class V>
-__device__ __forceinline__ V min4(const V (&x)[4]) {
-  return vmin(vmin(x[0], x[1]), vmin(x[2], x[3]));
-}
-template <class V>
-__device__ __forceinline__ float lane_of(V v, int h) {
-  if constexpr (vlanes<V>() == 1) {
-    return v;
+  for (int i = 0; i < H / 2; ++i) t[i] = x[2 * i] + x[2 * i + 1];
+  if constexpr (H == 2) {
+    return t[0];
   } else {
-    return h == 0 ? lo(v) : hi(v);
+    return sum_pk(t);
   }
+}
+// For every member the sum over the group's other members, and the group's total: the
+// pairs' halves are summed in lockstep, and each half's total and the other lanes' enter
+// the other half's sums.
+template <int SL, int H>
+__device__ __forceinline__ float exclusive(const F2 (&x)[H], F2 (&ex)[H]) {
+  static_assert(H == 4 || H == 8, "8 or 16 members a lane");
+  if constexpr (H == 4) {
+    const F2 p = x[0] + x[1], q = x[2] + x[3];
+    const F2 t = p + q;
+    const float own = __fadd_rn(lo(t), hi(t));
+    const float oth = sum_others<SL>(own);
+    const F2 beyond = SL == 1 ? swap(t) : swap(t) + f2(oth);
+    const F2 p1 = p + beyond, q1 = q + beyond;
+    ex[0] = x[1] + q1;
+    ex[1] = x[0] + q1;
+    ex[2] = x[3] + p1;
+    ex[3] = x[2] + p1;
+    return SL == 1 ? own : __fadd_rn(own, oth);
+  } else {
+    F2 p[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) p[i] = x[2 * i] + x[2 * i + 1];
+    const F2 q0 = p[0] + p[1], q1 = p[2] + p[3];
+    const F2 t = q0 + q1;
+    const float own = __fadd_rn(lo(t), hi(t));
+    const float oth = sum_others<SL>(own);
+    const F2 beyond = SL == 1 ? swap(t) : swap(t) + f2(oth);
+    const F2 r0 = q0 + beyond, r1 = q1 + beyond;
+    const F2 e[4] = {p[1] + r1, p[0] + r1, p[3] + r0, p[2] + r0};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      ex[2 * i] = x[2 * i + 1] + e[i];
+      ex[2 * i + 1] = x[2 * i] + e[i];
+    }
+    return SL == 1 ? own : __fadd_rn(own, oth);
+  }
+}
+template <int SL, int H>
+__device__ __forceinline__ float group_max(const F2 (&x)[H]) {
+  float m = fmaxf(lo(x[0]), hi(x[0]));
+#pragma unroll
+  for (int i = 1; i < H; ++i) m = fmax3(m, lo(x[i]), hi(x[i]));
+#pragma unroll
+  for (int o = 1; o < SL; o <<= 1) m = fmaxf(m, shfl_xor(m, o));
+  return m;
+}
+// The group's second largest value (ties count twice).
+template <int SL, int H>
+__device__ __forceinline__ float group_second(const F2 (&x)[H]) {
+  float h[H], s[H];
+#pragma unroll
+  for (int i = 0; i < H; ++i) h[i] = fmaxf(lo(x[i]), hi(x[i])), s[i] = fminf(lo(x[i]), hi(x[i]));
+#pragma unroll
+  for (int w = H / 2; w >= 1; w >>= 1) {
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      s[i] = fmax3(fminf(h[i], h[i + w]), s[i], s[i + w]);
+      h[i] = fmaxf(h[i], h[i + w]);
+    }
+  }
+  float m1 = h[0], m2 = s[0];
+#pragma unroll
+  for (int o = 1; o < SL; o <<= 1) {
+    const float o1 = shfl_xor(m1, o), o2 = shfl_xor(m2, o);
+    m2 = fmax3(fminf(m1, o1), m2, o2);
+    m1 = fmaxf(m1, o1);
+  }
+  return m2;
 }
 
 struct SliceArgs {
@@ -150,296 +183,339 @@ struct SliceArgs {
   unsigned int* status;
 };
 
-// Dynamic shared memory of the backward kernel (tile ring, then the step history).
+// Dynamic shared memory of the kernels (tile ring, then the step history, the queues).
 extern __shared__ __align__(128) uint8_t roi_slice_smem[];
 
-// Keys (log2 units, t = kappa log2 e) of L four-member slots (one per lane of V)
-// whose first elements have call-flat indices e0[h].
-template <class V>
-__device__ __forceinline__ void slot_keys(const float* const* p4, const int64_t* e0, const NoiseParams& np,
-                                          V (&kap)[4]) {
-  constexpr int L = vlanes<V>();
-  float ph[L][4];
-  uint32_t x[L][4];
+// Keys (log2 units, t = kappa log2 e) of the 2 H members whose logits are at p and whose
+// first has call-flat index e0 (a multiple of 8, as the call's first element is).
+template <int H>
+__device__ __forceinline__ void lane_keys(const float* p, int64_t e0, const NoiseParams& np, F2 (&kap)[H]) {
+  const uint64_t q = (np.e_base + uint64_t(e0)) >> 2;
 #pragma unroll
-  for (int h = 0; h < L; ++h) {
-    const float4 p = *reinterpret_cast<const float4*>(p4[h]);
-    ph[h][0] = p.x, ph[h][1] = p.y, ph[h][2] = p.z, ph[h][3] = p.w;
-    const uint4 q = noise_block_q(np, (np.e_base + uint64_t(e0[h])) >> 2);
-    x[h][0] = q.x, x[h][1] = q.y, x[h][2] = q.z, x[h][3] = q.w;
-  }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    V one_plus, phv;
-    if constexpr (L == 1) {
-      one_plus = one_plus_from_word(x[0][j]);
-      phv = ph[0][j];
-    } else {
-      one_plus = f2(one_plus_from_word(x[0][j]), one_plus_from_word(x[1][j]));
-      phv = f2(ph[0][j], ph[1][j]);
-    }
-    const V u = vsub(one_plus, vconst<V>(__uint_as_float(0x3f7fffffu)));
-    kap[j] = key_log2(phv, u, np.l2e_inv_lam);
+  for (int s = 0; s < H / 2; ++s) {
+    const float4 v = reinterpret_cast<const float4*>(p)[s];
+    const uint4 x = noise_block_q(np, q + s);
+    const F2 half = vconst<F2>(__uint_as_float(0x3f7fffffu));
+    kap[2 * s] = key_log2(f2(v.x, v.y), f2(one_plus_from_word(x.x), one_plus_from_word(x.y)) - half, np.l2e_inv_lam);
+    kap[2 * s + 1] =
+        key_log2(f2(v.z, v.w), f2(one_plus_from_word(x.z), one_plus_from_word(x.w)) - half, np.l2e_inv_lam);
   }
 }
 
-// Forward relaxation of the group(s) held by this slice; mu of every step kept
-// if KEEP.  forward() returns the fallback flags (bit h: lane h of V), uniform
-// over the slice.
-constexpr float kTinyTotal = 7.52316384526264e-37f;  // 2^-120
-
-template <int N, int M, bool TAU1, bool KEEP, class V>
+// Forward relaxation of the group held by this slice; with KEEP every step's mu is kept
+// for backward().  WIDE (tau != 1): as FastGroup's, no finite key leaves the range.
+template <int N, int M, int P, bool TAU1, bool KEEP, bool WIDE>
 struct SliceRelax {
-  static constexpr int SL = M / 4;
-  // KEEP: mu of the last step in registers, of steps 0 .. N-2 in shared memory
-  // at hist[(4 k + j) kThreads] (V = float)
-  V mu_last[4];
-  V* hist;
-  V S[4];
-  V rt_last;
-  __device__ __forceinline__ void put(int k, int j, V v) {
-    if (k == N - 1) {
-      mu_last[j] = v;
-    } else {
-      hist[(4 * k + j) * kThreads] = v;
+  static constexpr int SL = M / P;
+  static constexpr int kPk = P / 2;
+  static constexpr int T = BwdShape<M>::kThreads;
+  F2 S[kPk];                 // without KEEP
+  // KEEP: mu of the last R steps here, of the others in hist[(k P / 4 + i) T]
+  static constexpr int R = BwdShape<M>::kRegSteps;
+  F2 keep[KEEP ? R : 1][kPk];
+  ulonglong2* hist;
+
+  __device__ __forceinline__ void put(int k, const F2 (&mu)[kPk]) {
+#pragma unroll
+    for (int i = 0; i < P / 4; ++i) hist[(k * (P / 4) + i) * T] = make_ulonglong2(mu[2 * i].v, mu[2 * i + 1].v);
+  }
+  __device__ __forceinline__ void get(int k, F2 (&mu)[kPk]) const {
+#pragma unroll
+    for (int i = 0; i < P / 4; ++i) {
+      const ulonglong2 a = hist[(k * (P / 4) + i) * T];
+      mu[2 * i].v = a.x, mu[2 * i + 1].v = a.y;
     }
   }
-  __device__ __forceinline__ V get(int k, int j) const { return k == N - 1 ? mu_last[j] : hist[(4 * k + j) * kThreads]; }
-  // the other lanes' sum of mu of step k < N - 1, kept by forward() for the sweep
-  __device__ __forceinline__ void put_oth(int k, V v) { hist[(4 * (N - 1) + k) * kThreads] = v; }
-  __device__ __forceinline__ V get_oth(int k) const { return hist[(4 * (N - 1) + k) * kThreads]; }
-  __device__ __forceinline__ void get4(int k, V (&m)[4]) const {
+  // KEEP: the soft mask, summed from the history on demand (the backward's optional dW)
+  __device__ __forceinline__ void soft(F2 (&s)[kPk]) const {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) m[j] = get(k, j);
-  }
-  // S_j: accumulated by forward() without KEEP; with KEEP summed from the history
-  // on demand (in forward()'s order), which only the backward's optional dW asks for.
-  __device__ __forceinline__ V soft(int j) const {
-    if constexpr (!KEEP) {
-      return S[j];
-    } else {
-      V t = get(0, j);
+    for (int i = 0; i < kPk; ++i) {
+      s[i] = keep[0][i];
 #pragma unroll
-      for (int k = 1; k < N; ++k) t = vadd(t, get(k, j));
-      return t;
+      for (int j = 1; j < R; ++j) s[i] = s[i] + keep[j][i];
+    }
+#pragma unroll 1
+    for (int k = 0; k < N - R; ++k) {
+      F2 mu[kPk];
+      get(k, mu);
+#pragma unroll
+      for (int i = 0; i < kPk; ++i) s[i] = s[i] + mu[i];
     }
   }
 
-  __device__ __forceinline__ uint32_t forward(const V (&kap)[4], float inv_tau, int base_lane) {
-    uint32_t flag = 0;
-    V cur[4];
-    if constexpr (TAU1) {
-      // weights relative to the slice's first key; a member more than 100 log2
-      // units from it (or a non-finite key) sends the group to the exact routine
-      const V kref = shfl_idx(kap[0], base_lane);
-      V e[4];
+  // One step's mu joins the history or the soft mask.
+  __device__ __forceinline__ void use(int k, const F2 (&e)[kPk], F2 r) {
+    if constexpr (KEEP) {
+      F2 mu[kPk];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) e[j] = vmap(vsub(kap[j], kref), ex2_approx);
-      V tot;
-      Slice<SL, V>::others(sum4(e), tot);
-      flag = vbelow(min4(e), kTinyExcl) | vbelow(vsub(vconst<V>(1.0f / kTinyExcl), tot), 0.0f);
-      const V r = vmap(tot, rcp_approx);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) cur[j] = vmul(e[j], r);
-#pragma unroll
-      for (int k = 0; k < N; ++k) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if constexpr (KEEP) put(k, j, cur[j]);
-          if constexpr (!KEEP) S[j] = k == 0 ? cur[j] : vadd(S[j], cur[j]);
-        }
-        if (k + 1 < N) {
-          V totc, o[4], v[4];
-          const V oth = Slice<SL, V>::others(sum4(cur), totc);
-          if constexpr (KEEP) put_oth(k, oth);
-          excl4(cur, oth, o);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) v[j] = vmul(cur[j], o[j]);
-          const V rt = vmap(Slice<SL, V>::total(sum4(v)), rcp_approx);
-          if (k == N - 2) rt_last = rt;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) cur[j] = vmul(v[j], rt);
-        }
-      }
-    } else {
-      const V kmax = Slice<SL, V>::max(max4(kap));
-      const V sc = vconst<V>(inv_tau);
-      V d[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) d[j] = vmul(vsub(kap[j], kmax), sc);
-      flag = vbelow(vsub(kmax, kmax), 0.0f);  // non-finite maximum
-#pragma unroll
-      for (int k = 0; k < N; ++k) {
-        V e[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) e[j] = vmap(d[j], ex2_approx);
-        V tot;
-        const V oth = Slice<SL, V>::others(sum4(e), tot);
-        const V r = vmap(tot, rcp_approx);
-        if constexpr (KEEP) {
-          if (k + 1 < N) put_oth(k, vmul(oth, r));
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          cur[j] = vmul(e[j], r);
-          if constexpr (KEEP) put(k, j, cur[j]);
-          if constexpr (!KEEP) S[j] = k == 0 ? cur[j] : vadd(S[j], cur[j]);
-        }
-        if (k + 1 < N) {
-          // d_l += log2(1 - mu_l) / tau, the offsets first renormalised by log2 of the
-          // total (so sum 2^d = 1, every offset <= 0 and the largest >= -log2 M): the
-          // total comes from the butterfly above, so no maximum over the slice is
-          // needed on the step's critical path.  A group whose exclusive sums drop
-          // below 2^-100 of the total, or whose total drops below 2^-120 (offsets that
-          // fell too far in one step, possible only for tau well below 0.05), goes
-          // to the exact routine.
-          V ex[4], om[4];
-          excl4(e, oth, ex);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) om[j] = vmul(ex[j], r);
-          flag |= vbelow(min4(om), kTinyExcl) | vbelow(tot, kTinyTotal);
-          const V lz = vmap(tot, lg2_approx);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) d[j] = vfma(vmap(om[j], lg2_approx), sc, vsub(d[j], lz));
-        }
-      }
-    }
-    return Slice<SL, V>::any(flag);
-  }
-
-  // dk = dL/dkappa of this slot's members for c = dL/dS (the sweep of FastGroup).
-  __device__ __forceinline__ void backward(const V (&c)[4], float inv_tau, V (&dk)[4]) const {
-    static_assert(KEEP, "needs the steps");
-    const V itau = vconst<V>(inv_tau);
-    V b[4], hl[4];
-    {
-      V cm[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) cm[j] = vmul(c[j], mu_last[j]);
-      const V cmu = Slice<SL, V>::total(sum4(cm));
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        V t = vsub(c[j], cmu);
-        if constexpr (!TAU1) t = vmul(itau, t);
-        b[j] = vmul(mu_last[j], t);
-        if constexpr (TAU1) hl[j] = vmul(vmul(get(N - 2, j), rt_last), t);
-      }
-    }
-#pragma unroll
-    for (int k = N - 2; k >= 0; --k) {
-      V cm[4], h[4], H[4], mk[4];
-      get4(k, mk);
-      if (TAU1 && k == N - 2) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) h[j] = hl[j];
+      for (int i = 0; i < kPk; ++i) mu[i] = e[i] * r;
+      if (k < N - R) {
+        put(k, mu);
       } else {
-        V om[4];
-        excl4(mk, get_oth(k), om);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) h[j] = vmul(b[j], vmap(om[j], rcp_approx));
+        for (int j = 0; j < R; ++j)
+          if (k == N - R + j) {
+#pragma unroll
+            for (int i = 0; i < kPk; ++i) keep[j][i] = mu[i];
+          }
       }
-      // c_l - <c, mu> + H_l - B as (c_l + H_l) - K, K = <c, mu> + B = sum of (c mu + b)
+    } else {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) cm[j] = vfma(c[j], mk[j], b[j]);
-      const V K = Slice<SL, V>::total(sum4(cm));
-      V tmp;
-      excl4(h, Slice<SL, V>::others(sum4(h), tmp), H);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const V mu_j = TAU1 ? mk[j] : vmul(mk[j], itau);
-        b[j] = vfma(mu_j, vsub(vadd(c[j], H[j]), K), b[j]);
-      }
+      for (int i = 0; i < kPk; ++i) S[i] = vfma(e[i], r, S[i]);
     }
+  }
+
+  // Returns whether the group left the float range (or has a non-finite key), the same on
+  // every lane of the slice.
+  __device__ __forceinline__ bool forward(const F2 (&kap)[kPk], float inv_tau, int base_lane) {
+    const F2 itau = f2(inv_tau);
+    constexpr int kPeel = KEEP ? R : 1;  // steps outside the rolled loop
+    bool flag = false;
+    F2 x[kPk], e[kPk], ex[kPk];
+    if constexpr (!KEEP) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) dk[j] = b[j];
+      for (int i = 0; i < kPk; ++i) S[i] = f2(0.0f);
+    }
+    if constexpr (TAU1) {
+      // weights relative to the slice's first key; a member more than 100 log2 units from
+      // it (or a non-finite key) sends the group to the exact routine
+      const F2 ref = f2(__shfl_sync(0xffffffffu, lo(kap[0]), base_lane));
+      float emin = INFINITY;
+#pragma unroll
+      for (int i = 0; i < kPk; ++i) {
+        x[i] = vmap(kap[i] - ref, ex2_approx);
+        emin = fminf(emin, fminf(lo(x[i]), hi(x[i])));
+      }
+      const float tot = group_sum<SL>(sum_pk(x));
+      bool out = !(emin >= kTinyExcl) || !(tot <= 1.0f / kTinyExcl);
+      flag = (__ballot_sync(0xffffffffu, out) >> base_lane & ((1u << SL) - 1u)) != 0u;
+      F2 r = f2(rcp_approx(tot));
+      auto step = [&](int k) {
+        use(k, x, r);
+        if (k + 1 < N) {
+          F2 cur[kPk];
+#pragma unroll
+          for (int i = 0; i < kPk; ++i) cur[i] = x[i] * r;
+          exclusive<SL>(cur, ex);
+#pragma unroll
+          for (int i = 0; i < kPk; ++i) x[i] = cur[i] * ex[i];
+          r = f2(rcp_approx(group_sum<SL>(sum_pk(x))));
+        }
+      };
+#pragma unroll 2
+      for (int k = 0; k < N - kPeel; ++k) step(k);
+#pragma unroll
+      for (int k = N - kPeel; k < N; ++k) step(k);
+    } else if constexpr (WIDE) {
+      float sq = 0.0f;
+#pragma unroll
+      for (int i = 0; i < kPk; ++i) sq = fmaf(lo(kap[i]), lo(kap[i]), fmaf(hi(kap[i]), hi(kap[i]), sq));
+      sq = group_sum<SL>(f2(sq, 0.0f));
+      flag = !(sq - sq >= 0.0f);  // a non-finite key, or one beyond 2^63
+      const F2 ref = f2(group_second<SL>(kap));
+#pragma unroll
+      for (int i = 0; i < kPk; ++i) x[i] = (kap[i] - ref) * itau;
+      auto step = [&](int k) {
+        F2 c[kPk];
+#pragma unroll
+        for (int i = 0; i < kPk; ++i) {
+          c[i] = vmin(x[i], f2(kLeadCap));
+          e[i] = vmap(c[i], ex2_approx);
+        }
+        if (k + 1 < N) {
+          const F2 r = f2(rcp_approx(exclusive<SL>(e, ex)));
+          use(k, e, r);
+#pragma unroll
+          for (int i = 0; i < kPk; ++i) x[i] = vfma(vmap(ex[i] * r, lg2_approx) - (x[i] - c[i]), itau, x[i]);
+          const F2 m = f2(group_second<SL>(x));
+#pragma unroll
+          for (int i = 0; i < kPk; ++i) x[i] = x[i] - m;
+        } else {
+          use(k, e, f2(rcp_approx(group_sum<SL>(sum_pk(e)))));
+        }
+      };
+#pragma unroll 1
+      for (int k = 0; k < N - kPeel; ++k) step(k);
+#pragma unroll
+      for (int k = N - kPeel; k < N; ++k) step(k);
+    } else {
+      const float kmax = group_max<SL>(kap);
+      // Range check, from the totals alone: a leader's complement eps (its share of the
+      // total) leaves a next total of at most eps + eps^(1 / tau), so eps times the total,
+      // the sum that was formed, is at least 2^-99 while
+      // log2 total + max(1, tau) log2 (next total) >= -98, and members that were flushed
+      // to zero are below the sum's last bit.
+      const float tau1 = fmaxf(1.0f, __fdiv_rn(1.0f, inv_tau));
+      float lz_prev = 0.0f;
+#pragma unroll
+      for (int i = 0; i < kPk; ++i) x[i] = (kap[i] - f2(kmax)) * itau;
+      auto step = [&](int k) {
+#pragma unroll
+        for (int i = 0; i < kPk; ++i) e[i] = vmap(x[i], ex2_approx);
+        const float tot = k + 1 < N ? exclusive<SL>(e, ex) : group_sum<SL>(sum_pk(e));
+        const float lz = lg2_approx(tot);
+        flag = flag || !(fmaf(lz, tau1, lz_prev) >= kLeastRange);
+        lz_prev = lz;
+        const F2 r = f2(rcp_approx(tot));
+        use(k, e, r);
+        if (k + 1 < N) {
+          // offset - log2(total) + log2(1 - mu) / tau: normalised, so that the weights of
+          // the next step start from mu
+#pragma unroll
+          for (int i = 0; i < kPk; ++i) x[i] = vfma(vmap(ex[i] * r, lg2_approx), itau, x[i] - f2(lz));
+        }
+      };
+#pragma unroll 1
+      for (int k = 0; k < N - kPeel; ++k) step(k);
+#pragma unroll
+      for (int k = N - kPeel; k < N; ++k) step(k);
+    }
+    return flag;
+  }
+
+  // After forward() with KEEP: dk = tau dL/dkappa of this lane's members for c = dL/dS (the
+  // sweep of FastGroup, with b = dk / tau).
+  __device__ __forceinline__ void backward(const F2 (&c)[kPk], float inv_tau, F2 (&b)[kPk]) const {
+    static_assert(KEEP, "needs the steps");
+    const F2 itau = f2(inv_tau);
+    {
+      F2 cm[kPk];
+#pragma unroll
+      for (int i = 0; i < kPk; ++i) cm[i] = c[i] * keep[R - 1][i];
+      const F2 cmu = f2(group_sum<SL>(sum_pk(cm)));
+#pragma unroll
+      for (int i = 0; i < kPk; ++i) b[i] = keep[R - 1][i] * (c[i] - cmu);
+    }
+    auto sweep = [&](const F2 (&mk)[kPk]) {
+      F2 om[kPk], h[kPk], H[kPk];
+      exclusive<SL>(mk, om);
+      // K = <c, mu> + sum b / tau
+      F2 dot = c[0] * mk[0];
+#pragma unroll
+      for (int i = 1; i < kPk; ++i) dot = vfma(c[i], mk[i], dot);
+      const F2 K = f2(group_sum<SL>(vfma(sum_pk(b), itau, dot)));
+#pragma unroll
+      for (int i = 0; i < kPk; ++i) h[i] = b[i] * vmap(om[i], rcp_approx);
+      exclusive<SL>(h, H);
+#pragma unroll
+      for (int i = 0; i < kPk; ++i) b[i] = vfma(mk[i], vfma(H[i], itau, c[i] - K), b[i]);
+    };
+#pragma unroll
+    for (int j = R - 2; j >= 0; --j) sweep(keep[j]);
+#pragma unroll 2
+    for (int k = N - R - 1; k >= 0; --k) {
+      F2 mk[kPk];
+      get(k, mk);
+      sweep(mk);
+    }
   }
 };
 
-// Hard bits of a slot: rank of each own key among the group's M keys.
-template <int M>
-__device__ __forceinline__ uint32_t slice_topn_bits(const float (&kap)[4], int N, int base_lane, int q) {
-  constexpr int SL = M / 4;
-  float kk[4];
-  int rank[4] = {0, 0, 0, 0};
+// Hard bits of a lane's members: rank of each own key among the group's M keys.
+template <int M, int P>
+__device__ __forceinline__ uint32_t slice_topn_bits(const float (&kap)[P], int N, int base_lane, int q) {
+  constexpr int SL = M / P;
+  float kk[P];
+  int rank[P];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) kk[j] = fmaxf(kap[j], -INFINITY);
-#pragma unroll
+  for (int j = 0; j < P; ++j) kk[j] = fmaxf(kap[j], -INFINITY), rank[j] = 0;
+#pragma unroll 1
   for (int qq = 0; qq < SL; ++qq) {
 #pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
+    for (int jj = 0; jj < P; ++jj) {
       const float ko = __shfl_sync(0xffffffffu, kk[jj], base_lane + qq);
-      const int io = qq * 4 + jj;
+      const int io = qq * P + jj;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int im = q * 4 + j;
+      for (int j = 0; j < P; ++j) {
+        const int im = q * P + j;
         rank[j] += io < im ? (ko >= kk[j]) : (io > im ? (ko > kk[j]) : 0);
       }
     }
   }
   uint32_t bits = 0;
 #pragma unroll
-  for (int j = 0; j < 4; ++j) bits |= uint32_t(rank[j] < N) << j;
+  for (int j = 0; j < P; ++j) bits |= uint32_t(rank[j] < N) << j;
   return bits;
 }
 
 // Compare-exchange keeping x[a] >= x[b].
-__device__ __forceinline__ void ce_desc(float (&x)[4], int a, int b) {
+template <int P>
+__device__ __forceinline__ void ce_desc(float (&x)[P], int a, int b) {
   const float u = x[a], v = x[b];
   x[a] = fmaxf(u, v);
   x[b] = fminf(u, v);
 }
-// Sorts a bitonic run of four descending.
-__device__ __forceinline__ void bitonic4_desc(float (&x)[4]) {
-  ce_desc(x, 0, 2), ce_desc(x, 1, 3), ce_desc(x, 0, 1), ce_desc(x, 2, 3);
+// Sorts x[at .. at + 7] descending (Batcher's odd-even merge network).
+template <int P>
+__device__ __forceinline__ void sort8_desc(float (&x)[P], int at) {
+  auto ce = [&](int a, int b) { ce_desc(x, at + a, at + b); };
+  ce(0, 1), ce(2, 3), ce(4, 5), ce(6, 7);
+  ce(0, 2), ce(1, 3), ce(4, 6), ce(5, 7);
+  ce(1, 2), ce(5, 6);
+  ce(0, 4), ce(1, 5), ce(2, 6), ce(3, 7);
+  ce(2, 4), ce(3, 5);
+  ce(1, 2), ce(3, 4), ce(5, 6);
 }
-// One bitonic merge step across lanes: with this lane's four keys sorted
-// descending and the partner lane's (lane ^ o) too, the lane keeps the larger
-// (upper = false) or smaller (upper = true) element of each pair (i, partner's
-// 3 - i); the result is a bitonic run, sorted again in the lane.
-__device__ __forceinline__ void merge_across(float (&x)[4], int o, bool upper) {
-  float p[4];
+// Sorts a bitonic run x[at .. at + n - 1] descending.
+template <int n, int P>
+__device__ __forceinline__ void bitonic_desc(float (&x)[P], int at) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) p[i] = __shfl_xor_sync(0xffffffffu, x[3 - i], o);
+  for (int d = n / 2; d >= 1; d >>= 1)
 #pragma unroll
-  for (int i = 0; i < 4; ++i) x[i] = upper ? fminf(x[i], p[i]) : fmaxf(x[i], p[i]);
-  bitonic4_desc(x);
+    for (int i = 0; i < n; ++i)
+      if ((i & d) == 0) ce_desc(x, at + i, at + i + d);
 }
 
-// Hard bits of a slot for N = M / 2 (the two patterns of these kernels) from the
-// group's N-th largest key.  Each lane sorts its four keys; bitonic merges across
-// lanes sort each half of the slice (M / 2 keys over SL / 2 lanes); the top M / 2
-// of the group are then the larger elements of the pairs (i-th of the first half,
-// i-th from the end of the second half), so their minimum is the threshold.  A
-// member is kept iff its key is at least the threshold.  Returns false (bits
-// unusable) if the slice's keys are not all finite or the threshold is tied, so
-// that more than N members pass: the caller ranks such groups by comparison.
-template <int N, int M>
-__device__ __forceinline__ bool slice_topn_threshold(const float (&kap)[4], int q, uint32_t& bits) {
+// Hard bits of a lane's members for N = M / 2 (the two patterns of these kernels) from the
+// group's N-th largest key: each half of the group is sorted, in the lane and (P = 8,
+// M = 32) by a bitonic merge across lane pairs (the partner's keys in reverse, the larger
+// half to the lower lane); the top M / 2 of the group are then the larger elements of the
+// pairs (i-th of the first half, i-th from the end of the second), so their minimum is the
+// threshold.  A member is kept iff its key reaches it.  Returns false (bits unusable) if
+// the slice's keys are not all finite or the threshold is tied, so that more than N
+// members pass: the caller ranks such groups by comparison.
+template <int N, int M, int P>
+__device__ __forceinline__ bool slice_topn_threshold(const float (&kap)[P], int q, uint32_t& bits) {
   static_assert(2 * N == M, "threshold selection needs N = M / 2");
-  constexpr int SL = M / 4;
-  float x[4] = {kap[0], kap[1], kap[2], kap[3]};
-  ce_desc(x, 0, 1), ce_desc(x, 2, 3), ce_desc(x, 0, 2), ce_desc(x, 1, 3), ce_desc(x, 1, 2);
-  // sorted runs of 8 over lane pairs
-  merge_across(x, 1, (q & 1) != 0);
-  if constexpr (SL == 8) {
-    // sorted runs of 16 over lane quads: the larger / smaller 8 of the two runs of
-    // 8 go to the quad's lower / upper lane pair (each lane's four sorted), and a
-    // merge within each pair orders them
-    merge_across(x, 3, (q & 2) != 0);
-    merge_across(x, 1, (q & 1) != 0);
-  }
-  // pairs (i, M/2 - 1 - i) across the two halves: lane q pairs with lane SL - 1 - q
+  constexpr int SL = M / P;
+  float x[P];
+#pragma unroll
+  for (int i = 0; i < P; ++i) x[i] = kap[i];
+#pragma unroll
+  for (int i = 0; i < P; i += 8) sort8_desc(x, i);
   float m = INFINITY;
+  if constexpr (SL == 1) {
+    static_assert(SL != 1 || P == 16, "one lane a group: 16 members");
 #pragma unroll
-  for (int i = 0; i < 4; ++i) m = fminf(m, fmaxf(x[i], __shfl_xor_sync(0xffffffffu, x[3 - i], SL - 1)));
+    for (int i = 0; i < P / 2; ++i) m = fminf(m, fmaxf(x[i], x[P - 1 - i]));
+  } else {
+    if constexpr (P == 16) {
+      // the lane's two sorted runs into one
 #pragma unroll
-  for (int o = 1; o < SL / 2; o <<= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      for (int i = 0; i < 8; ++i) ce_desc(x, i, 15 - i);
+      bitonic_desc<8>(x, 0);
+      bitonic_desc<8>(x, 8);
+    }
+    if constexpr (SL == 4) {
+      float p[P];
+#pragma unroll
+      for (int i = 0; i < P; ++i) p[i] = shfl_xor(x[P - 1 - i], 1);
+      const bool upper = (q & 1) != 0;
+#pragma unroll
+      for (int i = 0; i < P; ++i) x[i] = upper ? fminf(x[i], p[i]) : fmaxf(x[i], p[i]);
+      bitonic_desc<P>(x, 0);
+    }
+#pragma unroll
+    for (int i = 0; i < P; ++i) m = fminf(m, fmaxf(x[i], shfl_xor(x[P - 1 - i], SL - 1)));
+#pragma unroll
+    for (int o = 1; o < SL / 2; o <<= 1) m = fminf(m, shfl_xor(m, o));
+  }
   bits = 0;
   float fin = 0.0f;
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    bits |= uint32_t(kap[j] >= m) << j;
-    fin += kap[j] - kap[j];  // 0 for finite keys, NaN otherwise
+  for (int i = 0; i < P; ++i) {
+    bits |= uint32_t(kap[i] >= m) << i;
+    fin += kap[i] - kap[i];  // 0 for finite keys, NaN otherwise
   }
   int cnt = __popc(bits) + (fin == 0.0f ? 0 : 64);
 #pragma unroll
@@ -447,22 +523,21 @@ __device__ __forceinline__ bool slice_topn_threshold(const float (&kap)[4], int 
   return cnt == N;
 }
 
-// Hard bits of L slots (one per lane of V): the threshold selection, and for a
-// group it cannot settle (a tie at the threshold, a non-finite key) comparison
-// ranking, run by the whole warp when any of its slots needs it.
-template <int N, int M, class V>
-__device__ __forceinline__ void slot_topn(const V (&kap)[4], int base_lane, int q, uint32_t (&bits)[vlanes<V>()]) {
+// Hard bits of a lane's members: the threshold selection, and for a group it cannot
+// settle (a tie at the threshold, a non-finite key) comparison ranking, run by the whole
+// warp when any of its groups needs it.
+template <int N, int M, int H>
+__device__ __forceinline__ uint32_t lane_topn(const F2 (&kap)[H], int base_lane, int q) {
+  float k[2 * H];
 #pragma unroll
-  for (int h = 0; h < vlanes<V>(); ++h) {
-    float k[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) k[j] = lane_of(kap[j], h);
-    const bool ok = slice_topn_threshold<N, M>(k, q, bits[h]);
-    if (__any_sync(0xffffffffu, !ok)) {
-      const uint32_t b = slice_topn_bits<M>(k, N, base_lane, q);
-      if (!ok) bits[h] = b;
-    }
+  for (int i = 0; i < H; ++i) k[2 * i] = lo(kap[i]), k[2 * i + 1] = hi(kap[i]);
+  uint32_t bits;
+  const bool ok = slice_topn_threshold<N, M>(k, q, bits);
+  if (__any_sync(0xffffffffu, !ok)) {
+    const uint32_t b = slice_topn_bits<M>(k, N, base_lane, q);
+    if (!ok) bits = b;
   }
+  return bits;
 }
 
 // The keys of all M elements of one group, in log2 units, from logits at phi_g
@@ -470,22 +545,20 @@ __device__ __forceinline__ void slot_topn(const V (&kap)[4], int base_lane, int 
 template <int N, int M>
 __device__ __forceinline__ void group_keys_all(const float* phi_g, int64_t g0, const NoiseParams& np, float (&k)[M]) {
 #pragma unroll
-  for (int s = 0; s < M / 4; ++s) {
-    const float* p[1] = {phi_g + 4 * s};
-    const int64_t e[1] = {g0 + 4 * s};
-    float k4[4];
-    slot_keys<float>(p, e, np, k4);
+  for (int s = 0; s < M / 8; ++s) {
+    F2 k8[4];
+    lane_keys(phi_g + 8 * s, g0 + 8 * s, np, k8);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) k[4 * s + j] = k4[j];
+    for (int i = 0; i < 4; ++i) k[8 * s + 2 * i] = lo(k8[i]), k[8 * s + 2 * i + 1] = hi(k8[i]);
   }
 }
-// The exact relaxation of one group with keys t (log2 units): WideRobustGroup for
-// finite keys, ExactGroup (natural-log keys) otherwise; soft mask S and, with c,
+// The exact relaxation of one group with keys t (log2 units): WideRobustGroup for finite
+// keys (which never come here from a WIDE kernel), ExactGroup (natural-log keys) otherwise; soft mask S and, with c,
 // dk = dL/dkappa.
-template <int N, int M, bool BWD>
+template <int N, int M, bool BWD, bool WIDE>
 __device__ __forceinline__ void exact_relax(float (&t)[M], const float (&c)[M], const SliceArgs& a, float (&S)[M],
                                             float (&dk)[M]) {
-  if (all_finite(t)) {
+  if (!WIDE && all_finite(t)) {
     WideRobustGroup<N, M> rg;
     rg.forward(t, a.inv_tau, S);
     if constexpr (BWD) rg.backward(c, a.inv_tau, dk);
@@ -513,12 +586,12 @@ __device__ __forceinline__ void unpack_bf16x4(uint2 q, float (&out)[4]) {
 
 // The exact routine for one group (first element g0, call-flat), from global
 // memory: the forward's outputs (Wm unless straight-through, soft).
-template <int N, int M>
+template <int N, int M, bool WIDE>
 __device__ __forceinline__ void exact_group_fwd(int64_t g0, const SliceArgs& a) {
   if (a.soft == nullptr && a.st) return;
   float k[M], S[M], unused[M];
   group_keys_all<N, M>(a.phi + g0, g0, a.np, k);
-  exact_relax<N, M, false>(k, k, a, S, unused);
+  exact_relax<N, M, false, WIDE>(k, k, a, S, unused);
 #pragma unroll 1
   for (int s = 0; s < M / 4; ++s) {
     float wv[4], sv[4];
@@ -532,7 +605,7 @@ __device__ __forceinline__ void exact_group_fwd(int64_t g0, const SliceArgs& a) 
 // The backward's outputs of one group: dphi, the fused AdamW step, dW unless the
 // straight-through variant (which wrote it with the fast path).  The group's logits
 // are untouched until here (the fast path skips its AdamW step).
-template <int N, int M>
+template <int N, int M, bool WIDE>
 __device__ __forceinline__ void exact_group_bwd(int64_t g0, const SliceArgs& a) {
   float k[M], cc[M], S[M], dkk[M];
   group_keys_all<N, M>(a.phi + g0, g0, a.np, k);
@@ -544,7 +617,7 @@ __device__ __forceinline__ void exact_group_bwd(int64_t g0, const SliceArgs& a) 
 #pragma unroll
     for (int j = 0; j < 4; ++j) cc[4 * s + j] = __fmul_rn(dv[j], wv[j]);
   }
-  exact_relax<N, M, true>(k, cc, a, S, dkk);
+  exact_relax<N, M, true, WIDE>(k, cc, a, S, dkk);
 #pragma unroll 1
   for (int s = 0; s < M / 4; ++s) {
     const int64_t e = g0 + 4 * s;
@@ -562,210 +635,197 @@ __device__ __forceinline__ void exact_group_bwd(int64_t g0, const SliceArgs& a) 
   }
 }
 
-// Forward of L slots (one per lane of V; p/w: each slot's logits and weights in
-// shared or global memory, e0: call-flat index of its first element).  All 32
-// lanes of the warp call this together; inactive slots (ragged tail, V = float
-// only) take part in the shuffles with zero keys.  Returns each slot's hard bits.
-template <int N, int M, bool TAU1, class V>
-__device__ __forceinline__ void fwd_slots(const float* const* p, const uint16_t* const* w, const int64_t* e0,
-                                          bool active, const SliceArgs& a, uint32_t (&bits)[vlanes<V>()],
-                                          uint32_t& defer) {
-  constexpr int SL = M / 4;
-  constexpr int L = vlanes<V>();
-  const int lane = threadIdx.x & 31;
-  const int q = lane % SL;
-  const int base_lane = lane - q;
-  V kap[4];
-  if (active) {
-    slot_keys<V>(p, e0, a.np, kap);
-  } else {
+// A lane's 2 H members' worth of bf16 at `p` (16-byte aligned).
+template <int H>
+__device__ __forceinline__ void unpack_lane(const uint16_t* p, F2 (&out)[H]) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) kap[j] = vconst<V>(0.0f);
+  for (int j = 0; j < H / 4; ++j) {
+    const uint4 v = reinterpret_cast<const uint4*>(p)[j];
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) out[4 * j + i] = f2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xffff0000u));
   }
-  slot_topn<N, M, V>(kap, base_lane, q, bits);
-  SliceRelax<N, M, TAU1, false, V> rx;
-  const uint32_t flag = rx.forward(kap, a.inv_tau, base_lane);
-  // groups out of the fast path's range: queued by their first lane for the exact
-  // routine, which writes their outputs
-  defer = active && q == 0 ? flag : 0u;
-  if (!active) return;
+}
+template <int H>
+__device__ __forceinline__ void store_lane(uint16_t* p, const F2 (&v)[H]) {
 #pragma unroll
-  for (int h = 0; h < L; ++h) {
-    // straight-through: every slot keeps the weights its hard bits select
-    if (a.st) *reinterpret_cast<uint2*>(a.Wm + e0[h]) = keep4(*reinterpret_cast<const uint2*>(w[h]), bits[h]);
-    if (!((flag >> h) & 1u)) {
-      float wv[4], sv[4];
-      unpack_bf16x4(*reinterpret_cast<const uint2*>(w[h]), wv);
+  for (int j = 0; j < H; j += 4)
+    reinterpret_cast<uint4*>(p)[j / 4] =
+        make_uint4(pack_bf16x2(lo(v[j]), hi(v[j])), pack_bf16x2(lo(v[j + 1]), hi(v[j + 1])),
+                   pack_bf16x2(lo(v[j + 2]), hi(v[j + 2])), pack_bf16x2(lo(v[j + 3]), hi(v[j + 3])));
+}
+template <int H>
+__device__ __forceinline__ void store_lane(float* p, const F2 (&v)[H]) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) sv[j] = lane_of(rx.S[j], h);
-      if (!a.st) *reinterpret_cast<uint2*>(a.Wm + e0[h]) = pack4(wv, sv);
-      if (a.soft != nullptr) *reinterpret_cast<float4*>(a.soft + e0[h]) = make_float4(sv[0], sv[1], sv[2], sv[3]);
-    }
+  for (int j = 0; j < H; j += 2)
+    reinterpret_cast<float4*>(p)[j / 2] = make_float4(lo(v[j]), hi(v[j]), lo(v[j + 1]), hi(v[j + 1]));
+}
+// Straight-through: the bf16 values of `src` where the bits are set, +0 elsewhere.
+template <int P>
+__device__ __forceinline__ void keep_lane(uint16_t* dst, const uint16_t* src, uint32_t bits) {
+#pragma unroll
+  for (int j = 0; j < P / 8; ++j) {
+    const uint4 v = reinterpret_cast<const uint4*>(src)[j];
+    const uint2 a = keep4(make_uint2(v.x, v.y), bits >> (8 * j)), b = keep4(make_uint2(v.z, v.w), bits >> (8 * j + 4));
+    reinterpret_cast<uint4*>(dst)[j] = make_uint4(a.x, a.y, b.x, b.y);
   }
 }
 
-// Backward of L slots (as fwd_slots).
-template <int N, int M, bool TAU1, class V>
-__device__ __forceinline__ void bwd_slots(const float* const* p, const uint16_t* const* w, const uint16_t* const* dw,
-                                          const int64_t* e0, bool active, const SliceArgs& a, uint32_t& defer) {
-  constexpr int SL = M / 4;
-  constexpr int L = vlanes<V>();
-  const int lane = threadIdx.x & 31;
-  const int q = lane % SL;
-  const int base_lane = lane - q;
-  V kap[4], c[4];
+// Forward of a lane's members (p, w: their logits and weights in shared or global memory,
+// e0: call-flat index of the first).  All 32 lanes call this together; inactive ones
+// (ragged tail) take part in the shuffles with zero keys.  Returns whether the group goes
+// to the exact routine (on its first lane).
+template <int N, int M, int P, bool TAU1, bool WIDE, class Release>
+__device__ __forceinline__ bool fwd_lane(const float* p, const uint16_t* w, int64_t e0, bool active, const SliceArgs& a,
+                                         const Release& release) {
+  constexpr int SL = M / P, kPk = P / 2;
+  const int lane = threadIdx.x & 31, q = lane % SL, base_lane = lane - q;
+  F2 kap[kPk];
   if (active) {
-    slot_keys<V>(p, e0, a.np, kap);
-    float wv[L][4], dv[L][4];
-#pragma unroll
-    for (int h = 0; h < L; ++h) {
-      unpack_bf16x4(*reinterpret_cast<const uint2*>(w[h]), wv[h]);
-      unpack_bf16x4(*reinterpret_cast<const uint2*>(dw[h]), dv[h]);
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if constexpr (L == 1) {
-        c[j] = vmul(dv[0][j], wv[0][j]);
-      } else {
-        c[j] = vmul(f2(dv[0][j], dv[1][j]), f2(wv[0][j], wv[1][j]));
-      }
-    }
+    lane_keys(p, e0, a.np, kap);
   } else {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) kap[j] = c[j] = vconst<V>(0.0f);
+    for (int i = 0; i < kPk; ++i) kap[i] = f2(0.0f);
   }
-  SliceRelax<N, M, TAU1, true, V> rx;
-  rx.hist = reinterpret_cast<V*>(roi_slice_smem + kSliceHistOffset<M>) + threadIdx.x;
-  const uint32_t flag = rx.forward(kap, a.inv_tau, base_lane);
-  defer = active && q == 0 ? flag : 0u;
+  uint32_t bits = 0;
+  if (a.hard != nullptr || a.st) bits = lane_topn<N, M>(kap, base_lane, q);
+  SliceRelax<N, M, P, TAU1, false, WIDE> rx;
+  const bool flag = rx.forward(kap, a.inv_tau, base_lane);
+  if (active) {
+    if (a.st) {
+      keep_lane<P>(a.Wm + e0, w, bits);
+    } else if (!flag) {
+      F2 m[kPk];
+      unpack_lane(w, m);
+#pragma unroll
+      for (int i = 0; i < kPk; ++i) m[i] = m[i] * rx.S[i];
+      store_lane(a.Wm + e0, m);
+    }
+    if (a.soft != nullptr && !flag) store_lane(a.soft + e0, rx.S);
+  }
+  release();
+  if (a.hard != nullptr) {
+    constexpr int kPerWord = 32 / P;
+    uint32_t v = active ? bits << ((lane % kPerWord) * P) : 0u;
+#pragma unroll
+    for (int o = 1; o < kPerWord; o <<= 1) v |= __shfl_xor_sync(0xffffffffu, v, o);
+    if (active && lane % kPerWord == 0) a.hard[e0 >> 5] = v;
+  }
+  return active && q == 0 && flag;
+}
+
+// Backward of a lane's members (as fwd_lane).
+template <int N, int M, int P, bool TAU1, bool WIDE, class Release>
+__device__ __forceinline__ bool bwd_lane(const float* p, const uint16_t* w, const uint16_t* dw, int64_t e0, bool active,
+                                         const SliceArgs& a, const Release& release) {
+  constexpr int SL = M / P, kPk = P / 2;
+  const int lane = threadIdx.x & 31, q = lane % SL, base_lane = lane - q;
+  F2 kap[kPk], c[kPk], b[kPk];
+  if (active) {
+    lane_keys(p, e0, a.np, kap);
+    F2 wv[kPk];
+    unpack_lane(w, wv);
+    unpack_lane(dw, c);
+#pragma unroll
+    for (int i = 0; i < kPk; ++i) c[i] = c[i] * wv[i];
+  } else {
+#pragma unroll
+    for (int i = 0; i < kPk; ++i) kap[i] = c[i] = f2(0.0f);
+  }
+  // the stage is free from here on: its refill lands during the relaxation, so one stage
+  // suffices and the shared memory goes to the step history
+  release();
+  SliceRelax<N, M, P, TAU1, true, WIDE> rx;
+  rx.hist = reinterpret_cast<ulonglong2*>(roi_slice_smem + kHistOffset<N, M>) + threadIdx.x;
+  const bool flag = rx.forward(kap, a.inv_tau, base_lane);
   if (active && a.dW != nullptr) {
+    if (a.hard_in != nullptr) {
+      // straight-through: dWm where the forward's hard mask is set
+      keep_lane<P>(a.dW + e0, a.dWm + e0, a.hard_in[e0 >> 5] >> (uint32_t(e0) & 31u));
+    } else if (!flag) {
+      F2 s[kPk], d[kPk];
+      rx.soft(s);
+      unpack_lane(a.dWm + e0, d);
 #pragma unroll
-    for (int h = 0; h < L; ++h) {
-      if (a.hard_in != nullptr) {
-        // straight-through: dWm where the forward's hard mask is set
-        *reinterpret_cast<uint2*>(a.dW + e0[h]) = keep4(*reinterpret_cast<const uint2*>(dw[h]), hard4(a.hard_in, e0[h]));
-      } else if (!((flag >> h) & 1u)) {
-        float dv[4], sv[4];
-        unpack_bf16x4(*reinterpret_cast<const uint2*>(dw[h]), dv);
+      for (int i = 0; i < kPk; ++i) s[i] = d[i] * s[i];
+      store_lane(a.dW + e0, s);
+    }
+  }
+  rx.backward(c, a.inv_tau, b);
+  if (active && !flag) {
+    const F2 scale = f2(a.inv_tau * a.np.inv_lam);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) sv[j] = lane_of(rx.soft(j), h);
-        *reinterpret_cast<uint2*>(a.dW + e0[h]) = pack4(dv, sv);
+    for (int i = 0; i < kPk; ++i) b[i] = b[i] * scale;
+    if (a.dphi != nullptr) store_lane(a.dphi + e0, b);
+    if (a.phi_out != nullptr) {
+#pragma unroll
+      for (int s = 0; s < P / 4; ++s) {
+        const float g4[4] = {lo(b[2 * s]), hi(b[2 * s]), lo(b[2 * s + 1]), hi(b[2 * s + 1])};
+        adamw4(a.phi_out, a.m, a.v, e0 + 4 * s, reinterpret_cast<const float4*>(a.phi + e0)[s], g4, a.opt);
       }
     }
   }
-  V dk[4];
-  // 8:16: the sweep re-reads the step history from shared memory (a compiler memory
-  // barrier here keeps the forward's values from being carried in registers, which
-  // spills at two CTAs per SM); 16:32 runs one CTA per SM and keeps them in registers.
-  if constexpr (kReloadHist<M>) asm volatile("" ::: "memory");
-  rx.backward(c, a.inv_tau, dk);
-  if (!active) return;
-  if (a.np.inv_lam != 1.0f) {  // lambda = 1: nothing to scale, the same bits
+  return active && q == 0 && flag;
+}
+
+// Runs `tile` for the CTA's full tiles and, on the last CTA, for the ragged tail straight
+// from global memory, queueing the groups it returns true for and handling them by `exact`.
+template <int M, class Shape, int NARR, class Exact, class Lane>
+__device__ __forceinline__ void slice_walk(const SliceArgs& a, const TileSrc<NARR>& src, size_t defer_at, const Exact& exact,
+                                           const Lane& lane_fn) {
+  constexpr int kTile = kTileOf<Shape>, P = Shape::kP;
+  DeferredGroups<kDeferCap<M, Shape>> dg;
+  dg.init(roi_slice_smem + defer_at);
+  // a batch's next tensor may start on the SMs this launch frees (no-op otherwise)
+  pdl_launch_dependents();
+  const bool ok = run_tiles<Shape::kThreads, kTile, Shape::kStages, NARR>(
+      roi_slice_smem, src, a.full_tiles, a.status, [&](const uint8_t* const* stage, int64_t tile, const auto& release) {
+        const int64_t e0 = tile * kTile + P * int64_t(threadIdx.x);
+        const uint8_t* at[NARR];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) dk[j] = vmul(dk[j], vconst<V>(a.np.inv_lam));
-  }
+        for (int i = 0; i < NARR; ++i) at[i] = stage[i] + size_t(P) * src.esize[i] * threadIdx.x;
+        dg.push(lane_fn(at, e0, true, release), e0);
+        dg.drain(false, exact);
+      });
+  if (ok) {
+    const int64_t t0 = a.full_tiles * kTile;
+    const int64_t lanes = blockIdx.x == gridDim.x - 1 ? (a.E - t0) / P : 0;
+    for (int64_t r = 0;; r += Shape::kThreads) {
+      if (r < lanes) {
+        const bool active = threadIdx.x + r < lanes;
+        const int64_t e0 = t0 + P * (active ? threadIdx.x + r : 0);
+        const uint8_t* at[NARR];
 #pragma unroll
-  for (int h = 0; h < L; ++h) {
-    if (!((flag >> h) & 1u)) {
-      const float g4[4] = {lane_of(dk[0], h), lane_of(dk[1], h), lane_of(dk[2], h), lane_of(dk[3], h)};
-      if (a.dphi != nullptr) *reinterpret_cast<float4*>(a.dphi + e0[h]) = make_float4(g4[0], g4[1], g4[2], g4[3]);
-      if (a.phi_out != nullptr) adamw4(a.phi_out, a.m, a.v, e0[h], *reinterpret_cast<const float4*>(p[h]), g4, a.opt);
+        for (int i = 0; i < NARR; ++i) at[i] = src.ptr[i] + size_t(e0) * src.esize[i];
+        dg.push(lane_fn(at, e0, active, [] {}), e0);
+      }
+      const bool done = r + Shape::kThreads >= lanes;
+      dg.drain(done, exact);
+      if (done) break;
     }
   }
+  // the launch completes only after the batch's previous one (stream order)
+  if (blockIdx.x == 0) pdl_wait();
 }
 
-// Hard words of one slot per lane (8 lanes fill a word).
-__device__ __forceinline__ void store_hard_slot(uint32_t* hard, int64_t e0, uint32_t bits, bool active) {
-  const int lane = threadIdx.x & 31;
-  uint32_t v = active ? bits << ((lane & 7) * 4) : 0u;
-  v |= __shfl_xor_sync(0xffffffffu, v, 1);
-  v |= __shfl_xor_sync(0xffffffffu, v, 2);
-  v |= __shfl_xor_sync(0xffffffffu, v, 4);
-  if (active && (lane & 7) == 0) hard[e0 >> 5] = v;
-}
-// The same for the two slots of a thread (first elements e0a, e0b; all lanes
-// active): both masks travel in one register, the first slot's in the low
-// half-word; after the shuffles within each 4-lane half, one exchange between
-// the halves completes the first slot's word on lane 0 of the 8 and the second
-// slot's word on lane 4.
-__device__ __forceinline__ void store_hard_slot_pair(uint32_t* hard, int64_t e0a, int64_t e0b, uint32_t bits_a,
-                                                     uint32_t bits_b) {
-  const int lane = threadIdx.x & 31;
-  const int sh = (lane & 3) * 4;
-  uint32_t v = (bits_a << sh) | (bits_b << (16 + sh));
-  v |= __shfl_xor_sync(0xffffffffu, v, 1);
-  v |= __shfl_xor_sync(0xffffffffu, v, 2);
-  const uint32_t o = __shfl_xor_sync(0xffffffffu, v, 4);
-  const bool upper = (lane & 4) != 0;
-  const uint32_t word = __byte_perm(v, o, upper ? 0x3276u : 0x5410u);
-  if ((lane & 3) == 0) hard[(upper ? e0b : e0a) >> 5] = word;
-}
-
-template <int N, int M, bool TAU1>
-__global__ void __launch_bounds__(kThreads, kMinBlocksFwd) roi_slice_fwd_kernel(SliceArgs a) {
-  extern __shared__ __align__(128) uint8_t smem[];
+template <int N, int M, bool TAU1, bool WIDE>
+__global__ void __launch_bounds__(FwdShape<M>::kThreads, 1) roi_slice_fwd_kernel(SliceArgs a) {
+  using C = FwdShape<M>;
   TileSrc<2> src;
   src.ptr[0] = reinterpret_cast<const uint8_t*>(a.phi);
   src.esize[0] = 4;
   src.ptr[1] = reinterpret_cast<const uint8_t*>(a.W);
   src.esize[1] = 2;
-  DeferredGroups<kDeferCap> dg;
-  dg.init(reinterpret_cast<int64_t*>(smem + kFwdDeferOffset));
-  const auto exact = [&](int64_t g0) { exact_group_fwd<N, M>(g0, a); };
-  // a batch's next tensor may start on the SMs this launch frees (no-op otherwise)
-  pdl_launch_dependents();
-  const bool ok = run_tiles<kThreads, kTile, kStagesFwd, 2>(
-      smem, src, a.full_tiles, a.status, [&](const uint8_t* const* stage, int64_t tile) {
-        const float* sphi = reinterpret_cast<const float*>(stage[0]);
-        const uint16_t* sW = reinterpret_cast<const uint16_t*>(stage[1]);
-        const int64_t base = tile * kTile;
-        const int s0 = threadIdx.x, s1 = threadIdx.x + kThreads;
-        const float* pp[2] = {sphi + 4 * s0, sphi + 4 * s1};
-        const uint16_t* pw[2] = {sW + 4 * s0, sW + 4 * s1};
-        const int64_t e0[2] = {base + 4 * s0, base + 4 * s1};
-        uint32_t bits[2], defer[2];
-        if constexpr (kPairedFwd<M>) {
-          uint32_t d2;
-          fwd_slots<N, M, TAU1, F2>(pp, pw, e0, true, a, bits, d2);
-          defer[0] = d2 & 1u, defer[1] = d2 >> 1;
-        } else {
-#pragma unroll 1
-          for (int j = 0; j < 2; ++j) {
-            uint32_t b1[1];
-            fwd_slots<N, M, TAU1, float>(pp + j, pw + j, e0 + j, true, a, b1, defer[j]);
-            bits[j] = b1[0];
-          }
-        }
-        if (a.hard != nullptr) store_hard_slot_pair(a.hard, e0[0], e0[1], bits[0], bits[1]);
-        dg.push(defer[0] != 0u, e0[0]);
-        dg.push(defer[1] != 0u, e0[1]);
-        dg.drain(false, exact);
-      });
-  if (ok && blockIdx.x == gridDim.x - 1) {
-    const int64_t t0 = a.full_tiles * kTile;
-    const int64_t slots = (a.E - t0) / 4;
-    for (int64_t r = 0; r * kThreads < slots; ++r) {
-      const int64_t si = threadIdx.x + r * kThreads;
-      const bool active = si < slots;
-      const int64_t off = t0 + 4 * (active ? si : 0);
-      const float* pp[1] = {a.phi + off};
-      const uint16_t* pw[1] = {a.W + off};
-      const int64_t e0[1] = {t0 + 4 * si};
-      uint32_t bits[1], defer;
-      fwd_slots<N, M, TAU1, float>(pp, pw, e0, active, a, bits, defer);
-      if (a.hard != nullptr) store_hard_slot(a.hard, e0[0], bits[0], active);
-      dg.push(defer != 0u, e0[0]);
-      dg.drain(false, exact);
-    }
-  }
-  if (ok) dg.drain(true, exact);
-  // the launch completes only after the batch's previous one (stream order)
-  if (blockIdx.x == 0) pdl_wait();
+  slice_walk<M, C>(a, src, kFwdDeferOffset<M>, [&](int64_t g0) { exact_group_fwd<N, M, WIDE>(g0, a); },
+                [&](const uint8_t* const* at, int64_t e0, bool active, const auto& release) {
+                  return fwd_lane<N, M, C::kP, TAU1, WIDE>(reinterpret_cast<const float*>(at[0]),
+                                                    reinterpret_cast<const uint16_t*>(at[1]), e0, active, a, release);
+                });
 }
 
-template <int N, int M, bool TAU1>
-__global__ void __launch_bounds__(kThreads, kMinBlocksBwd<M>) roi_slice_bwd_kernel(SliceArgs a) {
-  uint8_t* smem = roi_slice_smem;
+template <int N, int M, bool TAU1, bool WIDE>
+__global__ void __launch_bounds__(BwdShape<M>::kThreads, 1) roi_slice_bwd_kernel(SliceArgs a) {
+  using C = BwdShape<M>;
   TileSrc<3> src;
   src.ptr[0] = reinterpret_cast<const uint8_t*>(a.phi);
   src.esize[0] = 4;
@@ -773,97 +833,62 @@ __global__ void __launch_bounds__(kThreads, kMinBlocksBwd<M>) roi_slice_bwd_kern
   src.esize[1] = 2;
   src.ptr[2] = reinterpret_cast<const uint8_t*>(a.dWm);
   src.esize[2] = 2;
-  DeferredGroups<kDeferCap> dg;
-  dg.init(reinterpret_cast<int64_t*>(smem + kSliceDeferOffset<N, M>));
-  const auto exact = [&](int64_t g0) { exact_group_bwd<N, M>(g0, a); };
-  pdl_launch_dependents();
-  const bool ok = run_tiles<kThreads, kTile, kStagesBwd<M>, 3>(
-      smem, src, a.full_tiles, a.status, [&](const uint8_t* const* stage, int64_t tile) {
-        const float* sphi = reinterpret_cast<const float*>(stage[0]);
-        const uint16_t* sW = reinterpret_cast<const uint16_t*>(stage[1]);
-        const uint16_t* sdW = reinterpret_cast<const uint16_t*>(stage[2]);
-        const int64_t base = tile * kTile;
-        const int s0 = threadIdx.x, s1 = threadIdx.x + kThreads;
-        const float* pp[2] = {sphi + 4 * s0, sphi + 4 * s1};
-        const uint16_t* pw[2] = {sW + 4 * s0, sW + 4 * s1};
-        const uint16_t* pd[2] = {sdW + 4 * s0, sdW + 4 * s1};
-        const int64_t e0[2] = {base + 4 * s0, base + 4 * s1};
-        uint32_t defer[2];
-        if constexpr (kPairedBwd<M>) {
-          uint32_t d2;
-          bwd_slots<N, M, TAU1, F2>(pp, pw, pd, e0, true, a, d2);
-          defer[0] = d2 & 1u, defer[1] = d2 >> 1;
-        } else {
-#pragma unroll 1
-          for (int j = 0; j < 2; ++j)
-            bwd_slots<N, M, TAU1, float>(pp + j, pw + j, pd + j, e0 + j, true, a, defer[j]);
-        }
-        dg.push(defer[0] != 0u, e0[0]);
-        dg.push(defer[1] != 0u, e0[1]);
-        dg.drain(false, exact);
-      });
-  if (ok && blockIdx.x == gridDim.x - 1) {
-    const int64_t t0 = a.full_tiles * kTile;
-    const int64_t slots = (a.E - t0) / 4;
-    for (int64_t r = 0; r * kThreads < slots; ++r) {
-      const int64_t si = threadIdx.x + r * kThreads;
-      const bool active = si < slots;
-      const int64_t off = t0 + 4 * (active ? si : 0);
-      const float* pp[1] = {a.phi + off};
-      const uint16_t* pw[1] = {a.W + off};
-      const uint16_t* pd[1] = {a.dWm + off};
-      const int64_t e0[1] = {t0 + 4 * si};
-      uint32_t defer;
-      bwd_slots<N, M, TAU1, float>(pp, pw, pd, e0, active, a, defer);
-      dg.push(defer != 0u, e0[0]);
-      dg.drain(false, exact);
-    }
-  }
-  if (ok) dg.drain(true, exact);
-  if (blockIdx.x == 0) pdl_wait();
+  slice_walk<M, C>(a, src, kBwdDeferOffset<N, M>, [&](int64_t g0) { exact_group_bwd<N, M, WIDE>(g0, a); },
+                [&](const uint8_t* const* at, int64_t e0, bool active, const auto& release) {
+                  return bwd_lane<N, M, C::kP, TAU1, WIDE>(reinterpret_cast<const float*>(at[0]),
+                                                    reinterpret_cast<const uint16_t*>(at[1]),
+                                                    reinterpret_cast<const uint16_t*>(at[2]), e0, active, a, release);
+                });
 }
+
+// Whether a tau != 1 call takes the WIDE relaxation.
+bool slice_wide(const SliceArgs& a) { return a.tau < kSliceWideTau || a.tau < kSliceWideTauLambda * a.np.inv_lam; }
 
 struct LaunchCache {
   int per_sm[64] = {0};
 };
 
-template <class Kern>
-int launch_persistent(Kern kern, LaunchCache& cache, size_t smem, const SliceArgs& a, cudaStream_t stream,
-                      bool pdl) {
+template <class Shape, class Kern>
+int launch_persistent(Kern kern, LaunchCache& cache, size_t smem, SliceArgs a, cudaStream_t stream, bool pdl) {
+  a.full_tiles = a.E / kTileOf<Shape>;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
   if (cache.per_sm[dev] == 0) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
       return -1;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem) != cudaSuccess) return -1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, Shape::kThreads, smem) != cudaSuccess) return -1;
     cache.per_sm[dev] = per_sm < 1 ? 1 : per_sm;
   }
   const int64_t cap = int64_t(sm_count()) * cache.per_sm[dev];
   const int grid = int(a.full_tiles < 1 ? 1 : (a.full_tiles < cap ? a.full_tiles : cap));
-  return launch_maybe_pdl(kern, grid, kThreads, smem, stream, pdl, a);
+  return launch_maybe_pdl(kern, grid, Shape::kThreads, smem, stream, pdl, a);
 }
 
-template <int N, int M, bool TAU1>
+template <int N, int M, bool TAU1, bool WIDE>
 int slice_fwd(const SliceArgs& a, cudaStream_t stream, bool pdl) {
   static LaunchCache cache;
-  return launch_persistent(roi_slice_fwd_kernel<N, M, TAU1>, cache, kFwdDeferOffset + kDeferBytes, a, stream, pdl);
+  constexpr size_t smem = kFwdDeferOffset<M> + kDeferBytes<M, FwdShape<M>>;
+  static_assert(smem <= 232448, "shared memory per CTA");
+  return launch_persistent<FwdShape<M>>(roi_slice_fwd_kernel<N, M, TAU1, WIDE>, cache, smem, a, stream, pdl);
 }
-template <int N, int M, bool TAU1>
+template <int N, int M, bool TAU1, bool WIDE>
 int slice_bwd(const SliceArgs& a, cudaStream_t stream, bool pdl) {
   static LaunchCache cache;
-  constexpr size_t smem = kSliceDeferOffset<N, M> + kDeferBytes;
+  constexpr size_t smem = kBwdDeferOffset<N, M> + kDeferBytes<M, BwdShape<M>>;
   static_assert(smem <= 232448, "shared memory per CTA");
-  return launch_persistent(roi_slice_bwd_kernel<N, M, TAU1>, cache, smem, a, stream, pdl);
+  return launch_persistent<BwdShape<M>>(roi_slice_bwd_kernel<N, M, TAU1, WIDE>, cache, smem, a, stream, pdl);
 }
 
 template <int N, int M>
 int slice_fwd_nm(const SliceArgs& a, cudaStream_t stream, bool pdl) {
-  return a.tau == 1.0f ? slice_fwd<N, M, true>(a, stream, pdl) : slice_fwd<N, M, false>(a, stream, pdl);
+  if (a.tau == 1.0f) return slice_fwd<N, M, true, false>(a, stream, pdl);
+  return slice_wide(a) ? slice_fwd<N, M, false, true>(a, stream, pdl) : slice_fwd<N, M, false, false>(a, stream, pdl);
 }
 template <int N, int M>
 int slice_bwd_nm(const SliceArgs& a, cudaStream_t stream, bool pdl) {
-  return a.tau == 1.0f ? slice_bwd<N, M, true>(a, stream, pdl) : slice_bwd<N, M, false>(a, stream, pdl);
+  if (a.tau == 1.0f) return slice_bwd<N, M, true, false>(a, stream, pdl);
+  return slice_wide(a) ? slice_bwd<N, M, false, true>(a, stream, pdl) : slice_bwd<N, M, false, false>(a, stream, pdl);
 }
 
 }  // namespace
@@ -879,7 +904,6 @@ int launch_slice_fwd(const FwdCall& c, bool pdl) {
   a.hard = c.hard;
   a.st = c.st;
   a.E = c.E;
-  a.full_tiles = c.E / kTile;
   a.tau = c.tau;
   a.inv_tau = 1.0f / c.tau;
   a.np = c.np;
@@ -902,7 +926,6 @@ int launch_slice_bwd(const BwdCall& c, bool pdl) {
   a.v = c.v;
   a.opt = c.opt;
   a.E = c.E;
-  a.full_tiles = c.E / kTile;
   a.tau = c.tau;
   a.inv_tau = 1.0f / c.tau;
   a.np = c.np;

@@ -24,9 +24,11 @@ constexpr size_t tile_smem_bytes(uint32_t bytes_per_element) {
   return ((size_t(STAGES) * TILE * bytes_per_element + 7) & ~size_t(7)) + size_t(STAGES) * 16;
 }
 
-// Runs `compute(stage_ptrs, tile)` for every tile of this CTA among tiles
+// Runs `compute(stage_ptrs, tile, release)` for every tile of this CTA among tiles
 // 0 .. full_tiles - 1; `src_of(tile, a)` gives the global address of input array
-// a's part of the tile (TILE * esize[a] contiguous bytes, 16-byte aligned).
+// a's part of the tile (TILE * esize[a] contiguous bytes, 16-byte aligned).  Each warp
+// calls `release()` once per tile, all its lanes together, after its last read of the
+// stage: the last warp's call issues the copies that refill it.
 // Returns false if a wait timed out (status recorded, copies drained).
 template <int THREADS, int TILE, int STAGES, int NARR, class SrcOf, class Compute>
 __device__ __forceinline__ bool run_tiles_src(uint8_t* smem, const uint32_t (&esize)[NARR], int64_t full_tiles,
@@ -95,19 +97,20 @@ __device__ __forceinline__ bool run_tiles_src(uint8_t* smem, const uint32_t (&es
     const uint8_t* stage[NARR];
 #pragma unroll
     for (int a = 0; a < NARR; ++a) stage[a] = smem + arr_off[a] + size_t(s) * TILE * esize[a];
-    compute(stage, tile);
-    __syncwarp();
-    if (lane == 0) {
-      __threadfence_block();
-      if (atomicAdd(&done[s], 1u) == kWarps - 1) {
-        // every warp is done reading this fill: refill it with the tile STAGES ahead
-        done[s] = 0;
-        if (i + STAGES < my_tiles) {
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          issue(s, tile + STAGES * stride);
+    compute(stage, tile, [&]() {
+      __syncwarp();
+      if (lane == 0) {
+        __threadfence_block();
+        if (atomicAdd(&done[s], 1u) == kWarps - 1) {
+          // every warp is done reading this fill: refill it with the tile STAGES ahead
+          done[s] = 0;
+          if (i + STAGES < my_tiles) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            issue(s, tile + STAGES * stride);
+          }
         }
       }
-    }
+    });
     if (++s == STAGES) {
       s = 0;
       parity ^= 1u;
@@ -116,7 +119,7 @@ __device__ __forceinline__ bool run_tiles_src(uint8_t* smem, const uint32_t (&es
   return true;
 }
 
-// One tensor per input array: tile t of array a starts at ptr[a] + t * TILE * esize[a].
+// As run_tiles_src with one tensor per input array: tile t of array a starts at ptr[a] + t * TILE * esize[a].
 template <int THREADS, int TILE, int STAGES, int NARR, class Compute>
 __device__ __forceinline__ bool run_tiles(uint8_t* smem, const TileSrc<NARR>& src, int64_t full_tiles,
                                           unsigned int* status, Compute&& compute) {

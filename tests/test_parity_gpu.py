@@ -312,6 +312,18 @@ def test_schedule_temperatures(roi, N, M, tau, lam):
     check_against_oracle(got, ph, Wb, dWb, N, M, tau, 123456789, 5, 2, lam, 0)
 
 
+# The warp-slice kernels' rule (tau = 0.1, tau lambda = 0.05); 41 rows are full tiles of
+# neither direction's shape and a ragged tail, 64 rows full tiles and a tail.
+@pytest.mark.parametrize("rows", [1, 41, 64])
+@pytest.mark.parametrize("N,M", [(8, 16), (16, 32)])
+@pytest.mark.parametrize("tau,lam", [(0.6, 0.07), (0.35, 0.141), (0.35, 0.145), (1.5, 0.02), (1.5, 0.2)])
+def test_slice_schedule_temperatures(roi, rows, N, M, tau, lam):
+    W, phi, dWm, ph, Wb, dWb = make(rows, 608, "normal", data_seed=M + N)
+    st = roi.NoiseState(123456789, 5, 2, lam, 0)
+    got = gpu_run(roi, phi, W, dWm, N, M, tau, st)
+    check_against_oracle(got, ph, Wb, dWb, N, M, tau, 123456789, 5, 2, lam, 0)
+
+
 @pytest.mark.parametrize("rows,cols", [(4, 64), (8, 2112)])
 def test_non_finite_logits_propagate(roi, rows, cols):
     """NaN / +inf logits make their group's outputs NaN (for N = 1 a +inf member
