@@ -637,42 +637,6 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
   if (blockIdx.x == 0) pdl_wait();
 }
 
-__global__ void __launch_bounds__(128) roi_bwd_generic_kernel(BwdArgs a, BwdOptArgs o, int N, int M) {
-  const int64_t groups = a.E / M;
-  for (int64_t g = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; g < groups;
-       g += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t e0 = g * M;
-    float kap[32], S[32], c[32], dk[32];
-    for (int l = 0; l < M; ++l) {
-      const uint32_t x = noise_word(a.np, a.np.e_base + uint64_t(e0 + l));
-      kap[l] = fmaf(a.phi[e0 + l], a.np.inv_lam, gumbel_from_word(x));
-      c[l] = bf16_bits_to_float(a.dWm[e0 + l]) * bf16_bits_to_float(a.W[e0 + l]);
-    }
-    ExactGroup<31, 32> ex;
-    ex.forward(kap, N, M, a.tau, S);
-    ex.backward(c, N, M, a.tau, dk);
-    for (int l = 0; l < M; ++l) {
-      const int64_t e = e0 + l;
-      const float g = dk[l] * a.np.inv_lam;
-      if (a.dphi != nullptr) a.dphi[e] = g;
-      if (o.phi_out != nullptr) {
-        float ph = a.phi[e], mm = o.m[e], vv = o.v[e];
-        adamw_elem(ph, g, mm, vv, o.opt);
-        o.phi_out[e] = ph;
-        o.m[e] = mm;
-        o.v[e] = vv;
-      }
-      if (a.dW != nullptr) {
-        if (a.hard_in != nullptr) {
-          a.dW[e] = ((a.hard_in[e >> 5] >> (e & 31)) & 1u) ? a.dWm[e] : uint16_t(0);
-        } else {
-          a.dW[e] = __bfloat16_as_ushort(__float2bfloat16_rn(bf16_bits_to_float(a.dWm[e]) * S[l]));
-        }
-      }
-    }
-  }
-}
-
 struct LaunchCache {
   int per_sm[64] = {0};
 };
@@ -838,13 +802,7 @@ int launch_bwd_impl(const BwdCall& c, bool pdl) {
   if (c.N == 4 && c.M == 8) return launch_nm<4, 8>(a, o, c.stream, pdl);
   if (c.N == 2 && c.M == 8) return launch_nm<2, 8>(a, o, c.stream, pdl);
   if (slice_supported(c.N, c.M)) return launch_slice_bwd(c, pdl);
-  const int64_t groups = c.E / c.M;
-  int64_t blocks = (groups + 127) / 128;
-  const int64_t cap = int64_t(sm_count()) * 16;
-  if (blocks > cap) blocks = cap;
-  if (blocks < 1) blocks = 1;
-  roi_bwd_generic_kernel<<<int(blocks), 128, 0, c.stream>>>(a, o, c.N, c.M);
-  return cudaGetLastError() == cudaSuccess ? 1 : -1;
+  return launch_any_bwd(c);
 }
 }  // namespace
 

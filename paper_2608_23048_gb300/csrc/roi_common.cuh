@@ -883,7 +883,7 @@ __device__ __forceinline__ V min_of(const V (&x)[M]) {
 // of min(largest, largest) and the two seconds.
 template <int M, class V>
 __device__ __forceinline__ V second_of(const V (&x)[M]) {
-  static_assert(M == 4 || M == 8, "second of 4 or 8");
+  static_assert(M >= 4 && (M & (M - 1)) == 0, "second of 4, 8, 16, 32");
   V h[M / 2], s[M / 2];
 #pragma unroll
   for (int i = 0; i < M / 2; ++i) {

@@ -496,37 +496,6 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
   if (blockIdx.x == 0) pdl_wait();
 }
 
-// Any 1 <= N < M <= 32: one thread per group, exact log-space routine, direct
-// loads; hard words are zeroed beforehand and assembled with atomicOr.
-__global__ void __launch_bounds__(128) roi_fwd_generic_kernel(FwdArgs a, int N, int M) {
-  const int64_t groups = a.E / M;
-  for (int64_t g = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; g < groups;
-       g += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t e0 = g * M;
-    float kap[32], S[32];
-    for (int l = 0; l < M; ++l) {
-      const uint32_t x = noise_word(a.np, a.np.e_base + uint64_t(e0 + l));
-      kap[l] = fmaf(a.phi[e0 + l], a.np.inv_lam, gumbel_from_word(x));
-    }
-    ExactGroup<31, 32> ex;
-    ex.forward(kap, N, M, a.tau, S);
-    const uint32_t bits = (a.hard != nullptr || a.st) ? topn_bits_dyn(kap, N, M) : 0u;
-    for (int l = 0; l < M; ++l) {
-      const float w = bf16_bits_to_float(a.W[e0 + l]);
-      a.Wm[e0 + l] = a.st ? (((bits >> l) & 1u) ? a.W[e0 + l] : uint16_t(0))
-                          : __bfloat16_as_ushort(__float2bfloat16_rn(w * S[l]));
-      if (a.soft != nullptr) a.soft[e0 + l] = S[l];
-    }
-    if (a.hard != nullptr) {
-      for (int l = 0; l < M; ++l)
-        if ((bits >> l) & 1u) {
-          const int64_t e = e0 + l;
-          atomicOr(&a.hard[e >> 5], 1u << (e & 31));
-        }
-    }
-  }
-}
-
 struct LaunchCache {
   int per_sm[64] = {0};
 };
@@ -650,19 +619,7 @@ int launch_fwd_impl(const FwdCall& c, bool pdl) {
   if (c.N == 4 && c.M == 8) return launch_nm<4, 8>(a, c.stream, pdl);
   if (c.N == 2 && c.M == 8) return launch_nm<2, 8>(a, c.stream, pdl);
   if (slice_supported(c.N, c.M)) return launch_slice_fwd(c, pdl);
-  // generic path
-  int launched = 0;
-  if (c.hard != nullptr) {
-    if (cudaMemsetAsync(c.hard, 0, size_t((c.E + 31) / 32) * 4, c.stream) != cudaSuccess) return -1;
-  }
-  const int64_t groups = c.E / c.M;
-  int64_t blocks = (groups + 127) / 128;
-  const int64_t cap = int64_t(sm_count()) * 16;
-  if (blocks > cap) blocks = cap;
-  if (blocks < 1) blocks = 1;
-  roi_fwd_generic_kernel<<<int(blocks), 128, 0, c.stream>>>(a, c.N, c.M);
-  launched += 1;
-  return cudaGetLastError() == cudaSuccess ? launched : -1;
+  return launch_any_fwd(c);
 }
 }  // namespace
 

@@ -312,6 +312,20 @@ def test_schedule_temperatures(roi, N, M, tau, lam):
     check_against_oracle(got, ph, Wb, dWb, N, M, tau, 123456789, 5, 2, lam, 0)
 
 
+# Patterns without a kernel of their own: every padded width, M that divides a hard word
+# (assembled by shuffles) and M that does not, group counts that leave a lane of the last
+# pair empty, N = 1, the largest N, small tau lambda.
+@pytest.mark.parametrize("rows,groups", [(1, 1), (3, 43), (13, 101)])
+@pytest.mark.parametrize("N,M,tau,lam", [(1, 2, 0.7, 1.0), (2, 3, 0.5, 0.1), (1, 4, 0.2236, 0.0447), (3, 4, 1.0, 1.0),
+                                         (4, 5, 0.8, 1.0), (1, 8, 0.3, 0.2), (7, 8, 0.9, 0.5), (5, 12, 0.7, 1.0),
+                                         (4, 16, 0.6, 0.5), (15, 16, 1.0, 1.0), (7, 24, 1.5, 1.0), (8, 32, 0.8, 0.7)])
+def test_patterns_without_own_kernel(roi, rows, groups, N, M, tau, lam):
+    W, phi, dWm, ph, Wb, dWb = make(rows, groups * M, "normal", data_seed=M + N)
+    st = roi.NoiseState(123456789, 5, 2, lam, 3)
+    got = gpu_run(roi, phi, W, dWm, N, M, tau, st)
+    check_against_oracle(got, ph, Wb, dWb, N, M, tau, 123456789, 5, 2, lam, 3)
+
+
 # The warp-slice kernels' rule (tau = 0.1, tau lambda = 0.05); 41 rows are full tiles of
 # neither direction's shape and a ragged tail, 64 rows full tiles and a tail.
 @pytest.mark.parametrize("rows", [1, 41, 64])
