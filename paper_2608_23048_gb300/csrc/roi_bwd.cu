@@ -22,6 +22,11 @@ struct Cfg {
   static constexpr int kStages = M == 4 ? 3 : 2;  // 192 KB (M = 4), 96 KB + 72 KB step history (M = 8)
   static constexpr int kMinBlocks = 1;
   static constexpr int kTile = 2 * kPairs * kThreads * M;  // elements
+  // rounds of one pair a thread up to which a lone tensor takes no tiles (tile_grid): 2:4
+  // 0.5 M elements 3.1 against 4.6 us, 2.5 M 8.6 against 9.5, 3.5 M 10.0 against 9.9.  A
+  // tile at M = 8 is one pair a thread as it is.
+  static constexpr int kTailRounds = M == 4 ? 5 : 0;
+  static constexpr int kTailChunk = M == 4 ? 2 * kThreads : kThreads;  // groups of a CTA's round
   // Groups out of the fast path's range: queued per warp (DeferredGroups) at M = 4, where
   // it measured 2.7 % faster at tau = 1 on the 7B-shaped set, in place at M = 8 (at
   // tau = 0.5 the queue's code measured 3 % slower).  The queue holds at most 64 kPairs a
@@ -207,7 +212,7 @@ __device__ __forceinline__ void bwd_inputs(const float* const* phi_g, const uint
 template <int N, int M, bool TAU1, class V, bool HIST, bool ST, bool OPT, bool NARROW, bool DEFER, bool WIDE>
 __device__ __forceinline__ uint32_t bwd_groups(const float* const* phi_g, const uint16_t* const* W_g,
                                            const uint16_t* const* dWm_g, const int64_t* e0, const uint32_t* q0,
-                                           const BwdArgs& a, const BwdOptArgs& o, V* hist = nullptr) {
+                                           const BwdArgs& a, const BwdOptArgs& o, V* hist = nullptr, int have = 2) {
   constexpr int L = vlanes<V>();
   // straight-through: the forward's hard bits of these groups, loaded now so the
   // load's latency hides behind the relaxation.  With HIST (registers tight) dW,
@@ -354,6 +359,7 @@ __device__ __forceinline__ uint32_t bwd_groups(const float* const* phi_g, const 
         }
       }
     }
+    if (OPT && h >= have) continue;  // the tail's missing second group (its other outputs are written twice)
     if constexpr (OPT) {
       // fused AdamW step on these logits (their old values are still in phi_g)
 #pragma unroll
@@ -462,19 +468,38 @@ __device__ __forceinline__ void bwd_tile(const uint8_t* const* stage, int64_t ti
   if constexpr (C::kDefer) dg.drain(false, exact);
 }
 
-// The ragged tail of a tensor (fewer than one tile after its full tiles), by one
-// CTA, straight from global memory.
+// The groups of a tensor after its full tiles, straight from global memory: chunks chunk0,
+// chunk0 + step, ... of kTailChunk groups.  M = 4: a pair per thread in the tiles' packed
+// code, so that a whole small tensor may go this way.  M = 8: one group per thread, all in
+// registers.
 template <int N, int M, bool TAU1, bool ST, bool OPT, bool WIDE>
-__device__ __forceinline__ void bwd_tail(const BwdArgs& a, const BwdOptArgs& o) {
+__device__ __forceinline__ void bwd_tail(const BwdArgs& a, const BwdOptArgs& o, int64_t chunk0, int64_t step) {
   using C = Cfg<M>;
   const int64_t t0 = a.full_tiles * C::kTile;
   const int64_t tail_groups = (a.E - t0) / M;
-  for (int64_t gi = threadIdx.x; gi < tail_groups; gi += C::kThreads) {
-    const float* pp[1] = {a.phi + t0 + gi * M};
-    const uint16_t* pw[1] = {a.W + t0 + gi * M};
-    const uint16_t* pd[1] = {a.dWm + t0 + gi * M};
-    const int64_t e0[1] = {t0 + gi * M};
-    bwd_groups<N, M, TAU1, float, false, ST, OPT, false, false, WIDE>(pp, pw, pd, e0, nullptr, a, o);
+  for (int64_t g0 = chunk0 * C::kTailChunk; g0 < tail_groups; g0 += step * C::kTailChunk) {
+    if constexpr (M == 4) {
+      // the chunk's halves go to the two lanes; a missing second group doubles the first
+      const int64_t n = tail_groups - g0 < C::kTailChunk ? tail_groups - g0 : C::kTailChunk;
+      const int half = tail_half<M>(n);
+      if (threadIdx.x >= half) continue;
+      const bool two = threadIdx.x + half < n;
+      const int64_t ea = t0 + (g0 + threadIdx.x) * M;
+      const int64_t eb = two ? ea + int64_t(half) * M : ea;
+      const float* pp[2] = {a.phi + ea, a.phi + eb};
+      const uint16_t* pw[2] = {a.W + ea, a.W + eb};
+      const uint16_t* pd[2] = {a.dWm + ea, a.dWm + eb};
+      const int64_t e0[2] = {ea, eb};
+      bwd_groups<N, M, TAU1, F2, false, ST, OPT, false, false, WIDE>(pp, pw, pd, e0, nullptr, a, o, nullptr, two ? 2 : 1);
+    } else {
+      if (g0 + threadIdx.x >= tail_groups) continue;
+      const int64_t e = t0 + (g0 + threadIdx.x) * M;
+      const float* pp[1] = {a.phi + e};
+      const uint16_t* pw[1] = {a.W + e};
+      const uint16_t* pd[1] = {a.dWm + e};
+      const int64_t e0[1] = {e};
+      bwd_groups<N, M, TAU1, float, false, ST, OPT, false, false, WIDE>(pp, pw, pd, e0, nullptr, a, o);
+    }
   }
 }
 
@@ -509,7 +534,7 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks) roi_bwd_
   if constexpr (C::kDefer) {
     if (ok) dg.drain(true, exact);
   }
-  if (ok && blockIdx.x == gridDim.x - 1) bwd_tail<N, M, TAU1, ST, OPT, WIDE>(a, o);
+  if (ok) bwd_tail<N, M, TAU1, ST, OPT, WIDE>(a, o, tail_rank(a.full_tiles), gridDim.x);
   // the launch completes only after the batch's previous one (stream order)
   if (blockIdx.x == 0) pdl_wait();
 }
@@ -528,11 +553,12 @@ struct BwdItem {
   float* v;
   int64_t E;
   int64_t tile0;
+  int64_t tail0;  // first chunk of kTailChunk groups in the concatenation of the ragged tails
   NoiseParams np;
 };
 struct BwdMulti {
   int count;
-  int64_t total_tiles;
+  int64_t total_tiles, total_tails;
   float tau, inv_tau;
   unsigned int* status;
   AdamW opt;
@@ -629,9 +655,9 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
     if (ok) dg.drain(true, exact);
   }
   if (ok) {
-    for (int i = blockIdx.x; i < mm.count; i += gridDim.x) {
-      const BwdArgs ai = multi_args<M>(mm, i);
-      if (ai.full_tiles * C::kTile < ai.E) bwd_tail<N, M, TAU1, ST, OPT, WIDE>(ai, multi_opt(mm, i));
+    for (int64_t c = tail_rank(mm.total_tiles); c < mm.total_tails; c += gridDim.x) {
+      const int i = tail_item(mm, c);
+      bwd_tail<N, M, TAU1, ST, OPT, WIDE>(multi_args<M>(mm, i), multi_opt(mm, i), c - mm.it[i].tail0, mm.total_tails);
     }
   }
   if (blockIdx.x == 0) pdl_wait();
@@ -658,8 +684,9 @@ int launch_tiles(const BwdArgs& a, const BwdOptArgs& o, cudaStream_t stream, boo
     cache.per_sm[dev] = per_sm < 1 ? 1 : per_sm;
   }
   const int64_t cap = int64_t(sm_count()) * cache.per_sm[dev];
-  const int grid = int(a.full_tiles < 1 ? 1 : (a.full_tiles < cap ? a.full_tiles : cap));
-  return launch_maybe_pdl(kern, grid, C::kThreads, smem, stream, pdl, a, o);
+  BwdArgs b = a;
+  const int grid = tile_grid(b.full_tiles, a.E, M, C::kTailChunk, C::kTile, cap, pdl ? 0 : C::kTailRounds);
+  return launch_maybe_pdl(kern, grid, C::kThreads, smem, stream, pdl, b, o);
 }
 
 template <int N, int M, bool ST, bool OPT, bool NARROW_ONLY = false>
@@ -706,7 +733,7 @@ int launch_multi_kern(const BwdMulti& mm, cudaStream_t stream, bool pdl) {
     cache.per_sm[dev] = per_sm < 1 ? 1 : per_sm;
   }
   const int64_t cap = int64_t(sm_count()) * cache.per_sm[dev];
-  const int64_t want = mm.total_tiles > mm.count ? mm.total_tiles : mm.count;
+  const int64_t want = mm.total_tiles + mm.total_tails;
   const int grid = int(want < 1 ? 1 : (want < cap ? want : cap));
   return launch_maybe_pdl(kern, grid, C::kThreads, smem, stream, pdl, mm);
 }
@@ -736,7 +763,7 @@ int launch_multi(const BwdCall* calls, int count, bool pdl) {
   mm.inv_tau = 1.0f / calls[0].tau;
   mm.status = calls[0].status;
   mm.opt = calls[0].opt;
-  int64_t tiles = 0;
+  int64_t tiles = 0, tails = 0;
   for (int i = 0; i < count; ++i) {
     const BwdCall& c = calls[i];
     BwdItem& x = mm.it[i];
@@ -754,8 +781,11 @@ int launch_multi(const BwdCall* calls, int count, bool pdl) {
     x.np = c.np;
     x.np.narrow = counters_narrow(c.np, c.E);
     tiles += c.E / C::kTile;
+    x.tail0 = tails;
+    tails += (c.E % C::kTile / M + C::kTailChunk - 1) / C::kTailChunk;
   }
   mm.total_tiles = tiles;
+  mm.total_tails = tails;
   const cudaStream_t stream = calls[0].stream;
   const int kind = bwd_kind(calls[0]);
   const bool narrow = mm.it[0].np.narrow;

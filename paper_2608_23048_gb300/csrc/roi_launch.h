@@ -76,6 +76,7 @@ struct ExportCall {
   uint16_t* Wp;       // nullable
   int64_t E;
   int N, M;
+  unsigned int* status;
   cudaStream_t stream;
 };
 
@@ -85,6 +86,7 @@ struct CompressCall {
   uint16_t* values;  // [E / 2]
   uint32_t* meta;    // [E / 32]
   int64_t E;         // multiple of 32
+  unsigned int* status;
   cudaStream_t stream;
 };
 
@@ -154,6 +156,19 @@ int launch_maybe_pdl(void (*kern)(KArgs...), int grid, int threads, size_t smem,
 
 // Streaming multiprocessors of the current device (cached).
 int sm_count();
+
+// Grid of a tile kernel over one tensor of E elements (`tiles` full tiles, at most `cap`
+// CTAs).  `rounds`: a tensor that takes at most so many rounds of one pair of groups a
+// thread over the whole GPU is processed that way, as one ragged tail (tiles = 0): the few
+// CTAs that its tiles would occupy, each with a ring to fill, take longer (2:4 at tau = 1,
+// forward / backward of 32768 elements 5.3 / 4.5 -> 3.1 / 3.1 us, 896 x 896 5.4 / 4.6 ->
+// 4.7 / 4.5).  Launches that are chained behind others (rounds = 0) keep the tiles.
+inline int tile_grid(int64_t& tiles, int64_t E, int M, int chunk, int64_t tile, int64_t cap, int rounds) {
+  if ((E / M + chunk - 1) / chunk <= rounds * cap) tiles = 0;
+  const int64_t chunks = ((E - tiles * tile) / M + chunk - 1) / chunk;
+  const int64_t want = tiles + chunks;
+  return int(want < 1 ? 1 : (want < cap ? want : cap));
+}
 
 // Batched calls: a run of consecutive items with the same tile kernel, each of
 // them small (fewer than kMultiTilesPerSm full tiles per SM), goes to one

@@ -119,6 +119,34 @@ __device__ __forceinline__ bool run_tiles_src(uint8_t* smem, const uint32_t (&es
   return true;
 }
 
+// The order in which this CTA takes up work after `tiles` tiles were dealt out round robin:
+// first those that had one tile less.
+__device__ __forceinline__ int64_t tail_rank(int64_t tiles) {
+  const uint32_t r = uint32_t(tiles % gridDim.x);
+  return blockIdx.x >= r ? blockIdx.x - r : blockIdx.x + gridDim.x - r;
+}
+// How a chunk of n groups is split between the two lanes of the packed code: the first
+// `half` threads take groups t and t + half (whole hard-mask words in either half).
+template <int M>
+__device__ __forceinline__ int tail_half(int64_t n) {
+  constexpr int kPerWord = 32 / M;
+  return int((n + 2 * kPerWord - 1) / (2 * kPerWord)) * kPerWord;
+}
+// The item of a multi-tensor launch that holds chunk c of the concatenated ragged tails.
+template <class Multi>
+__device__ __forceinline__ int tail_item(const Multi& mm, int64_t c) {
+  int lo = 0, hi = mm.count - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (mm.it[mid].tail0 <= c) {
+      lo = mid;
+    } else {
+      hi = mid - 1;
+    }
+  }
+  return lo;
+}
+
 // As run_tiles_src with one tensor per input array: tile t of array a starts at ptr[a] + t * TILE * esize[a].
 template <int THREADS, int TILE, int STAGES, int NARR, class Compute>
 __device__ __forceinline__ bool run_tiles(uint8_t* smem, const TileSrc<NARR>& src, int64_t full_tiles,

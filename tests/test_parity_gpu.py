@@ -312,6 +312,25 @@ def test_schedule_temperatures(roi, N, M, tau, lam):
     check_against_oracle(got, ph, Wb, dWb, N, M, tau, 123456789, 5, 2, lam, 0)
 
 
+# The sizes around which a lone 2:4 tensor goes from one pair of groups a thread to tiles,
+# and whole rounds of that form (2 x 512 threads x SMs), with a remainder and an odd group
+# count: a row-sliced pair of calls, each below the rule, equals the whole above it.
+@pytest.mark.parametrize("N,M,tau", [(2, 4, 1.0), (2, 4, 0.3)])
+@pytest.mark.parametrize("rows", [1, 77, 610, 1217, 3101])
+def test_small_tensors_equal_slices(roi, N, M, tau, rows):
+    W, phi, dWm, *_ = make(rows, 1036, "normal", data_seed=6)
+    cut = rows // 3 * 2 // 8 * 8  # rows of the first slice: its last hard word is full
+    whole = gpu_run(roi, phi, W, dWm, N, M, tau, roi.NoiseState(9, 1, 4, 1.0, 0))
+    parts = [gpu_run(roi, phi[a:b].contiguous(), W[a:b].contiguous(), dWm[a:b].contiguous(), N, M, tau,
+                     roi.NoiseState(9, 1, 4, 1.0, a)) for a, b in ((0, cut), (cut, rows)) if a < b]
+    for key in whole:
+        assert np.array_equal(whole[key].ravel(), np.concatenate([p[key].ravel() for p in parts])), key
+    r0 = slice(max(0, rows - 2), rows)
+    got = {k: v[r0] for k, v in whole.items() if k != "hard_bits"}
+    check_against_oracle(got, phi[r0].numpy(), WL.bf16_bits(W[r0]), WL.bf16_bits(dWm[r0]), N, M, tau, 9, 1, 4, 1.0,
+                         max(0, rows - 2))
+
+
 # Patterns without a kernel of their own: every padded width, M that divides a hard word
 # (assembled by shuffles) and M that does not, group counts that leave a lane of the last
 # pair empty, N = 1, the largest N, small tau lambda.
