@@ -543,6 +543,8 @@ roi_status roi_export_compressed_2of4(const float* logits, const roi_bf16* W, in
   c.values = out_values;
   c.meta = out_meta;
   c.E = E;
+  c.status = status_word();
+  if (c.status == nullptr) return ROI_ERR_CUDA;
   c.stream = static_cast<cudaStream_t>(stream);
   return finish(launch_export_compressed_2of4(c));
 }
@@ -568,6 +570,8 @@ roi_status roi_hard_mask_export(const float* logits, int N, int M, int64_t rows,
   c.E = E;
   c.N = N;
   c.M = M;
+  c.status = status_word();
+  if (c.status == nullptr) return ROI_ERR_CUDA;
   c.stream = static_cast<cudaStream_t>(stream);
   return finish(launch_export(c));
 }
