@@ -305,10 +305,11 @@ __device__ __forceinline__ uint32_t bwd_groups(const float* const* phi_g, const 
   }
   if constexpr (HIST) bwd_upstream<M, V>(W_g, dWm_g, c);
   fg.backward(c, a.inv_tau, dkv);
-  // dL/dphi = dL/dkappa / lambda (lambda = 1: nothing to scale, the same bits)
-  if (a.np.inv_lam != 1.0f) {
+  // dL/dphi = dL/dkappa / lambda (at tau = 1, lambda = 1 nothing to scale, the same bits)
+  if (!TAU1 || a.np.inv_lam != 1.0f) {
+    const V scale = vconst<V>(TAU1 ? a.np.inv_lam : __fmul_rn(a.inv_tau, a.np.inv_lam));
 #pragma unroll
-    for (int l = 0; l < M; ++l) dkv[l] = vmul(dkv[l], vconst<V>(a.np.inv_lam));
+    for (int l = 0; l < M; ++l) dkv[l] = vmul(dkv[l], scale);
   }
   if constexpr (kStageMoments) cp_async_wait_all();
 #pragma unroll

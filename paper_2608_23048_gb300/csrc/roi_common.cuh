@@ -32,6 +32,8 @@ constexpr float kTinyExcl = 7.888609052210118e-31f;  // 2^-100
 // second maximum costs what the range checks it replaces did; at N = 4 it is formed three
 // times, and wide_range() in roi_launch.h decides.
 constexpr float kLeadCap = 100.0f;
+// Range of the plain tau != 1 relaxations (see FastGroup's forward).
+constexpr float kLeastRange = -98.0f;
 template <int N>
 constexpr bool kAlwaysWide = N <= 2;
 
@@ -311,7 +313,8 @@ __device__ __forceinline__ void topn_bits4_signs(const F2 (&k)[4], int N, uint32
       w2 = s02 | s12 | ~s23;
       w3 = s03 | s13 | s23;
     }
-    bits[h] = (w0 >> 31) | ((w1 >> 31) << 1) | ((w2 >> 31) << 2) | ((w3 >> 31) << 3);
+    // the four sign bits, one funnel shift each
+    bits[h] = __funnelshift_l(w0, __funnelshift_l(w1, __funnelshift_l(w2, w3 >> 31, 1), 1), 1);
   }
 }
 
@@ -373,13 +376,11 @@ __device__ __forceinline__ void topn_bits8_threshold(const F2 (&k)[8], uint32_t 
   }
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    // the sign bytes of members 0-3 and 4-7 into two words; their four top bits
-    // (7, 15, 23, 31) land in bits 28-31 of the product with 2^21 + 2^14 + 2^7 + 1
-    const uint32_t a = __byte_perm(__byte_perm(sg[h][0], sg[h][1], 0x0073u), __byte_perm(sg[h][2], sg[h][3], 0x0073u), 0x5410u);
-    const uint32_t b = __byte_perm(__byte_perm(sg[h][4], sg[h][5], 0x0073u), __byte_perm(sg[h][6], sg[h][7], 0x0073u), 0x5410u);
-    const uint32_t pa = ((~a & 0x80808080u) * 0x00204081u) >> 28;
-    const uint32_t pb = ((~b & 0x80808080u) * 0x00204081u) >> 28;
-    const uint32_t v = pa | (pb << 4);
+    // the members' sign bits (set: below the threshold), one funnel shift each
+    uint32_t below = sg[h][7] >> 31;
+#pragma unroll
+    for (int l = 6; l >= 0; --l) below = __funnelshift_l(sg[h][l], below, 1);
+    const uint32_t v = below ^ 0xffu;
     bits[h] = __popc(v) == N ? v : 0xffffffffu;
   }
 }
@@ -1066,21 +1067,28 @@ struct FastGroup {
       }
     } else {
       const V kmax = max_of(kap);
-      const V sc = vconst<V>(inv_tau);
       const V itau = vconst<V>(inv_tau);
-      V d[M];
+      const V tau1 = vconst<V>(fmaxf(1.0f, rcp_approx(inv_tau)));
+      V d[M], lz_prev;
 #pragma unroll
-      for (int l = 0; l < M; ++l) d[l] = vmul(vsub(kap[l], kmax), sc);
+      for (int l = 0; l < M; ++l) d[l] = vmul(vsub(kap[l], kmax), itau);
       const V ksum = sum_of(kap);
       flag = vbelow(vsub(ksum, ksum), 0.0f);  // a non-finite key (or a sum beyond the float range)
-      V tmin = vconst<V>(1.0f);
 #pragma unroll
       for (int k = 0; k < N; ++k) {
         V e[M];
 #pragma unroll
         for (int l = 0; l < M; ++l) e[l] = vmap(d[l], ex2_approx);
         const V tot = sum_of(e);
-        if (M >= 8 && k > 0) tmin = vmin(tmin, tot);
+        // Range check, from the totals alone: a leader's complement eps (its share of the
+        // total) leaves a next total of at most eps + eps^(1 / tau), so eps times the total,
+        // the sum that was formed, is at least 2^-99 while
+        // log2 total + max(1, tau) log2 (next total) >= -98, and members that were flushed
+        // to zero are below the sum's last bit.  Other groups go to the exact routine.  (The
+        // smallest exclusive sum of every step was compared before: 3 % more instructions.)
+        const V lz = vmap(tot, lg2_approx);
+        if (k > 0) flag |= vbelow(vfma(lz, tau1, lz_prev), kLeastRange);
+        lz_prev = lz;
         const V r = vmap(tot, rcp_approx);
         if (!KEEP && k > 0 && k + 1 == N) {
           // last step without KEEP: added into S as it is formed (one fma)
@@ -1095,34 +1103,19 @@ struct FastGroup {
           }
         }
         if (k + 1 < N) {
-          // d_l += log2(1 - mu_l) / tau.  A group whose exclusive sums fall below 2^-100
-          // of the total goes to the exact routine.  M = 8: the offsets are first
-          // renormalised by log2 of the total (so sum 2^d = 1 and every offset <= 0)
-          // instead of by their maximum after the update (seven comparisons per step;
-          // 1.5B-shaped 4:8 at tau = 0.5 2 % faster, the 2:4 step 1 % slower), and a
-          // total below 2^-120 (offsets that fell too far in one step) is flagged too.
+          // offset - log2(total) + log2(1 - mu) / tau: normalised, so that the weights of
+          // the next step start from mu
           V ex[M];
           exclusive_sums(e, ex);
-          if constexpr (M >= 8) {
-            flag |= vbelow(vmul(min_of(ex), r), kTinyExcl);
-            const V lz = vmap(tot, lg2_approx);
 #pragma unroll
-            for (int l = 0; l < M; ++l) d[l] = vfma(vmap(vmul(ex[l], r), lg2_approx), itau, vsub(d[l], lz));
-          } else {
-            flag |= vbelow(min_of(ex), kTinyExcl);
-#pragma unroll
-            for (int l = 0; l < M; ++l) d[l] = vfma(vmap(vmul(ex[l], r), lg2_approx), itau, d[l]);
-            const V dm = max_of(d);
-#pragma unroll
-            for (int l = 0; l < M; ++l) d[l] = vsub(d[l], dm);
-          }
+          for (int l = 0; l < M; ++l) d[l] = vfma(vmap(vmul(ex[l], r), lg2_approx), itau, vsub(d[l], lz));
         }
       }
-      if constexpr (M >= 8) flag |= vbelow(tmin, 7.52316384526264e-37f);  // 2^-120
     }
   }
 
-  // Reverse sweep (requires KEEP): dk = dL/dkappa for c = dL/dS.
+  // Reverse sweep (requires KEEP): dk = dL/dkappa for c = dL/dS at tau = 1, tau dL/dkappa
+  // otherwise (the sweep then runs on tau b: one product per member and step less).
   //   abar_l = b_l + (mu_l / tau) (c_l - <c, mu> + H_l - B),
   //   H_l = sum_{i != l} b_i / om_i,  B = sum_i b_i,
   // with om_i = 1 - mu_i formed as the sum of the other members' mu.  REUSE (tau = 1):
@@ -1140,8 +1133,7 @@ struct FastGroup {
       const V cmu = sum_of(cm);
 #pragma unroll
       for (int l = 0; l < M; ++l) {
-        V t = vsub(c[l], cmu);
-        if constexpr (!TAU1) t = vmul(itau, t);
+        const V t = vsub(c[l], cmu);
         b[l] = vmul(st.get(N - 1, l), t);
         // tau = 1: b / om(N-2) = mu(N-2) rt_last (c - <c, mu(N-1)>), no division
         if constexpr (TAU1 && N >= 2) hl[l] = vmul(vmul(st.get(N - 2, l), rt_last), t);
@@ -1160,21 +1152,29 @@ struct FastGroup {
 #pragma unroll
         for (int l = 0; l < M; ++l) h[l] = hl[l];
       }
-      // c_l - <c, mu> + H_l - B as (c_l + H_l) - K, K = <c, mu> + B = sum of (c mu + b)
-#pragma unroll
-      for (int l = 0; l < M; ++l) cm[l] = vfma(c[l], mk[l], b[l]);
-      const V K = sum_of(cm);
       exclusive_sums(h, H);
+      if constexpr (TAU1) {
+        // c_l - <c, mu> + H_l - B as (c_l + H_l) - K, K = <c, mu> + B = sum of (c mu + b)
 #pragma unroll
-      for (int l = 0; l < M; ++l) {
-        if constexpr (TAU1 && REUSE) {
-          // b + mu (c + H - K) = (c mu + b) + mu (H - K), and c mu + b is cm
-          b[l] = vfma(mk[l], vsub(H[l], K), cm[l]);
-        } else if constexpr (TAU1) {
-          b[l] = vfma(mk[l], vsub(vadd(c[l], H[l]), K), b[l]);
-        } else {
-          b[l] = vfma(vmul(mk[l], itau), vsub(vadd(c[l], H[l]), K), b[l]);
+        for (int l = 0; l < M; ++l) cm[l] = vfma(c[l], mk[l], b[l]);
+        const V K = sum_of(cm);
+#pragma unroll
+        for (int l = 0; l < M; ++l) {
+          if constexpr (REUSE) {
+            // b + mu (c + H - K) = (c mu + b) + mu (H - K), and c mu + b is cm
+            b[l] = vfma(mk[l], vsub(H[l], K), cm[l]);
+          } else {
+            b[l] = vfma(mk[l], vsub(vadd(c[l], H[l]), K), b[l]);
+          }
         }
+      } else {
+        // K = <c, mu> + sum b / tau
+        V p = vmul(c[0], mk[0]), q = vmul(c[1], mk[1]);
+#pragma unroll
+        for (int l = 2; l < M; l += 2) p = vfma(c[l], mk[l], p), q = vfma(c[l + 1], mk[l + 1], q);
+        const V K = vfma(sum_of(b), itau, vadd(p, q));
+#pragma unroll
+        for (int l = 0; l < M; ++l) b[l] = vfma(mk[l], vfma(H[l], itau, vsub(c[l], K)), b[l]);
       }
     };
 #pragma unroll

@@ -55,8 +55,6 @@ constexpr size_t kBwdDeferOffset = (kHistOffset<N, M> + kHistBytes<N, M> + 15) &
 // 576 / 560 at 0.1), and at small tau lambda nearly all groups of spread logits do.
 constexpr float kSliceWideTau = 0.1f;
 constexpr float kSliceWideTauLambda = 0.05f;
-constexpr float kLeastRange = -98.0f;  // of the plain tau != 1 relaxation (SliceRelax::forward)
-
 __device__ __forceinline__ float shfl_xor(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ F2 swap(F2 v) { return f2(hi(v), lo(v)); }
 
@@ -345,7 +343,7 @@ struct SliceRelax {
       // the sum that was formed, is at least 2^-99 while
       // log2 total + max(1, tau) log2 (next total) >= -98, and members that were flushed
       // to zero are below the sum's last bit.
-      const float tau1 = fmaxf(1.0f, __fdiv_rn(1.0f, inv_tau));
+      const float tau1 = fmaxf(1.0f, rcp_approx(inv_tau));
       float lz_prev = 0.0f;
 #pragma unroll
       for (int i = 0; i < kPk; ++i) x[i] = (kap[i] - f2(kmax)) * itau;
