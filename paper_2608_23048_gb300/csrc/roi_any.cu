@@ -35,6 +35,7 @@ struct AnyArgs {
   int N, M;
   float tau, inv_tau;
   NoiseParams np;
+  bool wait;  // pdl_begin
 };
 
 template <int MP>
@@ -212,6 +213,7 @@ template <int MP>
 __global__ void __launch_bounds__(kThreads) roi_any_fwd_kernel(AnyArgs a, bool words) {
   using V = typename Lanes<MP>::V;
   constexpr int L = vlanes<V>();
+  pdl_begin(a.wait);
   const int64_t lanes = (a.groups + L - 1) / L;
   const int64_t stride = int64_t(gridDim.x) * kThreads;
   for (int64_t t0 = int64_t(blockIdx.x) * kThreads; t0 < lanes; t0 += stride) {
@@ -308,6 +310,7 @@ template <int MP>
 __global__ void __launch_bounds__(kThreads) roi_any_bwd_kernel(AnyArgs a) {
   using V = typename Lanes<MP>::V;
   constexpr int L = vlanes<V>();
+  pdl_begin(a.wait);
   const V itau = vconst<V>(a.inv_tau);
   const int64_t lanes = (a.groups + L - 1) / L;
   const int64_t stride = int64_t(gridDim.x) * kThreads;
@@ -456,11 +459,13 @@ int launch_any_fwd(const FwdCall& c) {
     // groups straddle words: assembled with atomicOr
     if (cudaMemsetAsync(c.hard, 0, size_t((c.E + 31) / 32) * 4, c.stream) != cudaSuccess) return -1;
   }
-  if (c.M <= 4) roi_any_fwd_kernel<4><<<any_grid(a.groups, 2), kThreads, 0, c.stream>>>(a, words);
-  else if (c.M <= 8) roi_any_fwd_kernel<8><<<any_grid(a.groups, 2), kThreads, 0, c.stream>>>(a, words);
-  else if (c.M <= 16) roi_any_fwd_kernel<16><<<any_grid(a.groups, 1), kThreads, 0, c.stream>>>(a, words);
-  else roi_any_fwd_kernel<32><<<any_grid(a.groups, 1), kThreads, 0, c.stream>>>(a, words);
-  return cudaGetLastError() == cudaSuccess ? 1 : -1;
+  a.wait = lone_pdl(c.stream);
+  int r;
+  if (c.M <= 4) r = launch_maybe_pdl(roi_any_fwd_kernel<4>, any_grid(a.groups, 2), kThreads, 0, c.stream, a.wait, a, words);
+  else if (c.M <= 8) r = launch_maybe_pdl(roi_any_fwd_kernel<8>, any_grid(a.groups, 2), kThreads, 0, c.stream, a.wait, a, words);
+  else if (c.M <= 16) r = launch_maybe_pdl(roi_any_fwd_kernel<16>, any_grid(a.groups, 1), kThreads, 0, c.stream, a.wait, a, words);
+  else r = launch_maybe_pdl(roi_any_fwd_kernel<32>, any_grid(a.groups, 1), kThreads, 0, c.stream, a.wait, a, words);
+  return r;
 }
 
 int launch_any_bwd(const BwdCall& c) {
@@ -481,11 +486,13 @@ int launch_any_bwd(const BwdCall& c) {
   a.tau = c.tau;
   a.inv_tau = 1.0f / c.tau;
   a.np = c.np;
-  if (c.M <= 4) roi_any_bwd_kernel<4><<<any_grid(a.groups, 2), kThreads, 0, c.stream>>>(a);
-  else if (c.M <= 8) roi_any_bwd_kernel<8><<<any_grid(a.groups, 2), kThreads, 0, c.stream>>>(a);
-  else if (c.M <= 16) roi_any_bwd_kernel<16><<<any_grid(a.groups, 1), kThreads, 0, c.stream>>>(a);
-  else roi_any_bwd_kernel<32><<<any_grid(a.groups, 1), kThreads, 0, c.stream>>>(a);
-  return cudaGetLastError() == cudaSuccess ? 1 : -1;
+  a.wait = lone_pdl(c.stream);
+  int r;
+  if (c.M <= 4) r = launch_maybe_pdl(roi_any_bwd_kernel<4>, any_grid(a.groups, 2), kThreads, 0, c.stream, a.wait, a);
+  else if (c.M <= 8) r = launch_maybe_pdl(roi_any_bwd_kernel<8>, any_grid(a.groups, 2), kThreads, 0, c.stream, a.wait, a);
+  else if (c.M <= 16) r = launch_maybe_pdl(roi_any_bwd_kernel<16>, any_grid(a.groups, 1), kThreads, 0, c.stream, a.wait, a);
+  else r = launch_maybe_pdl(roi_any_bwd_kernel<32>, any_grid(a.groups, 1), kThreads, 0, c.stream, a.wait, a);
+  return r;
 }
 
 }  // namespace roi

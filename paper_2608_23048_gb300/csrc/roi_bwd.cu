@@ -83,6 +83,7 @@ struct BwdArgs {
   float tau, inv_tau;
   NoiseParams np;
   unsigned int* status;
+  bool wait;  // pdl_begin
 };
 
 // The fused optimizer's arguments (read only by the OPT instantiations).
@@ -525,7 +526,7 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks) roi_bwd_
   dg.init(smem + kDeferOffset<N, M, OPT>);
   const auto exact = [&](int64_t g0) { bwd_exact_group<N, M, ST, OPT>(g0, a, o); };
   // a batch's next tensor may start on the SMs this launch frees (no-op otherwise)
-  pdl_launch_dependents();
+  pdl_begin(a.wait);
   const bool ok = run_tiles<C::kThreads, C::kTile, C::kStages, 3>(
       smem, src, a.full_tiles, a.status,
       [&](const uint8_t* const* stage, int64_t tile, const auto& release) {
@@ -560,6 +561,7 @@ struct BwdItem {
 struct BwdMulti {
   int count;
   int64_t total_tiles, total_tails;
+  bool wait;
   float tau, inv_tau;
   unsigned int* status;
   AdamW opt;
@@ -582,6 +584,7 @@ __device__ __forceinline__ BwdArgs multi_args(const BwdMulti& mm, int i) {
   a.inv_tau = mm.inv_tau;
   a.np = x.np;
   a.status = mm.status;
+  a.wait = false;
   return a;
 }
 __device__ __forceinline__ BwdOptArgs multi_opt(const BwdMulti& mm, int i) {
@@ -627,7 +630,7 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
   BwdArgs a;
   BwdOptArgs o;
   const uint8_t* src_ptr[3] = {nullptr, nullptr, nullptr};
-  pdl_launch_dependents();
+  pdl_begin(mm.wait);
   const bool ok = run_tiles_src<C::kThreads, C::kTile, C::kStages, 3>(
       smem, esize, mm.total_tiles, mm.status,
       [&](int64_t t, int arr) {
@@ -686,8 +689,9 @@ int launch_tiles(const BwdArgs& a, const BwdOptArgs& o, cudaStream_t stream, boo
   }
   const int64_t cap = int64_t(sm_count()) * cache.per_sm[dev];
   BwdArgs b = a;
+  b.wait = !pdl && lone_pdl(stream);
   const int grid = tile_grid(b.full_tiles, a.E, M, C::kTailChunk, C::kTile, cap, pdl ? 0 : C::kTailRounds);
-  return launch_maybe_pdl(kern, grid, C::kThreads, smem, stream, pdl, b, o);
+  return launch_maybe_pdl(kern, grid, C::kThreads, smem, stream, pdl || b.wait, b, o);
 }
 
 template <int N, int M, bool ST, bool OPT, bool NARROW_ONLY = false>
@@ -736,7 +740,7 @@ int launch_multi_kern(const BwdMulti& mm, cudaStream_t stream, bool pdl) {
   const int64_t cap = int64_t(sm_count()) * cache.per_sm[dev];
   const int64_t want = mm.total_tiles + mm.total_tails;
   const int grid = int(want < 1 ? 1 : (want < cap ? want : cap));
-  return launch_maybe_pdl(kern, grid, C::kThreads, smem, stream, pdl, mm);
+  return launch_maybe_pdl(kern, grid, C::kThreads, smem, stream, pdl || mm.wait, mm);
 }
 
 template <int N, int M, bool ST, bool OPT, bool NARROW_ONLY = false>
@@ -788,6 +792,7 @@ int launch_multi(const BwdCall* calls, int count, bool pdl) {
   mm.total_tiles = tiles;
   mm.total_tails = tails;
   const cudaStream_t stream = calls[0].stream;
+  mm.wait = !pdl && lone_pdl(stream);
   const int kind = bwd_kind(calls[0]);
   const bool narrow = mm.it[0].np.narrow;
   if constexpr (N == 4 && M == 8) {

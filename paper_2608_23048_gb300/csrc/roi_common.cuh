@@ -1208,6 +1208,14 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t by
 // Programmatic dependent launch: let the stream's next launch start early / wait
 // for the previous launch to complete (both no-ops for an ordinary launch).
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// The start of a kernel that takes the programmatic launches up: `wait` (a launch that
+// follows arbitrary work, see lone_pdl) waits for everything before it, and only then may
+// what follows be let in, which need not wait itself.
+__device__ __forceinline__ void pdl_wait();
+__device__ __forceinline__ void pdl_begin(bool wait) {
+  if (wait) pdl_wait();
+  pdl_launch_dependents();
+}
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");

@@ -63,6 +63,7 @@ struct ExportArgs {
   int64_t full_tiles;
   int N;
   unsigned int* status;
+  bool wait;  // pdl_begin
 };
 
 // The deployment mask of one group.
@@ -119,6 +120,7 @@ __global__ void __launch_bounds__(kThreads, 1) roi_export_tiles_kernel(ExportArg
   extern __shared__ __align__(128) uint8_t smem[];
   using C = ExportCfg<M, MODE>;
   constexpr int NARR = MODE == kBits ? 1 : 2;
+  pdl_begin(a.wait);
   TileSrc<NARR> src;
   src.ptr[0] = reinterpret_cast<const uint8_t*>(a.phi);
   src.esize[0] = 4;
@@ -166,8 +168,8 @@ int launch_tiles(ExportArgs a, cudaStream_t stream) {
   if (a.full_tiles < sm_count()) a.full_tiles = 0;
   const int64_t want = a.full_tiles + ((a.E - a.full_tiles * C::kTile) / M + kThreads - 1) / kThreads;
   const int64_t cap = sm_count();
-  kern<<<int(want < 1 ? 1 : (want < cap ? want : cap)), kThreads, C::kSmem, stream>>>(a);
-  return cudaGetLastError() == cudaSuccess ? 1 : -1;
+  a.wait = lone_pdl(stream);
+  return launch_maybe_pdl(kern, int(want < 1 ? 1 : (want < cap ? want : cap)), kThreads, C::kSmem, stream, a.wait, a);
 }
 
 int grid_for(int64_t items, int threads) {

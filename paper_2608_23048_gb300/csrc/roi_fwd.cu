@@ -47,6 +47,7 @@ struct FwdArgs {
   float tau, inv_tau;
   NoiseParams np;
   unsigned int* status;
+  bool wait;  // pdl_begin
 };
 
 template <int M>
@@ -382,7 +383,7 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks) roi_fwd_
   src.ptr[1] = reinterpret_cast<const uint8_t*>(a.W);
   src.esize[1] = 2;
   // a batch's next tensor may start on the SMs this launch frees (no-op otherwise)
-  pdl_launch_dependents();
+  pdl_begin(a.wait);
   const bool ok = run_tiles<C::kThreads, C::kTile, C::kStages, 2>(
       smem, src, a.full_tiles, a.status,
       [&](const uint8_t* const* stage, int64_t tile, const auto& release) {
@@ -419,7 +420,7 @@ struct FwdItem {
 struct FwdMulti {
   int count;
   int64_t total_tiles, total_tails;
-  bool st;
+  bool st, wait;
   float tau, inv_tau;
   unsigned int* status;
   FwdItem it[kMultiMax];
@@ -441,6 +442,7 @@ __device__ __forceinline__ FwdArgs multi_args(const FwdMulti& mm, int i) {
   a.inv_tau = mm.inv_tau;
   a.np = x.np;
   a.status = mm.status;
+  a.wait = false;
   return a;
 }
 // The tile kernel over many small tensors at once: the persistent CTAs walk the
@@ -477,7 +479,7 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
   FwdArgs a;
   const float* src_phi = nullptr;
   const uint16_t* src_W = nullptr;
-  pdl_launch_dependents();
+  pdl_begin(mm.wait);
   const bool ok = run_tiles_src<C::kThreads, C::kTile, C::kStages, 2>(
       smem, esize, mm.total_tiles, mm.status,
       [&](int64_t t, int arr) {
@@ -540,8 +542,9 @@ int launch_tiles(const FwdArgs& a, cudaStream_t stream, bool pdl) {
   }
   const int64_t cap = int64_t(sm_count()) * cache.per_sm[dev];
   FwdArgs b = a;
+  b.wait = !pdl && lone_pdl(stream);
   const int grid = tile_grid(b.full_tiles, a.E, M, C::kTailChunk, C::kTile, cap, pdl ? 0 : C::kTailRounds);
-  return launch_maybe_pdl(kern, grid, C::kThreads, smem, stream, pdl, b);
+  return launch_maybe_pdl(kern, grid, C::kThreads, smem, stream, pdl || b.wait, b);
 }
 
 template <int N, int M, bool ST>
@@ -576,7 +579,7 @@ int launch_multi_kern(const FwdMulti& mm, cudaStream_t stream, bool pdl) {
   const int64_t cap = int64_t(sm_count()) * cache.per_sm[dev];
   const int64_t want = mm.total_tiles + mm.total_tails;
   const int grid = int(want < 1 ? 1 : (want < cap ? want : cap));
-  return launch_maybe_pdl(kern, grid, C::kThreads, C::kMultiSmem, stream, pdl, mm);
+  return launch_maybe_pdl(kern, grid, C::kThreads, C::kMultiSmem, stream, pdl || mm.wait, mm);
 }
 
 template <int N, int M, bool ST>
@@ -618,6 +621,7 @@ int launch_multi(const FwdCall* calls, int count, bool pdl) {
   mm.total_tiles = tiles;
   mm.total_tails = tails;
   const cudaStream_t stream = calls[0].stream;
+  mm.wait = !pdl && lone_pdl(stream);
   const bool wide = wide_range<N>(mm.tau, mm.it[0].np);
   return mm.st ? launch_multi_st<N, M, true>(mm, wide, stream, pdl)
                : launch_multi_st<N, M, false>(mm, wide, stream, pdl);

@@ -154,6 +154,20 @@ int launch_maybe_pdl(void (*kern)(KArgs...), int grid, int threads, size_t smem,
   return cudaLaunchKernelEx(&cfg, kern, args...) == cudaSuccess ? 1 : -1;
 }
 
+// Whether a launch that follows arbitrary work on `stream` may be made with programmatic
+// stream serialization all the same: its kernel then waits for that work itself
+// (pdl_begin), and the launch and the CTAs' start hide behind the end of a predecessor that
+// lets dependents in (2 us a call in a row of single calls).  Not under stream capture,
+// where the predecessor may be no kernel at all.
+inline bool lone_pdl(cudaStream_t stream) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &s) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return s == cudaStreamCaptureStatusNone;
+}
+
 // Streaming multiprocessors of the current device (cached).
 int sm_count();
 

@@ -58,6 +58,7 @@ struct LinArgs {
   float tau, inv_tau;
   NoiseParams np;
   unsigned int* status;
+  bool wait;              // pdl_wait before anything is read
 };
 
 // Shared-memory layout (bytes from the 1024-aligned dynamic base), per stage:
@@ -239,9 +240,6 @@ __global__ void __launch_bounds__(LinCfg<M>::kThreads + 32, 1)
   uint32_t* misc = reinterpret_cast<uint32_t*>(smem + L.misc);    // [0] TMEM base, [2] ok
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool producer = warp == kComputeWarps;  // TMA and MMA issue (one elected lane)
-  // the split-K reduction launch may be scheduled now (it waits for this grid)
-  pdl_launch_dependents();
-
   const int rb = blockIdx.x / a.splits, sp = blockIdx.x % a.splits;
   const int row0 = rb * kRows;
   const int base = a.nchunks / a.splits, rem = a.nchunks % a.splits;
@@ -263,6 +261,9 @@ __global__ void __launch_bounds__(LinCfg<M>::kThreads + 32, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = misc[0];
+  // the split-K reduction, or whatever follows, may be scheduled once the work before this
+  // launch is done (it waits for this grid)
+  pdl_begin(a.wait);
 
   bool ok = true;
   const uint64_t lim = ring_wait_limit(a.status);
@@ -373,7 +374,7 @@ __global__ void __launch_bounds__(LinCfg<M>::kThreads + 32, 1)
 // split order, four consecutive outputs per thread when n % 4 == 0 (part and Y are
 // 16-byte aligned), the loads of up to eight splits in flight.
 __global__ void __launch_bounds__(256) roi_linear_reduce_kernel(const float* part, float* Y, int splits, int64_t n) {
-  pdl_wait();  // the partials of the GEMM launched before
+  pdl_begin(true);  // the partials of the GEMM launched before
   const int64_t stride = int64_t(gridDim.x) * blockDim.x;
   if ((n & 3) == 0) {
     const int64_t n4 = n / 4;
@@ -466,8 +467,9 @@ int launch_nm(const LinearCall& c, const LinArgs& a) {
     cur = want;
   }
   const int64_t row_blocks = (a.rows + kRows - 1) / kRows;
-  kern<<<int(row_blocks * a.splits), LinCfg<M>::kThreads + 32, smem, c.stream>>>(tm_phi, tm_w, tm_x, a);
-  if (cudaGetLastError() != cudaSuccess) return -1;
+  if (launch_maybe_pdl(kern, int(row_blocks * a.splits), LinCfg<M>::kThreads + 32, smem, c.stream, a.wait, tm_phi, tm_w,
+                       tm_x, a) < 0)
+    return -1;
   if (a.splits == 1) return 1;
   const int64_t n = a.T * a.rows;
   const int64_t items = (n & 3) == 0 ? n / 4 : n;
@@ -517,6 +519,7 @@ int launch_masked_linear(const LinearCall& c) {
   a.np = c.np;
   a.np.narrow = counters_narrow(c.np, c.rows * c.cols);
   a.status = c.status;
+  a.wait = lone_pdl(c.stream);
   // split K only as far as the caller's workspace holds the partials
   int splits = linear_splits(c.T, c.rows, c.cols);
   const size_t per_split = size_t(c.T) * size_t(c.rows) * 4;

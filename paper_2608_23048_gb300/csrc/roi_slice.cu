@@ -179,6 +179,7 @@ struct SliceArgs {
   float tau, inv_tau;
   NoiseParams np;
   unsigned int* status;
+  bool wait;  // pdl_begin
 };
 
 // Dynamic shared memory of the kernels (tile ring, then the step history, the queues).
@@ -775,7 +776,7 @@ __device__ __forceinline__ void slice_walk(const SliceArgs& a, const TileSrc<NAR
   DeferredGroups<kDeferCap<M, Shape>> dg;
   dg.init(roi_slice_smem + defer_at);
   // a batch's next tensor may start on the SMs this launch frees (no-op otherwise)
-  pdl_launch_dependents();
+  pdl_begin(a.wait);
   const bool ok = run_tiles<Shape::kThreads, kTile, Shape::kStages, NARR>(
       roi_slice_smem, src, a.full_tiles, a.status, [&](const uint8_t* const* stage, int64_t tile, const auto& release) {
         const int64_t e0 = tile * kTile + P * int64_t(threadIdx.x);
@@ -849,6 +850,7 @@ struct LaunchCache {
 template <class Shape, class Kern>
 int launch_persistent(Kern kern, LaunchCache& cache, size_t smem, SliceArgs a, cudaStream_t stream, bool pdl) {
   a.full_tiles = a.E / kTileOf<Shape>;
+  a.wait = !pdl && lone_pdl(stream);
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
   if (cache.per_sm[dev] == 0) {
@@ -860,7 +862,7 @@ int launch_persistent(Kern kern, LaunchCache& cache, size_t smem, SliceArgs a, c
   }
   const int64_t cap = int64_t(sm_count()) * cache.per_sm[dev];
   const int grid = int(a.full_tiles < 1 ? 1 : (a.full_tiles < cap ? a.full_tiles : cap));
-  return launch_maybe_pdl(kern, grid, Shape::kThreads, smem, stream, pdl, a);
+  return launch_maybe_pdl(kern, grid, Shape::kThreads, smem, stream, pdl || a.wait, a);
 }
 
 template <int N, int M, bool TAU1, bool WIDE>
