@@ -106,7 +106,8 @@ roi_status roi_mask_fwd_ex(const float* logits, const roi_bf16* W, int N, int M,
  * its predecessor, so the work queued after the call sees every item done.  For
  * (2, 4), (4, 8) and (2, 8), runs of consecutive items small enough that each would
  * give an SM fewer than 12 tiles of work share one launch (runs of at least 8 items;
- * 2 for roi_mask_bwd_batch).  Items with rows == 0 are skipped.
+ * 2 for roi_mask_bwd_batch); for (8, 16) and (16, 32) runs of at least 8 of fewer than 4
+ * tiles, or 4 of fewer than one.  Items with rows == 0 are skipped.
  * `items` is host memory, read during the call. */
 typedef struct {
     const float* logits;  /* [rows, cols] */

@@ -685,6 +685,17 @@ int launch_fwd_batch(const FwdCall* calls, int count) {
         continue;
       }
     }
+    if (slice_supported(c.N, c.M)) {
+      const int n = slice_fwd_run(calls + i, count - i);
+      if (n > 0) {
+        const int r = launch_slice_fwd_multi(calls + i, n, prev_tiled);
+        if (r < 0) return -1;
+        launched += r;
+        prev_tiled = true;
+        i += n;
+        continue;
+      }
+    }
     const bool tiled = (c.N == 2 && c.M == 4) || (c.N == 4 && c.M == 8) || (c.N == 2 && c.M == 8) ||
                        slice_supported(c.N, c.M);
     const int r = launch_fwd_impl(c, tiled && prev_tiled);

@@ -120,6 +120,11 @@ int launch_export_compressed_2of4(const CompressCall& c);
 bool slice_supported(int N, int M);
 int launch_slice_fwd(const FwdCall& c, bool pdl = false);
 int launch_slice_bwd(const BwdCall& c, bool pdl = false);
+// A batch's runs of small tensors, one launch each.
+int slice_fwd_run(const FwdCall* calls, int count);
+int slice_bwd_run(const BwdCall* calls, int count);
+int launch_slice_fwd_multi(const FwdCall* calls, int count, bool pdl);
+int launch_slice_bwd_multi(const BwdCall* calls, int count, bool pdl);
 // Every other (N, M) (roi_any.cu).
 int launch_any_fwd(const FwdCall& c);
 int launch_any_bwd(const BwdCall& c);

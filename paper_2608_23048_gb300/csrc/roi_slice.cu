@@ -8,6 +8,8 @@
 // memory.  Groups whose keys leave the fast path's range are queued by the slice's first
 // lane (DeferredGroups) and handled 32 at a time, one per lane, by WideRobustGroup
 // (ExactGroup for non-finite keys).
+#include <type_traits>
+
 #include "roi_launch.h"
 #include "roi_tiles.cuh"
 
@@ -751,23 +753,41 @@ __device__ __forceinline__ bool bwd_lane(const float* p, const uint16_t* w, cons
     }
   }
   rx.backward(c, a.inv_tau, b);
-  if (active && !flag) {
-    const F2 scale = f2(a.inv_tau * a.np.inv_lam);
+  const F2 scale = f2(a.inv_tau * a.np.inv_lam);
 #pragma unroll
-    for (int i = 0; i < kPk; ++i) b[i] = b[i] * scale;
-    if (a.dphi != nullptr) store_lane(a.dphi + e0, b);
-    if (a.phi_out != nullptr) {
+  for (int i = 0; i < kPk; ++i) b[i] = b[i] * scale;
+  if (a.phi_out == nullptr) {
+    if (active && !flag) store_lane(a.dphi + e0, b);
+  } else {
+    // Fused AdamW: the gradients go through this warp's own slots of the step history (read
+    // for the last time above), so that consecutive lanes load and store consecutive 16
+    // bytes of logits and moments; a lane's own 64 bytes at a time cost the 8:16 backward
+    // 25 % (a 67 M element block 996 -> 790 us).  The plain gradients alone are not worth it
+    // (16:32, one 3B-shaped block 1664 -> 1750 us).
+    ulonglong2* row = rx.hist;
 #pragma unroll
-      for (int s = 0; s < P / 4; ++s) {
-        const float g4[4] = {lo(b[2 * s]), hi(b[2 * s]), lo(b[2 * s + 1]), hi(b[2 * s + 1])};
-        adamw4(a.phi_out, a.m, a.v, e0 + 4 * s, reinterpret_cast<const float4*>(a.phi + e0)[s], g4, a.opt);
+    for (int i = 0; i < P / 4; ++i) row[i * BwdShape<M>::kThreads] = make_ulonglong2(b[2 * i].v, b[2 * i + 1].v);
+    const uint32_t mine = __ballot_sync(0xffffffffu, active && !flag);
+    __syncwarp();
+    const int64_t warp_e0 = e0 - int64_t(lane) * P;
+#pragma unroll 1
+    for (int i = 0; i < P / 4; ++i) {
+      const int q4 = i * 32 + lane;  // which four of the warp's members
+      const int owner = q4 / (P / 4);
+      if ((mine >> owner) & 1u) {
+        const float4 g = *reinterpret_cast<const float4*>(row + (q4 % (P / 4)) * BwdShape<M>::kThreads + owner - lane);
+        const int64_t e = warp_e0 + 4 * q4;
+        if (a.dphi != nullptr) *reinterpret_cast<float4*>(a.dphi + e) = g;
+        const float g4[4] = {g.x, g.y, g.z, g.w};
+        adamw4(a.phi_out, a.m, a.v, e, *reinterpret_cast<const float4*>(a.phi + e), g4, a.opt);
       }
     }
+    __syncwarp();  // the next group's steps go to these slots
   }
   return active && q == 0 && flag;
 }
 
-// Runs `tile` for the CTA's full tiles and, on the last CTA, for the ragged tail straight
+// Runs `lane_fn` for the CTA's full tiles and its chunks of the ragged tail, these straight
 // from global memory, queueing the groups it returns true for and handling them by `exact`.
 template <int M, class Shape, int NARR, class Exact, class Lane>
 __device__ __forceinline__ void slice_walk(const SliceArgs& a, const TileSrc<NARR>& src, size_t defer_at, const Exact& exact,
@@ -787,21 +807,21 @@ __device__ __forceinline__ void slice_walk(const SliceArgs& a, const TileSrc<NAR
         dg.drain(false, exact);
       });
   if (ok) {
+    // the ragged tail in warps of lanes, dealt out over the SMs first
     const int64_t t0 = a.full_tiles * kTile;
-    const int64_t lanes = blockIdx.x == gridDim.x - 1 ? (a.E - t0) / P : 0;
-    for (int64_t r = 0;; r += Shape::kThreads) {
-      if (r < lanes) {
-        const bool active = threadIdx.x + r < lanes;
-        const int64_t e0 = t0 + P * (active ? threadIdx.x + r : 0);
-        const uint8_t* at[NARR];
+    const int64_t lanes = (a.E - t0) / P;
+    const int lane = threadIdx.x & 31;
+    for (int64_t r = 32 * (tail_rank(a.full_tiles) + int64_t(threadIdx.x >> 5) * gridDim.x); r < lanes;
+         r += int64_t(gridDim.x) * Shape::kThreads) {
+      const bool active = r + lane < lanes;
+      const int64_t e0 = t0 + P * (r + lane);
+      const uint8_t* at[NARR];
 #pragma unroll
-        for (int i = 0; i < NARR; ++i) at[i] = src.ptr[i] + size_t(e0) * src.esize[i];
-        dg.push(lane_fn(at, e0, active, [] {}), e0);
-      }
-      const bool done = r + Shape::kThreads >= lanes;
-      dg.drain(done, exact);
-      if (done) break;
+      for (int i = 0; i < NARR; ++i) at[i] = src.ptr[i] + (active ? size_t(e0) * src.esize[i] : 0);
+      dg.push(lane_fn(at, e0, active, [] {}), e0);
+      dg.drain(false, exact);
     }
+    dg.drain(true, exact);
   }
   // the launch completes only after the batch's previous one (stream order)
   if (blockIdx.x == 0) pdl_wait();
@@ -840,8 +860,93 @@ __global__ void __launch_bounds__(BwdShape<M>::kThreads, 1) roi_slice_bwd_kernel
                 });
 }
 
+// Multi-tensor launches (a batch's runs of small tensors): the tensors' warps, one after
+// another, dealt out over the SMs first; straight from global memory, as the ragged tails.
+constexpr int kMultiMax = 192;
+struct SliceItem {
+  const float* phi;
+  const uint16_t* W;
+  const uint16_t* dWm;
+  uint16_t* Wm;
+  float* soft;
+  uint32_t* hard;
+  float* dphi;
+  uint16_t* dW;
+  const uint32_t* hard_in;
+  float* phi_out;
+  float* m;
+  float* v;
+  int64_t E;
+  int64_t tail0;  // first warp of the tensor in the launch
+  NoiseParams np;
+};
+struct SliceMulti {
+  int count;
+  int64_t total;  // warps
+  bool st, wait;
+  float tau, inv_tau;
+  AdamW opt;
+  unsigned int* status;
+  SliceItem it[kMultiMax];
+};
+static_assert(sizeof(SliceMulti) <= 32764, "kernel parameter block");
+__device__ __forceinline__ SliceArgs slice_args(const SliceMulti& mm, int i) {
+  const SliceItem& x = mm.it[i];
+  SliceArgs a;
+  a.phi = x.phi, a.W = x.W, a.dWm = x.dWm;
+  a.Wm = x.Wm, a.soft = x.soft, a.hard = x.hard;
+  a.dphi = x.dphi, a.dW = x.dW, a.hard_in = x.hard_in;
+  a.phi_out = x.phi_out, a.m = x.m, a.v = x.v;
+  a.st = mm.st;
+  a.opt = mm.opt;
+  a.E = x.E;
+  a.full_tiles = 0;
+  a.tau = mm.tau, a.inv_tau = mm.inv_tau;
+  a.np = x.np;
+  a.status = mm.status;
+  a.wait = false;
+  return a;
+}
+template <int M, bool BWD>
+using ShapeOf = typename std::conditional<BWD, BwdShape<M>, FwdShape<M>>::type;
+template <int N, int M, bool TAU1, bool WIDE, bool BWD>
+__global__ void __launch_bounds__(ShapeOf<M, BWD>::kThreads, 1) roi_slice_multi_kernel(const __grid_constant__ SliceMulti mm) {
+  using C = ShapeOf<M, BWD>;
+  constexpr int P = C::kP;
+  constexpr int64_t kLow = (int64_t(1) << 48) - 1;
+  DeferredGroups<kDeferCap<M, C>> dg;
+  dg.init(roi_slice_smem + (BWD ? kBwdDeferOffset<N, M> : kFwdDeferOffset<M>));
+  const auto exact = [&](int64_t e) {
+    if constexpr (BWD) {
+      exact_group_bwd<N, M, WIDE>(e & kLow, slice_args(mm, int(e >> 48)));
+    } else {
+      exact_group_fwd<N, M, WIDE>(e & kLow, slice_args(mm, int(e >> 48)));
+    }
+  };
+  pdl_begin(mm.wait);
+  const int lane = threadIdx.x & 31;
+  for (int64_t w = blockIdx.x + int64_t(threadIdx.x >> 5) * gridDim.x; w < mm.total; w += int64_t(gridDim.x) * (C::kThreads / 32)) {
+    const int i = tail_item(mm, w);
+    const SliceArgs a = slice_args(mm, i);
+    const int64_t l = 32 * (w - mm.it[i].tail0) + lane;
+    const bool active = l < a.E / P;
+    const int64_t e0 = P * l, at = active ? e0 : 0;
+    bool defer;
+    if constexpr (BWD) {
+      defer = bwd_lane<N, M, P, TAU1, WIDE>(a.phi + at, a.W + at, a.dWm + at, e0, active, a, [] {});
+    } else {
+      defer = fwd_lane<N, M, P, TAU1, WIDE>(a.phi + at, a.W + at, e0, active, a, [] {});
+    }
+    dg.push(defer, int64_t(i) << 48 | e0);
+    dg.drain(false, exact);
+  }
+  dg.drain(true, exact);
+  // the launch completes only after the batch's previous one (stream order)
+  if (blockIdx.x == 0) pdl_wait();
+}
+
 // Whether a tau != 1 call takes the WIDE relaxation.
-bool slice_wide(const SliceArgs& a) { return a.tau < kSliceWideTau || a.tau < kSliceWideTauLambda * a.np.inv_lam; }
+bool slice_wide(float tau, const NoiseParams& np) { return tau < kSliceWideTau || tau < kSliceWideTauLambda * np.inv_lam; }
 
 struct LaunchCache {
   int per_sm[64] = {0};
@@ -861,7 +966,13 @@ int launch_persistent(Kern kern, LaunchCache& cache, size_t smem, SliceArgs a, c
     cache.per_sm[dev] = per_sm < 1 ? 1 : per_sm;
   }
   const int64_t cap = int64_t(sm_count()) * cache.per_sm[dev];
-  const int grid = int(a.full_tiles < 1 ? 1 : (a.full_tiles < cap ? a.full_tiles : cap));
+  // A lone tensor of less than one tile per SM goes as one ragged tail, its warps spread evenly
+  // over the SMs: a lane's sixteen members take N steps one after the other, and the fewer
+  // warps share an SM the sooner they are through.
+  if (a.full_tiles < cap && !pdl) a.full_tiles = 0;
+  const int64_t warps = ((a.E - a.full_tiles * kTileOf<Shape>) / Shape::kP + 31) / 32;
+  const int64_t want = a.full_tiles + warps;
+  const int grid = int(want < 1 ? 1 : (want < cap ? want : cap));
   return launch_maybe_pdl(kern, grid, Shape::kThreads, smem, stream, pdl || a.wait, a);
 }
 
@@ -883,17 +994,116 @@ int slice_bwd(const SliceArgs& a, cudaStream_t stream, bool pdl) {
 template <int N, int M>
 int slice_fwd_nm(const SliceArgs& a, cudaStream_t stream, bool pdl) {
   if (a.tau == 1.0f) return slice_fwd<N, M, true, false>(a, stream, pdl);
-  return slice_wide(a) ? slice_fwd<N, M, false, true>(a, stream, pdl) : slice_fwd<N, M, false, false>(a, stream, pdl);
+  return slice_wide(a.tau, a.np) ? slice_fwd<N, M, false, true>(a, stream, pdl) : slice_fwd<N, M, false, false>(a, stream, pdl);
 }
 template <int N, int M>
 int slice_bwd_nm(const SliceArgs& a, cudaStream_t stream, bool pdl) {
   if (a.tau == 1.0f) return slice_bwd<N, M, true, false>(a, stream, pdl);
-  return slice_wide(a) ? slice_bwd<N, M, false, true>(a, stream, pdl) : slice_bwd<N, M, false, false>(a, stream, pdl);
+  return slice_wide(a.tau, a.np) ? slice_bwd<N, M, false, true>(a, stream, pdl) : slice_bwd<N, M, false, false>(a, stream, pdl);
+}
+
+template <int N, int M, bool TAU1, bool WIDE, bool BWD>
+int slice_multi(const SliceMulti& mm, cudaStream_t stream, bool pdl) {
+  using C = ShapeOf<M, BWD>;
+  static LaunchCache cache;
+  constexpr size_t smem = (BWD ? kBwdDeferOffset<N, M> : kFwdDeferOffset<M>) + kDeferBytes<M, C>;
+  auto kern = roi_slice_multi_kernel<N, M, TAU1, WIDE, BWD>;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
+  if (cache.per_sm[dev] == 0) {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) return -1;
+    cache.per_sm[dev] = 1;
+  }
+  const int64_t cap = sm_count();
+  const int grid = int(mm.total < 1 ? 1 : (mm.total < cap ? mm.total : cap));
+  return launch_maybe_pdl(kern, grid, C::kThreads, smem, stream, pdl || mm.wait, mm);
+}
+template <int N, int M, bool BWD>
+int slice_multi_nm(const SliceMulti& mm, bool wide, cudaStream_t stream, bool pdl) {
+  if (mm.tau == 1.0f) return slice_multi<N, M, true, false, BWD>(mm, stream, pdl);
+  return wide ? slice_multi<N, M, false, true, BWD>(mm, stream, pdl) : slice_multi<N, M, false, false, BWD>(mm, stream, pdl);
+}
+
+void to_item(const FwdCall& c, SliceItem& x) {
+  x.Wm = c.Wm;
+  x.soft = c.soft;
+  x.hard = c.hard;
+}
+void to_item(const BwdCall& c, SliceItem& x) {
+  x.dWm = c.dWm;
+  x.dphi = c.dphi;
+  x.dW = c.dW;
+  x.hard_in = c.hard_in;
+  x.phi_out = c.phi_out;
+  x.m = c.m;
+  x.v = c.v;
+}
+void to_multi(const FwdCall& c, SliceMulti& mm) { mm.st = c.st; }
+void to_multi(const BwdCall& c, SliceMulti& mm) { mm.opt = c.opt; }
+
+// A batch's run of consecutive tensors that shares a launch: at least multi_min_run(false)
+// of less than four tiles per SM each, or four of less than one.  One launch per small
+// tensor costs its N serial steps each time (16:32, 70 tensors of a few thousand elements:
+// 374 -> 31 us forward and backward; 42 of up to 0.8 M: 680 -> 432; the seven of a block of
+// 0.4 M at the most: 42 -> 25).  The q, k, v, o tensors between a 3B-shaped block's large
+// ones are as fast chained (8:16 forward 317 against 325 us).
+template <class Call>
+int slice_run(const Call* calls, int count, int64_t tile) {
+  const auto run = [&](int64_t tiles_per_sm) {
+    int n = 0;
+    while (n < count && n < kMultiMax && calls[n].N == calls[0].N && calls[n].M == calls[0].M &&
+           calls[n].E < tiles_per_sm * tile * sm_count() &&
+           (calls[0].tau == 1.0f || slice_wide(calls[0].tau, calls[n].np) == slice_wide(calls[0].tau, calls[0].np)))
+      ++n;
+    return n;
+  };
+  const int n = run(4);
+  if (n >= multi_min_run(false)) return n;
+  const int m = run(1);
+  return m >= 4 ? m : 0;
+}
+template <bool BWD, class Call>
+int launch_slice_multi(const Call* calls, int count, bool pdl) {
+  static thread_local SliceMulti mm;
+  const Call& c0 = calls[0];
+  mm.count = count;
+  mm.tau = c0.tau;
+  mm.inv_tau = 1.0f / c0.tau;
+  mm.status = c0.status;
+  mm.wait = !pdl && lone_pdl(c0.stream);
+  mm.st = false;
+  to_multi(c0, mm);
+  int64_t warps = 0;
+  for (int i = 0; i < count; ++i) {
+    SliceItem& x = mm.it[i];
+    x = SliceItem{};
+    x.phi = calls[i].phi;
+    x.W = calls[i].W;
+    x.E = calls[i].E;
+    x.tail0 = warps;
+    x.np = calls[i].np;
+    to_item(calls[i], x);
+    warps += (calls[i].E / 16 + 31) / 32;
+  }
+  mm.total = warps;
+  const bool wide = slice_wide(c0.tau, c0.np);
+  if (c0.M == 16) return slice_multi_nm<8, 16, BWD>(mm, wide, c0.stream, pdl);
+  return slice_multi_nm<16, 32, BWD>(mm, wide, c0.stream, pdl);
 }
 
 }  // namespace
 
 bool slice_supported(int N, int M) { return (N == 8 && M == 16) || (N == 16 && M == 32); }
+
+// The run of small tensors that starts calls[0 .. count) and shares a launch (0: none).
+int slice_fwd_run(const FwdCall* calls, int count) {
+  return slice_run(calls, count, calls[0].M == 16 ? kTileOf<FwdShape<16>> : kTileOf<FwdShape<32>>);
+}
+int slice_bwd_run(const BwdCall* calls, int count) {
+  return slice_run(calls, count, calls[0].M == 16 ? kTileOf<BwdShape<16>> : kTileOf<BwdShape<32>>);
+}
+int launch_slice_fwd_multi(const FwdCall* calls, int count, bool pdl) { return launch_slice_multi<false>(calls, count, pdl); }
+int launch_slice_bwd_multi(const BwdCall* calls, int count, bool pdl) { return launch_slice_multi<true>(calls, count, pdl); }
 
 int launch_slice_fwd(const FwdCall& c, bool pdl) {
   SliceArgs a{};

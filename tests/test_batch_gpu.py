@@ -101,6 +101,53 @@ def test_batch_equals_single_calls(roi, N, M, tau):
         assert_same(a, b)
 
 
+# Runs of small tensors of the wide patterns share a launch: odd group counts, a tensor of
+# one group, outlier logits whose groups go to the exact routine (queue entries that name
+# their tensor), lambda on both sides of the relaxation's rule (tau lambda = 0.05).
+@pytest.mark.parametrize("N,M", [(8, 16), (16, 32)])
+@pytest.mark.parametrize("kind", ["soft", "st", "adamw"])
+@pytest.mark.parametrize("tau", [0.3, 1.0])
+def test_wide_pattern_runs_equal_single_calls(roi, N, M, kind, tau):
+    import torch
+    ts = make_set([(37, 32 * 13), (1, 32), (64, 512), (5, 96), (128, 1024), (3, 32 * 7)] * 3, 71)
+    g = torch.Generator().manual_seed(5)
+    for k, t in enumerate(ts):
+        t["st"] = t["st"][:3] + (0.15 if k // 6 == 1 else 1.1, 0)
+        out = torch.randint(0, 16, t["phi"].shape, generator=g).cuda()
+        t["phi"] = t["phi"] + 100.0 * (out == 0) - 100.0 * (out == 1)
+    flags = [(True, True, True)] * len(ts)
+    if kind == "soft":
+        for a, b in zip(run_single(roi, ts, N, M, tau, flags), run_batch(roi, ts, N, M, tau, flags)):
+            assert_same(a, b)
+        return
+    opt = roi.AdamW(1e-3, 0.9, 0.95, 1e-8, 0.05, 3)
+    res = []
+    for batch in (False, True):
+        os_ = [outputs(roi, t, *f) for t, f in zip(ts, flags)]
+        state = [[t["phi"].clone(), torch.full_like(t["phi"], 1e-5), torch.full_like(t["phi"], 1e-9)] for t in ts]
+        fwd = [(t["phi"], t["W"], t["st"], o["Wm"], o["soft"], o["hard"]) for t, o in zip(ts, os_)]
+        st = [(t["phi"], t["W"], t["st"], t["dWm"], o["hard"], o["dphi"], o["dW"]) for t, o in zip(ts, os_)]
+        ad = [(x[0], t["W"], t["st"], t["dWm"], x[1], x[2], o["dphi"], o["dW"]) for t, o, x in zip(ts, os_, state)]
+        if kind == "st" and batch:
+            roi.roi_mask_fwd_st_batch(fwd, N, M, tau)
+            roi.roi_mask_bwd_st_batch(st, N, M, tau)
+        elif kind == "st":
+            for p, W, s, Wm, soft, hard in fwd:
+                roi.roi_mask_fwd_st(p, W, N, M, tau, s, Wm, soft, hard)
+            for p, W, s, d, hard, dphi, dW in st:
+                roi.roi_mask_bwd_st(p, W, s, N, M, d, hard, tau, dphi, dW)
+        elif batch:
+            roi.roi_mask_bwd_adamw_batch(ad, N, M, tau, opt)
+        else:
+            for p, W, s, d, m, v, dphi, dW in ad:
+                roi.roi_mask_bwd_adamw(p, W, s, N, M, d, tau, m, v, opt, dphi, dW)
+        roi.roi_device_status()
+        res.append([dict(o, **dict(zip(("phi", "m", "v"), x))) for o, x in zip(os_, state)])
+    for a, b in zip(*res):
+        assert_same({k: v for k, v in a.items() if kind == "st" or k in ("phi", "m", "v", "dphi", "dW")},
+                    {k: v for k, v in b.items() if kind == "st" or k in ("phi", "m", "v", "dphi", "dW")})
+
+
 def test_batch_mixes_relaxations(roi):
     """lambda is each item's own, and at 4:8 it decides which relaxation an item takes: a
     run of small tensors on both sides of the rule is split there."""
