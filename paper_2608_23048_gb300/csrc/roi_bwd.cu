@@ -14,10 +14,13 @@ namespace {
 // tile (the two groups of a pair are relaxed in lockstep on packed FP32),
 // shared-memory stages, and the CTAs per SM the register budget is sized for.
 // One CTA per SM (see roi_fwd.cu): M = 4 with two pairs per thread and up to 128
-// registers; M = 8, whose paired sweep needs ~170 registers, with 384 threads.
-template <int M>
+// registers; M = 8, whose paired sweep needs ~170 registers, with 384 threads, but for
+// the straight-through and fused-AdamW forms (AUX) of 2:8, which wait on their extra
+// memory traffic and whose single sweep fits 128 (8960 x 1536 at tau = 0.3: straight-through
+// 48.1 -> 45.4 us, AdamW 101.4 -> 94.2, while the plain form measured 37.8 -> 38.9).
+template <int N, int M, bool AUX>
 struct Cfg {
-  static constexpr int kThreads = M == 4 ? 512 : 384;
+  static constexpr int kThreads = M == 4 || (N == 2 && AUX) ? 512 : 384;
   static constexpr int kPairs = M == 4 ? 2 : 1;
   static constexpr int kStages = M == 4 ? 3 : 2;  // 192 KB (M = 4), 96 KB + 72 KB step history (M = 8)
   static constexpr int kMinBlocks = 1;
@@ -34,35 +37,39 @@ struct Cfg {
   static constexpr bool kDefer = M == 4;
   static constexpr int kDeferCap = kDefer ? 32 + 64 * kPairs : 0;
 };
+// Patterns with narrow-only instantiations (NARROW_ONLY below).
+template <int N, int M>
+constexpr bool kNarrowKernels = N == 2;
 // Tensors of one multi-tensor launch, at most (its parameter block holds them all).
 constexpr int kMultiMaxBwd = 192;
 // Byte offset of the shared-memory step history (M = 8) behind the tile ring,
 // and its size: steps 0 .. N-2 of two groups (one F2 per member) per thread.
-template <int M>
-constexpr size_t kHistOffset = (tile_smem_bytes<Cfg<M>::kTile, Cfg<M>::kStages>(8) + 15) & ~size_t(15);
-template <int N, int M>
-constexpr size_t kHistBytes = M == 8 ? size_t(N - 1) * M * Cfg<M>::kThreads * sizeof(F2) : 0;
+template <int N, int M, bool AUX>
+constexpr size_t kHistOffset = (tile_smem_bytes<Cfg<N, M, AUX>::kTile, Cfg<N, M, AUX>::kStages>(8) + 15) & ~size_t(15);
+template <int N, int M, bool AUX>
+constexpr size_t kHistBytes = M == 8 ? size_t(N - 1) * M * Cfg<N, M, AUX>::kThreads * sizeof(F2) : 0;
 // Fused optimizer with the step history in shared memory (M = 8): each thread's
 // AdamW moments (two groups, m and v) are staged behind the history by per-thread
 // async copies issued when the groups start, so their latency hides behind the
 // relaxation without holding registers.
 template <int N, int M>
-constexpr size_t kMomOffset = (kHistOffset<M> + kHistBytes<N, M> + 15) & ~size_t(15);
-template <int M>
-constexpr size_t kMomBytes = size_t(2) * M * 2 * sizeof(float) * Cfg<M>::kThreads;
+constexpr size_t kMomOffset = (kHistOffset<N, M, true> + kHistBytes<N, M, true> + 15) & ~size_t(15);
+template <int N, int M>
+constexpr size_t kMomBytes = size_t(2) * M * 2 * sizeof(float) * Cfg<N, M, true>::kThreads;
 // The deferred queues behind everything else.
-template <int N, int M, bool OPT>
+template <int N, int M, bool ST, bool OPT>
 constexpr size_t kDeferOffset =
-    (kHistBytes<N, M> == 0 ? tile_smem_bytes<Cfg<M>::kTile, Cfg<M>::kStages>(8) + 15
-     : OPT                 ? kMomOffset<N, M> + kMomBytes<M> + 15
-                           : kHistOffset<M> + kHistBytes<N, M> + 15) & ~size_t(15);
-template <int N, int M, bool OPT>
-constexpr size_t kBwdSmem = kDeferOffset<N, M, OPT> + size_t(Cfg<M>::kDeferCap) * 8 * (Cfg<M>::kThreads / 32);
+    (M == 4 ? tile_smem_bytes<Cfg<N, M, ST || OPT>::kTile, Cfg<N, M, ST || OPT>::kStages>(8) + 15
+     : OPT  ? kMomOffset<N, M> + kMomBytes<N, M> + 15
+            : kHistOffset<N, M, ST || OPT> + kHistBytes<N, M, ST || OPT> + 15) & ~size_t(15);
+template <int N, int M, bool ST, bool OPT>
+constexpr size_t kBwdSmem = kDeferOffset<N, M, ST, OPT> +
+                            size_t(Cfg<N, M, ST || OPT>::kDeferCap) * 8 * (Cfg<N, M, ST || OPT>::kThreads / 32);
 // multi-tensor launches: the tensors' first tiles behind the queues
-template <int N, int M, bool OPT>
-constexpr size_t kBwdMultiOffset = (kBwdSmem<N, M, OPT> + 15) & ~size_t(15);
-template <int N, int M, bool OPT>
-constexpr size_t kBwdMultiSmem = kBwdMultiOffset<N, M, OPT> + size_t(kMultiMaxBwd + 1) * 8;
+template <int N, int M, bool ST, bool OPT>
+constexpr size_t kBwdMultiOffset = (kBwdSmem<N, M, ST, OPT> + 15) & ~size_t(15);
+template <int N, int M, bool ST, bool OPT>
+constexpr size_t kBwdMultiSmem = kBwdMultiOffset<N, M, ST, OPT> + size_t(kMultiMaxBwd + 1) * 8;
 
 // This thread's moment slot (M = 8 fused optimizer) in the dynamic shared memory.
 extern __shared__ __align__(128) uint8_t roi_bwd_smem[];
@@ -237,7 +244,7 @@ __device__ __forceinline__ uint32_t bwd_groups(const float* const* phi_g, const 
   // (M = 4) or into this thread's shared-memory slot `mom` (with HIST)
   constexpr bool kPrefetchMoments = OPT && !HIST;
   constexpr bool kStageMoments = OPT && HIST;
-  constexpr int kT = Cfg<M>::kThreads;
+  constexpr int kT = Cfg<N, M, ST || OPT>::kThreads;
   if constexpr (kStageMoments) {
     float4* mom = moment_slot<N, M>();
 #pragma unroll
@@ -260,7 +267,7 @@ __device__ __forceinline__ uint32_t bwd_groups(const float* const* phi_g, const 
         mom_v[h][s] = reinterpret_cast<const float4*>(o.v + e0[h])[s];
       }
   }
-  using Steps = typename std::conditional<HIST, SmemSteps<N, M, V, Cfg<M>::kThreads>, RegSteps<N, M, V>>::type;
+  using Steps = typename std::conditional<HIST, SmemSteps<N, M, V, Cfg<N, M, ST || OPT>::kThreads>, RegSteps<N, M, V>>::type;
   FastGroup<N, M, TAU1, true, V, Steps, WIDE> fg;
   if constexpr (HIST) fg.st.at = hist;
   V kap[HIST ? 1 : M], c[M], dkv[M];
@@ -438,7 +445,7 @@ template <int N, int M, bool TAU1, bool ST, bool OPT, bool NARROW, bool WIDE, cl
 __device__ __forceinline__ void bwd_tile(const uint8_t* const* stage, int64_t tile, const BwdArgs& a,
                                          const BwdOptArgs& o, uint8_t* smem, Defer& dg, int64_t tag,
                                          const Exact& exact) {
-  using C = Cfg<M>;
+  using C = Cfg<N, M, ST || OPT>;
   const float* sphi = reinterpret_cast<const float*>(stage[0]);
   const uint16_t* sW = reinterpret_cast<const uint16_t*>(stage[1]);
   const uint16_t* sdW = reinterpret_cast<const uint16_t*>(stage[2]);
@@ -459,7 +466,7 @@ __device__ __forceinline__ void bwd_tile(const uint8_t* const* stage, int64_t ti
     } else {
       // M = 8: the paired step history does not fit the register file; steps
       // 0 .. N-2 go to shared memory behind the tile ring
-      F2* hist = reinterpret_cast<F2*>(smem + kHistOffset<M>) + threadIdx.x;
+      F2* hist = reinterpret_cast<F2*>(smem + kHistOffset<N, M, ST || OPT>) + threadIdx.x;
       flag = bwd_groups<N, M, TAU1, F2, true, ST, OPT, NARROW, C::kDefer, WIDE>(pp, pw, pd, e0, q0, a, o, hist);
     }
     if constexpr (C::kDefer) {
@@ -476,7 +483,7 @@ __device__ __forceinline__ void bwd_tile(const uint8_t* const* stage, int64_t ti
 // registers.
 template <int N, int M, bool TAU1, bool ST, bool OPT, bool WIDE>
 __device__ __forceinline__ void bwd_tail(const BwdArgs& a, const BwdOptArgs& o, int64_t chunk0, int64_t step) {
-  using C = Cfg<M>;
+  using C = Cfg<N, M, ST || OPT>;
   const int64_t t0 = a.full_tiles * C::kTile;
   const int64_t tail_groups = (a.E - t0) / M;
   for (int64_t g0 = chunk0 * C::kTailChunk; g0 < tail_groups; g0 += step * C::kTailChunk) {
@@ -508,13 +515,14 @@ __device__ __forceinline__ void bwd_tail(const BwdArgs& a, const BwdOptArgs& o, 
 // ST: straight-through dW from the forward's hard bits; OPT: fused AdamW step on
 // the logits (separate instantiations, so the plain kernel's code is not touched)
 // NARROW_ONLY: launched only for calls whose counters are all below 2^32 (32-bit
-// counters): every M = 4 variant, and the 4:8 tau = 1 backward fused with AdamW (at
+// counters): every N = 2 variant, and the 4:8 tau = 1 backward fused with AdamW (at
 // 4:8 the narrow plain backward spilled, 225 against 192 us per 18944 x 3584
 // tensor, while the fused one gained, 386 against 418 us)
 template <int N, int M, bool TAU1, bool ST, bool OPT, bool NARROW_ONLY, bool WIDE>
-__global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks) roi_bwd_kernel(BwdArgs a, BwdOptArgs o) {
+__global__ void __launch_bounds__(Cfg<N, M, ST || OPT>::kThreads, Cfg<N, M, ST || OPT>::kMinBlocks)
+    roi_bwd_kernel(BwdArgs a, BwdOptArgs o) {
   uint8_t* smem = roi_bwd_smem;
-  using C = Cfg<M>;
+  using C = Cfg<N, M, ST || OPT>;
   TileSrc<3> src;
   src.ptr[0] = reinterpret_cast<const uint8_t*>(a.phi);
   src.esize[0] = 4;
@@ -523,7 +531,7 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks) roi_bwd_
   src.ptr[2] = reinterpret_cast<const uint8_t*>(a.dWm);
   src.esize[2] = 2;
   DeferredGroups<C::kDeferCap> dg;
-  dg.init(smem + kDeferOffset<N, M, OPT>);
+  dg.init(smem + kDeferOffset<N, M, ST, OPT>);
   const auto exact = [&](int64_t g0) { bwd_exact_group<N, M, ST, OPT>(g0, a, o); };
   // a batch's next tensor may start on the SMs this launch frees (no-op otherwise)
   pdl_begin(a.wait);
@@ -568,7 +576,7 @@ struct BwdMulti {
   BwdItem it[kMultiMaxBwd];
 };
 static_assert(sizeof(BwdMulti) <= 32764, "kernel parameter block");
-template <int M>
+template <int N, int M, bool AUX>
 __device__ __forceinline__ BwdArgs multi_args(const BwdMulti& mm, int i) {
   const BwdItem& x = mm.it[i];
   BwdArgs a;
@@ -579,7 +587,7 @@ __device__ __forceinline__ BwdArgs multi_args(const BwdMulti& mm, int i) {
   a.dW = x.dW;
   a.hard_in = x.hard_in;
   a.E = x.E;
-  a.full_tiles = x.E / Cfg<M>::kTile;
+  a.full_tiles = x.E / Cfg<N, M, AUX>::kTile;
   a.tau = mm.tau;
   a.inv_tau = mm.inv_tau;
   a.np = x.np;
@@ -598,13 +606,13 @@ __device__ __forceinline__ BwdOptArgs multi_opt(const BwdMulti& mm, int i) {
 // roi_bwd_kernel over many small tensors at once, walked as roi_fwd_multi_kernel
 // walks them.
 template <int N, int M, bool TAU1, bool ST, bool OPT, bool NARROW_ONLY, bool WIDE>
-__global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
+__global__ void __launch_bounds__(Cfg<N, M, ST || OPT>::kThreads, Cfg<N, M, ST || OPT>::kMinBlocks)
     roi_bwd_multi_kernel(const __grid_constant__ BwdMulti mm) {
   uint8_t* smem = roi_bwd_smem;
-  using C = Cfg<M>;
+  using C = Cfg<N, M, ST || OPT>;
   const uint32_t esize[3] = {4, 2, 2};
   constexpr int64_t kLow = (int64_t(1) << 48) - 1;
-  int64_t* tile0 = reinterpret_cast<int64_t*>(smem + kBwdMultiOffset<N, M, OPT>);
+  int64_t* tile0 = reinterpret_cast<int64_t*>(smem + kBwdMultiOffset<N, M, ST, OPT>);
   for (int i = threadIdx.x; i <= mm.count; i += C::kThreads) tile0[i] = i < mm.count ? mm.it[i].tile0 : mm.total_tiles;
   __syncthreads();
   const auto find = [&](int64_t t) {
@@ -620,10 +628,10 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
     return lo;
   };
   DeferredGroups<C::kDeferCap> dg;
-  dg.init(smem + kDeferOffset<N, M, OPT>);
+  dg.init(smem + kDeferOffset<N, M, ST, OPT>);
   const auto exact = [&](int64_t e) {
     const int i = int(e >> 48);
-    bwd_exact_group<N, M, ST, OPT>(e & kLow, multi_args<M>(mm, i), multi_opt(mm, i));
+    bwd_exact_group<N, M, ST, OPT>(e & kLow, multi_args<N, M, ST || OPT>(mm, i), multi_opt(mm, i));
   };
   int cur = -1, src_cur = -1;
   int64_t lo = 0, hi = 0, src_lo = 0, src_hi = 0;
@@ -649,7 +657,7 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
           cur = find(t);
           lo = tile0[cur];
           hi = tile0[cur + 1];
-          a = multi_args<M>(mm, cur);
+          a = multi_args<N, M, ST || OPT>(mm, cur);
           o = multi_opt(mm, cur);
         }
         bwd_tile<N, M, TAU1, ST, OPT, NARROW_ONLY, WIDE>(stage, t - lo, a, o, smem, dg, int64_t(cur) << 48, exact);
@@ -661,7 +669,7 @@ __global__ void __launch_bounds__(Cfg<M>::kThreads, Cfg<M>::kMinBlocks)
   if (ok) {
     for (int64_t c = tail_rank(mm.total_tiles); c < mm.total_tails; c += gridDim.x) {
       const int i = tail_item(mm, c);
-      bwd_tail<N, M, TAU1, ST, OPT, WIDE>(multi_args<M>(mm, i), multi_opt(mm, i), c - mm.it[i].tail0, mm.total_tails);
+      bwd_tail<N, M, TAU1, ST, OPT, WIDE>(multi_args<N, M, ST || OPT>(mm, i), multi_opt(mm, i), c - mm.it[i].tail0, mm.total_tails);
     }
   }
   if (blockIdx.x == 0) pdl_wait();
@@ -673,10 +681,10 @@ struct LaunchCache {
 
 template <int N, int M, bool TAU1, bool ST, bool OPT, bool NARROW_ONLY, bool WIDE>
 int launch_tiles(const BwdArgs& a, const BwdOptArgs& o, cudaStream_t stream, bool pdl = false) {
-  using C = Cfg<M>;
+  using C = Cfg<N, M, ST || OPT>;
   auto kern = roi_bwd_kernel<N, M, TAU1, ST, OPT, NARROW_ONLY, WIDE>;
-  const size_t smem = kBwdSmem<N, M, OPT>;
-  static_assert(kBwdSmem<N, M, OPT> <= 232448, "shared memory per CTA");
+  const size_t smem = kBwdSmem<N, M, ST, OPT>;
+  static_assert(kBwdSmem<N, M, ST, OPT> <= 232448, "shared memory per CTA");
   static LaunchCache cache;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
@@ -689,6 +697,7 @@ int launch_tiles(const BwdArgs& a, const BwdOptArgs& o, cudaStream_t stream, boo
   }
   const int64_t cap = int64_t(sm_count()) * cache.per_sm[dev];
   BwdArgs b = a;
+  b.full_tiles = a.E / C::kTile;
   b.wait = !pdl && lone_pdl(stream);
   const int grid = tile_grid(b.full_tiles, a.E, M, C::kTailChunk, C::kTile, cap, pdl ? 0 : C::kTailRounds);
   return launch_maybe_pdl(kern, grid, C::kThreads, smem, stream, pdl || b.wait, b, o);
@@ -709,7 +718,7 @@ int launch_nm(const BwdArgs& a, const BwdOptArgs& o, cudaStream_t stream, bool p
     if (a.tau == 1.0f && a.np.narrow && o.phi_out != nullptr)
       return launch_tiles<N, M, true, false, true, true, false>(a, o, stream, pdl);
   }
-  if constexpr (M == 4) {
+  if constexpr (kNarrowKernels<N, M>) {
     if (a.np.narrow) {
       if (o.phi_out != nullptr) return launch_tau<N, M, false, true, true>(a, o, stream, pdl);
       if (a.hard_in != nullptr && a.dW != nullptr) return launch_tau<N, M, true, false, true>(a, o, stream, pdl);
@@ -723,9 +732,9 @@ int launch_nm(const BwdArgs& a, const BwdOptArgs& o, cudaStream_t stream, bool p
 
 template <int N, int M, bool TAU1, bool ST, bool OPT, bool NARROW_ONLY, bool WIDE>
 int launch_multi_kern(const BwdMulti& mm, cudaStream_t stream, bool pdl) {
-  using C = Cfg<M>;
+  using C = Cfg<N, M, ST || OPT>;
   auto kern = roi_bwd_multi_kernel<N, M, TAU1, ST, OPT, NARROW_ONLY, WIDE>;
-  constexpr size_t smem = kBwdMultiSmem<N, M, OPT>;
+  constexpr size_t smem = kBwdMultiSmem<N, M, ST, OPT>;
   static_assert(smem <= 232448, "shared memory per CTA");
   static LaunchCache cache;
   int dev = 0;
@@ -761,7 +770,9 @@ int bwd_kind(const BwdCall& c) { return c.phi_out != nullptr ? 2 : (c.hard_in !=
 // choice of variant.
 template <int N, int M>
 int launch_multi(const BwdCall* calls, int count, bool pdl) {
-  using C = Cfg<M>;
+  const int kind = bwd_kind(calls[0]);
+  const int64_t tile = kind != 0 ? Cfg<N, M, true>::kTile : Cfg<N, M, false>::kTile;
+  const int64_t chunk = kind != 0 ? Cfg<N, M, true>::kTailChunk : Cfg<N, M, false>::kTailChunk;
   static thread_local BwdMulti mm;
   mm.count = count;
   mm.tau = calls[0].tau;
@@ -785,21 +796,20 @@ int launch_multi(const BwdCall* calls, int count, bool pdl) {
     x.tile0 = tiles;
     x.np = c.np;
     x.np.narrow = counters_narrow(c.np, c.E);
-    tiles += c.E / C::kTile;
+    tiles += c.E / tile;
     x.tail0 = tails;
-    tails += (c.E % C::kTile / M + C::kTailChunk - 1) / C::kTailChunk;
+    tails += (c.E % tile / M + chunk - 1) / chunk;
   }
   mm.total_tiles = tiles;
   mm.total_tails = tails;
   const cudaStream_t stream = calls[0].stream;
   mm.wait = !pdl && lone_pdl(stream);
-  const int kind = bwd_kind(calls[0]);
   const bool narrow = mm.it[0].np.narrow;
   if constexpr (N == 4 && M == 8) {
     if (mm.tau == 1.0f && narrow && kind == 2)
       return launch_multi_kern<N, M, true, false, true, true, false>(mm, stream, pdl);
   }
-  if constexpr (M == 4) {
+  if constexpr (kNarrowKernels<N, M>) {
     if (narrow) {
       if (kind == 2) return launch_multi_tau<N, M, false, true, true>(mm, stream, pdl);
       if (kind == 1) return launch_multi_tau<N, M, true, false, true>(mm, stream, pdl);
@@ -828,7 +838,7 @@ int launch_bwd_impl(const BwdCall& c, bool pdl) {
   o.v = c.v;
   o.opt = c.opt;
   a.E = c.E;
-  a.full_tiles = c.E / (c.M == 8 ? Cfg<8>::kTile : Cfg<4>::kTile);
+  a.full_tiles = 0;  // launch_tiles
   a.tau = c.tau;
   a.inv_tau = 1.0f / c.tau;
   a.np = c.np;
@@ -855,8 +865,11 @@ int launch_bwd_batch(const BwdCall* calls, int count) {
     const BwdCall& c = calls[i];
     if ((c.N == 2 && c.M == 4) || (c.N == 4 && c.M == 8) || (c.N == 2 && c.M == 8)) {
       // the run of small items from i on with the same tile kernel
-      const int64_t tile = c.M == 8 ? Cfg<8>::kTile : Cfg<4>::kTile;
       const int kind = bwd_kind(c);
+      const int64_t tile = c.M == 4   ? Cfg<2, 4, false>::kTile
+                           : c.N == 4 ? Cfg<4, 8, false>::kTile
+                           : kind != 0 ? Cfg<2, 8, true>::kTile
+                                       : Cfg<2, 8, false>::kTile;
       const bool narrow = counters_narrow(c.np, c.E);
       int n = 0;
       while (i + n < count && n < kMultiMaxBwd && calls[i + n].N == c.N && calls[i + n].M == c.M &&
