@@ -491,7 +491,7 @@ __device__ __forceinline__ void bwd_tail(const BwdArgs& a, const BwdOptArgs& o, 
       // the chunk's halves go to the two lanes; a missing second group doubles the first
       const int64_t n = tail_groups - g0 < C::kTailChunk ? tail_groups - g0 : C::kTailChunk;
       const int half = tail_half<M>(n);
-      if (threadIdx.x >= half) continue;
+      if (threadIdx.x >= half || threadIdx.x >= n) continue;
       const bool two = threadIdx.x + half < n;
       const int64_t ea = t0 + (g0 + threadIdx.x) * M;
       const int64_t eb = two ? ea + int64_t(half) * M : ea;

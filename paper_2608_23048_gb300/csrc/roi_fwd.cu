@@ -339,7 +339,7 @@ __device__ __forceinline__ void fwd_tail(const FwdArgs& a, int64_t chunk0, int64
       // the chunk's halves go to the two lanes; a missing second group doubles the first
       const int64_t n = tail_groups - g0 < C::kTailChunk ? tail_groups - g0 : C::kTailChunk;
       const int half = tail_half<M>(n);
-      const bool active = threadIdx.x < half, two = threadIdx.x + half < n;
+      const bool active = threadIdx.x < half && threadIdx.x < n, two = threadIdx.x + half < n;
       const int64_t ea = t0 + (g0 + (active ? threadIdx.x : 0)) * M;
       const int64_t eb = two ? ea + int64_t(half) * M : ea;
       uint32_t bits[2] = {0u, 0u};

@@ -126,7 +126,8 @@ __device__ __forceinline__ int64_t tail_rank(int64_t tiles) {
   return blockIdx.x >= r ? blockIdx.x - r : blockIdx.x + gridDim.x - r;
 }
 // How a chunk of n groups is split between the two lanes of the packed code: the first
-// `half` threads take groups t and t + half (whole hard-mask words in either half).
+// `half` threads take groups t and t + half (whole hard-mask words in either half; with
+// fewer groups than a word holds, half exceeds n).
 template <int M>
 __device__ __forceinline__ int tail_half(int64_t n) {
   constexpr int kPerWord = 32 / M;

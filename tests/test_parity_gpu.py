@@ -331,6 +331,38 @@ def test_small_tensors_equal_slices(roi, N, M, tau, rows):
                          max(0, rows - 2))
 
 
+# Outputs end where the tensor does: every buffer carries a margin whose contents must
+# survive, at sizes whose last chunk holds a few groups only (one to a hard word's worth and
+# one more) alone, behind whole chunks and behind whole tiles.
+@pytest.mark.parametrize("N,M", [(2, 4), (4, 8), (2, 8), (8, 16), (16, 32), (1, 4), (3, 7)])
+@pytest.mark.parametrize("base", [0, 12288 * 3, 4096 * 5])
+@pytest.mark.parametrize("groups", [1, 3, 5, 7, 8, 9, 17])
+def test_nothing_written_past_the_tensor(roi, N, M, base, groups):
+    import torch
+    cols = (base // M + groups) * M
+    pad = 4096
+    phi = torch.randn(cols + pad, device="cuda")
+    W, dWm = ((torch.randn(cols + pad, device="cuda") * s).to(torch.bfloat16) for s in (0.02, 1e-3))
+    f32 = lambda: torch.full((cols + pad,), 7.0, device="cuda")  # noqa: E731
+    b16 = lambda: torch.full((cols + pad,), 7.0, dtype=torch.bfloat16, device="cuda")  # noqa: E731
+    soft, dphi, m, v, Wm, dW = f32(), f32(), f32(), f32(), b16(), b16()
+    words = roi.hard_words(1, cols)
+    hard = torch.full((words + pad,), 7, dtype=torch.int32, device="cuda")
+    cut = lambda t: t[:cols].view(1, cols)  # noqa: E731
+    st, tau = roi.NoiseState(3, 1, 2, 1.0, 0), 0.5
+    before = phi.clone()
+    roi.roi_mask_fwd_ex(cut(phi), cut(W), N, M, tau, st, cut(Wm), cut(soft), hard[:words])
+    roi.roi_mask_bwd(cut(phi), cut(W), st, N, M, cut(dWm), tau, cut(dphi), cut(dW))
+    opt = roi.AdamW(1e-3, 0.9, 0.95, 1e-8, 0.05, 3)
+    roi.roi_mask_bwd_adamw(cut(phi), cut(W), st, N, M, cut(dWm), tau, cut(m), cut(v), opt)
+    roi.roi_device_status()
+    for t in (soft, dphi, m, v, Wm, dW):
+        assert torch.all(t[cols:] == 7)
+        assert not torch.any(t[:cols] == 7)
+    assert torch.all(hard[words:] == 7) and torch.equal(phi[cols:], before[cols:])
+    assert torch.equal(soft[:cols].view(-1, M).sum(1).round(), torch.full((cols // M,), float(N), device="cuda"))
+
+
 # Patterns without a kernel of their own: every padded width, M that divides a hard word
 # (assembled by shuffles) and M that does not, group counts that leave a lane of the last
 # pair empty, N = 1, the largest N, small tau lambda.
