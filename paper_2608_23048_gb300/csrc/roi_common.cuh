@@ -22,9 +22,9 @@ namespace roi {
 // ---------------------------------------------------------------------------
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
-// Exclusive sums below this value mean all other members of a group are more
-// than ~69 natural-log units below the top key: exp() of them no longer fits the
-// fast path's float range and the group is recomputed by the exact routine.
+// The tau = 1 slice kernels' range: members whose weights relative to the group's first
+// key lie outside [2^-100, 2^100] (~69 natural-log units) send the group to the exact
+// routine.
 constexpr float kTinyExcl = 7.888609052210118e-31f;  // 2^-100
 
 // FastGroup's WIDE relaxation: the largest lead of a group's first member over its second,
@@ -823,10 +823,11 @@ struct DeferredGroups {
 // S to within fp32 rounding (packed products may be fused into FMAs by the
 // compiler, see roi_vec.cuh).  The fallback decision depends only on sums of
 // exp2 outputs and is therefore the same in both kernels.
-// `flag` (one bit per lane) is raised when a key is not finite and, depending on
-// tau, when a key lies more than 100 log2 units from the first one (tau = 1) or
-// an exclusive sum drops below 2^-100 (a key gap of ~69 natural-log units); the
-// caller then recomputes that group with ExactGroup (and re-ranks it with the
+// `flag` (one bit per lane) is raised when a key is not finite (or beyond 2^63) and,
+// for finite keys, when one lies more than 100 log2 units from the first (tau = 1) or
+// two consecutive steps' totals leave the range of kLeastRange (tau != 1; the WIDE
+// variant below has no such range); the caller then recomputes that group with
+// RobustGroup or ExactGroup (and re-ranks one with non-finite keys with the
 // comparison-based top-N, which orders NaN as -inf).
 // ---------------------------------------------------------------------------
 template <int M, class V>

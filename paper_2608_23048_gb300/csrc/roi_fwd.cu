@@ -50,21 +50,6 @@ struct FwdArgs {
   bool wait;  // pdl_begin
 };
 
-template <int M>
-__device__ __forceinline__ void load_group(const float* phi_g, const uint16_t* W_g, float (&ph)[M],
-                                           float (&w)[M]) {
-#pragma unroll
-  for (int s = 0; s < M / 4; ++s) {
-    const float4 p = reinterpret_cast<const float4*>(phi_g)[s];
-    ph[4 * s] = p.x, ph[4 * s + 1] = p.y, ph[4 * s + 2] = p.z, ph[4 * s + 3] = p.w;
-    const uint2 q = reinterpret_cast<const uint2*>(W_g)[s];
-    w[4 * s + 0] = bf16_bits_to_float(q.x & 0xffffu);
-    w[4 * s + 1] = bf16_bits_to_float(q.x >> 16);
-    w[4 * s + 2] = bf16_bits_to_float(q.y & 0xffffu);
-    w[4 * s + 3] = bf16_bits_to_float(q.y >> 16);
-  }
-}
-
 // Perturbed keys of L groups (one per lane of V), in log2 units
 // (t = (phi / lambda + g) log2 e), whose first elements have call-flat indices
 // e0[h]; ph[h] holds each group's logits.  NARROW: the call's counters are below

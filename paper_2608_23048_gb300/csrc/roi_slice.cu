@@ -1,9 +1,12 @@
 // Wide groups (M = 16, 32: the 8:16 and 16:32 patterns) on warp slices: the
-// SL = M / P consecutive lanes of a slice hold one group, P = 8 or 16 members each, as
-// packed pairs of neighbouring members (F2).  Same method as the one-thread-per-group
+// SL = M / P consecutive lanes of a slice hold one group, P = 16 members each (8:16: one
+// lane, 16:32: two), as packed pairs of neighbouring members (F2).  Each shuffle and tree
+// addition then covers more members than with fewer a lane (tau = 0.2, forward + backward
+// of 3B-shaped blocks, two at 8:16 and one at 16:32: P = 4 2119 and 2502 us, P = 8 1845
+// and 2024, P = 16 1669 and 1684).  Same method as the one-thread-per-group
 // kernels (Sec. 4.2.2 Eq. 10-12, Algorithm 1; Eq. 5; backward through the relaxation),
 // with the per-group sums and "sum of the other members" formed in the thread and then
-// across the slice's lanes by a shuffle butterfly that never subtracts.  The step loops
+// across the slice's lanes by a shuffle that never subtracts.  The step loops
 // are rolled: the history of the relaxation that the backward sweeps is indexed in shared
 // memory.  Groups whose keys leave the fast path's range are queued by the slice's first
 // lane (DeferredGroups) and handled 32 at a time, one per lane, by WideRobustGroup
@@ -468,17 +471,17 @@ __device__ __forceinline__ void bitonic_desc(float (&x)[P], int at) {
 }
 
 // Hard bits of a lane's members for N = M / 2 (the two patterns of these kernels) from the
-// group's N-th largest key: each half of the group is sorted, in the lane and (P = 8,
-// M = 32) by a bitonic merge across lane pairs (the partner's keys in reverse, the larger
-// half to the lower lane); the top M / 2 of the group are then the larger elements of the
-// pairs (i-th of the first half, i-th from the end of the second), so their minimum is the
-// threshold.  A member is kept iff its key reaches it.  Returns false (bits unusable) if
+// group's N-th largest key: each half of the group is sorted (8:16: both in the lane,
+// 16:32: one per lane of the slice); the top M / 2 of the group are then the larger
+// elements of the pairs (i-th of the first half, i-th from the end of the second), so
+// their minimum is the threshold.  A member is kept iff its key reaches it.  Returns false (bits unusable) if
 // the slice's keys are not all finite or the threshold is tied, so that more than N
 // members pass: the caller ranks such groups by comparison.
 template <int N, int M, int P>
-__device__ __forceinline__ bool slice_topn_threshold(const float (&kap)[P], int q, uint32_t& bits) {
+__device__ __forceinline__ bool slice_topn_threshold(const float (&kap)[P], uint32_t& bits) {
   static_assert(2 * N == M, "threshold selection needs N = M / 2");
   constexpr int SL = M / P;
+  static_assert(P == 16 && SL <= 2, "two runs of eight a lane, at most two lanes a group");
   float x[P];
 #pragma unroll
   for (int i = 0; i < P; ++i) x[i] = kap[i];
@@ -486,30 +489,16 @@ __device__ __forceinline__ bool slice_topn_threshold(const float (&kap)[P], int 
   for (int i = 0; i < P; i += 8) sort8_desc(x, i);
   float m = INFINITY;
   if constexpr (SL == 1) {
-    static_assert(SL != 1 || P == 16, "one lane a group: 16 members");
 #pragma unroll
     for (int i = 0; i < P / 2; ++i) m = fminf(m, fmaxf(x[i], x[P - 1 - i]));
   } else {
-    if constexpr (P == 16) {
-      // the lane's two sorted runs into one
+    // the lane's two sorted runs into one
 #pragma unroll
-      for (int i = 0; i < 8; ++i) ce_desc(x, i, 15 - i);
-      bitonic_desc<8>(x, 0);
-      bitonic_desc<8>(x, 8);
-    }
-    if constexpr (SL == 4) {
-      float p[P];
+    for (int i = 0; i < 8; ++i) ce_desc(x, i, 15 - i);
+    bitonic_desc<8>(x, 0);
+    bitonic_desc<8>(x, 8);
 #pragma unroll
-      for (int i = 0; i < P; ++i) p[i] = shfl_xor(x[P - 1 - i], 1);
-      const bool upper = (q & 1) != 0;
-#pragma unroll
-      for (int i = 0; i < P; ++i) x[i] = upper ? fminf(x[i], p[i]) : fmaxf(x[i], p[i]);
-      bitonic_desc<P>(x, 0);
-    }
-#pragma unroll
-    for (int i = 0; i < P; ++i) m = fminf(m, fmaxf(x[i], shfl_xor(x[P - 1 - i], SL - 1)));
-#pragma unroll
-    for (int o = 1; o < SL / 2; o <<= 1) m = fminf(m, shfl_xor(m, o));
+    for (int i = 0; i < P; ++i) m = fminf(m, fmaxf(x[i], shfl_xor(x[P - 1 - i], 1)));
   }
   bits = 0;
   float fin = 0.0f;
@@ -533,7 +522,7 @@ __device__ __forceinline__ uint32_t lane_topn(const F2 (&kap)[H], int base_lane,
 #pragma unroll
   for (int i = 0; i < H; ++i) k[2 * i] = lo(kap[i]), k[2 * i + 1] = hi(kap[i]);
   uint32_t bits;
-  const bool ok = slice_topn_threshold<N, M>(k, q, bits);
+  const bool ok = slice_topn_threshold<N, M>(k, bits);
   if (__any_sync(0xffffffffu, !ok)) {
     const uint32_t b = slice_topn_bits<M>(k, N, base_lane, q);
     if (!ok) bits = b;
@@ -554,8 +543,8 @@ __device__ __forceinline__ void group_keys_all(const float* phi_g, int64_t g0, c
   }
 }
 // The exact relaxation of one group with keys t (log2 units): WideRobustGroup for finite
-// keys (which never come here from a WIDE kernel), ExactGroup (natural-log keys) otherwise; soft mask S and, with c,
-// dk = dL/dkappa.
+// keys (which never come here from a WIDE kernel), ExactGroup (natural-log keys) otherwise;
+// soft mask S and, with c, dk = dL/dkappa.
 template <int N, int M, bool BWD, bool WIDE>
 __device__ __forceinline__ void exact_relax(float (&t)[M], const float (&c)[M], const SliceArgs& a, float (&S)[M],
                                             float (&dk)[M]) {
