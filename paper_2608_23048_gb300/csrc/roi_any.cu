@@ -4,7 +4,8 @@
 // 8, 16 or 32 members whose keys lie far below every real one: two groups in lockstep on
 // packed FP32 for MP <= 8, one for the wider ones.  The relaxation is FastGroup's WIDE one
 // (finite keys never leave its range) with the step loop rolled, and the backward keeps
-// the steps' weights in thread-local memory.  Non-finite keys go to ExactGroup in place.
+// the steps' weights in thread-local memory.  Non-finite keys, and every group at a
+// tau too small for WIDE (wide_holds), go to ExactGroup in place.
 #include "roi_launch.h"
 
 namespace roi {
@@ -35,6 +36,7 @@ struct AnyArgs {
   int N, M;
   float tau, inv_tau;
   NoiseParams np;
+  float max_sq;  // groups with a larger sum of squared keys go to ExactGroup (all if negative)
   bool wait;  // pdl_begin
 };
 
@@ -158,15 +160,15 @@ __device__ __forceinline__ V total_of(const V (&x)[MP]) {
 }
 
 // FastGroup's WIDE forward with N steps at run time; step(k, mu) sees every step's weights.
-// Returns the lanes' flags (a non-finite key, or one beyond the fast relaxation's range).
+// Returns the lanes' flags (a non-finite key, or keys beyond max_sq).
 template <int MP, class V, class Step>
-__device__ __forceinline__ uint32_t any_relax(const V (&kap)[MP], int N, int M, float inv_tau, Step&& step) {
+__device__ __forceinline__ uint32_t any_relax(const V (&kap)[MP], int N, int M, float inv_tau, float max_sq, Step&& step) {
   const V itau = vconst<V>(inv_tau);
   V sq = vmul(kap[0], kap[0]);
 #pragma unroll
   for (int l = 1; l < MP; ++l)
     if (l < M) sq = vfma(kap[l], kap[l], sq);
-  const uint32_t flag = vbelow(vsub(vconst<V>(kMaxKeySq), sq), 0.0f);
+  const uint32_t flag = vbelow(vsub(vconst<V>(max_sq), sq), 0.0f);
   V x[MP];
   V ref = second_of(kap);
 #pragma unroll
@@ -225,7 +227,7 @@ __global__ void __launch_bounds__(kThreads) roi_any_fwd_kernel(AnyArgs a, bool w
       any_keys<MP, V>(a, e0, kap);
 #pragma unroll
       for (int l = 0; l < MP; ++l) S[l] = vconst<V>(0.0f);
-      const uint32_t flag = any_relax<MP, V>(kap, a.N, a.M, a.inv_tau, [&](int, const V (&mu)[MP]) {
+      const uint32_t flag = any_relax<MP, V>(kap, a.N, a.M, a.inv_tau, a.max_sq, [&](int, const V (&mu)[MP]) {
 #pragma unroll
         for (int l = 0; l < MP; ++l) S[l] = vadd(S[l], mu[l]);
       });
@@ -320,7 +322,7 @@ __global__ void __launch_bounds__(kThreads) roi_any_bwd_kernel(AnyArgs a) {
     V hist[MP - 1][MP];  // mu of every step
     V kap[MP], c[MP], b[MP];
     any_keys<MP, V>(a, e0, kap);
-    const uint32_t flag = any_relax<MP, V>(kap, a.N, a.M, a.inv_tau, [&](int k, const V (&mu)[MP]) {
+    const uint32_t flag = any_relax<MP, V>(kap, a.N, a.M, a.inv_tau, a.max_sq, [&](int k, const V (&mu)[MP]) {
 #pragma unroll
       for (int l = 0; l < MP; ++l) hist[k][l] = mu[l];
     });
@@ -454,6 +456,7 @@ int launch_any_fwd(const FwdCall& c) {
   a.tau = c.tau;
   a.inv_tau = 1.0f / c.tau;
   a.np = c.np;
+  a.max_sq = wide_holds(c.N, c.tau) ? kMaxKeySq : -1.0f;
   const bool words = 32 % c.M == 0;
   if (c.hard != nullptr && !words) {
     // groups straddle words: assembled with atomicOr
@@ -486,6 +489,7 @@ int launch_any_bwd(const BwdCall& c) {
   a.tau = c.tau;
   a.inv_tau = 1.0f / c.tau;
   a.np = c.np;
+  a.max_sq = wide_holds(c.N, c.tau) ? kMaxKeySq : -1.0f;
   a.wait = lone_pdl(c.stream);
   int r;
   if (c.M <= 4) r = launch_maybe_pdl(roi_any_bwd_kernel<4>, any_grid(a.groups, 2), kThreads, 0, c.stream, a.wait, a);

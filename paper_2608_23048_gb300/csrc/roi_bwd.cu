@@ -844,11 +844,11 @@ int launch_bwd_impl(const BwdCall& c, bool pdl) {
   a.np = c.np;
   a.np.narrow = counters_narrow(c.np, c.E);
   a.status = c.status;
+  if (slice_supported(c.N, c.M)) return launch_slice_bwd(c, pdl);
+  if (!tile_pattern(c.N, c.M, c.tau)) return launch_any_bwd(c);
   if (c.N == 2 && c.M == 4) return launch_nm<2, 4>(a, o, c.stream, pdl);
   if (c.N == 4 && c.M == 8) return launch_nm<4, 8>(a, o, c.stream, pdl);
-  if (c.N == 2 && c.M == 8) return launch_nm<2, 8>(a, o, c.stream, pdl);
-  if (slice_supported(c.N, c.M)) return launch_slice_bwd(c, pdl);
-  return launch_any_bwd(c);
+  return launch_nm<2, 8>(a, o, c.stream, pdl);
 }
 }  // namespace
 
@@ -863,7 +863,7 @@ int launch_bwd_batch(const BwdCall* calls, int count) {
   bool prev_tiled = false;
   for (int i = 0; i < count;) {
     const BwdCall& c = calls[i];
-    if ((c.N == 2 && c.M == 4) || (c.N == 4 && c.M == 8) || (c.N == 2 && c.M == 8)) {
+    if (tile_pattern(c.N, c.M, c.tau)) {
       // the run of small items from i on with the same tile kernel
       const int kind = bwd_kind(c);
       const int64_t tile = c.M == 4   ? Cfg<2, 4, false>::kTile
@@ -899,8 +899,7 @@ int launch_bwd_batch(const BwdCall* calls, int count) {
         continue;
       }
     }
-    const bool tiled = (c.N == 2 && c.M == 4) || (c.N == 4 && c.M == 8) || (c.N == 2 && c.M == 8) ||
-                       slice_supported(c.N, c.M);
+    const bool tiled = tile_pattern(c.N, c.M, c.tau) || slice_supported(c.N, c.M);
     const int r = launch_bwd_impl(c, tiled && prev_tiled);
     if (r < 0) return -1;
     launched += r;

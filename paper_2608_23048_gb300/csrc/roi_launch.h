@@ -1,6 +1,7 @@
 // Host-side launch interface between the C ABI (roi_api.cu) and the kernels.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -25,10 +26,22 @@ inline bool counters_narrow(const NoiseParams& np, int64_t E) {
 // 69 tau is a few times 1 / lambda (986 / 349 us at tau = 0.22, lambda = 0.045, while
 // tau lambda = 0.1 still measured 336 plain).
 constexpr float kWideTau = 0.2f;
+// WIDE holds the weights of a group behind its leader's capped lead at 2^-100 or more where
+// they should vanish, and the backward multiplies such a remainder by 1 / tau once a step:
+// up to 2^-100 tau^-N of the gradient.  Below 2^-24 (N log2(1 / tau) <= 76: tau >= 4e-12 at
+// N = 2, 2e-6 at 4, 0.0014 at 8, 0.037 at 16) that is rounding; at smaller tau (8:16, tau =
+// 1e-10: 2e10 where the gradient is 0) the groups go to the log-space routines.
+constexpr float kWideBits = 76.0f;
+inline bool wide_holds(int N, float tau) { return float(N) * -log2f(tau) <= kWideBits; }
 constexpr float kWideTauLambda = 0.09f;
 template <int N>
 inline bool wide_range(float tau, const NoiseParams& np) {
-  return kAlwaysWide<N> || tau <= kWideTau || tau < kWideTauLambda * np.inv_lam;
+  return kAlwaysWide<N> || (wide_holds(N, tau) && (tau <= kWideTau || tau < kWideTauLambda * np.inv_lam));
+}
+// Patterns on the tile kernels.  2:4 and 2:8 have WIDE ones only (tau != 1); where that does
+// not hold they go to the any-(N, M) kernels.
+inline bool tile_pattern(int N, int M, float tau) {
+  return (N == 4 && M == 8) || (N == 2 && (M == 4 || M == 8) && wide_holds(N, tau));
 }
 // Whether two calls of a batch take the same relaxation (lambda is each item's own).
 inline bool same_range(int N, float tau, const NoiseParams& a, const NoiseParams& b) {

@@ -935,7 +935,9 @@ __global__ void __launch_bounds__(ShapeOf<M, BWD>::kThreads, 1) roi_slice_multi_
 }
 
 // Whether a tau != 1 call takes the WIDE relaxation.
-bool slice_wide(float tau, const NoiseParams& np) { return tau < kSliceWideTau || tau < kSliceWideTauLambda * np.inv_lam; }
+bool slice_wide(int N, float tau, const NoiseParams& np) {
+  return wide_holds(N, tau) && (tau < kSliceWideTau || tau < kSliceWideTauLambda * np.inv_lam);
+}
 
 struct LaunchCache {
   int per_sm[64] = {0};
@@ -983,12 +985,12 @@ int slice_bwd(const SliceArgs& a, cudaStream_t stream, bool pdl) {
 template <int N, int M>
 int slice_fwd_nm(const SliceArgs& a, cudaStream_t stream, bool pdl) {
   if (a.tau == 1.0f) return slice_fwd<N, M, true, false>(a, stream, pdl);
-  return slice_wide(a.tau, a.np) ? slice_fwd<N, M, false, true>(a, stream, pdl) : slice_fwd<N, M, false, false>(a, stream, pdl);
+  return slice_wide(N, a.tau, a.np) ? slice_fwd<N, M, false, true>(a, stream, pdl) : slice_fwd<N, M, false, false>(a, stream, pdl);
 }
 template <int N, int M>
 int slice_bwd_nm(const SliceArgs& a, cudaStream_t stream, bool pdl) {
   if (a.tau == 1.0f) return slice_bwd<N, M, true, false>(a, stream, pdl);
-  return slice_wide(a.tau, a.np) ? slice_bwd<N, M, false, true>(a, stream, pdl) : slice_bwd<N, M, false, false>(a, stream, pdl);
+  return slice_wide(N, a.tau, a.np) ? slice_bwd<N, M, false, true>(a, stream, pdl) : slice_bwd<N, M, false, false>(a, stream, pdl);
 }
 
 template <int N, int M, bool TAU1, bool WIDE, bool BWD>
@@ -1042,7 +1044,7 @@ int slice_run(const Call* calls, int count, int64_t tile) {
     int n = 0;
     while (n < count && n < kMultiMax && calls[n].N == calls[0].N && calls[n].M == calls[0].M &&
            calls[n].E < tiles_per_sm * tile * sm_count() &&
-           (calls[0].tau == 1.0f || slice_wide(calls[0].tau, calls[n].np) == slice_wide(calls[0].tau, calls[0].np)))
+           (calls[0].tau == 1.0f || slice_wide(calls[0].N, calls[0].tau, calls[n].np) == slice_wide(calls[0].N, calls[0].tau, calls[0].np)))
       ++n;
     return n;
   };
@@ -1075,7 +1077,7 @@ int launch_slice_multi(const Call* calls, int count, bool pdl) {
     warps += (calls[i].E / 16 + 31) / 32;
   }
   mm.total = warps;
-  const bool wide = slice_wide(c0.tau, c0.np);
+  const bool wide = slice_wide(c0.N, c0.tau, c0.np);
   if (c0.M == 16) return slice_multi_nm<8, 16, BWD>(mm, wide, c0.stream, pdl);
   return slice_multi_nm<16, 32, BWD>(mm, wide, c0.stream, pdl);
 }

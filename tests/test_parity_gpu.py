@@ -377,6 +377,20 @@ def test_patterns_without_own_kernel(roi, rows, groups, N, M, tau, lam):
     check_against_oracle(got, ph, Wb, dWb, N, M, tau, 123456789, 5, 2, lam, 3)
 
 
+# Tiny temperatures, where every group's weights saturate: no NaN, and no remainder of the
+# capped lead in the gradient (2^-24 of the incoming one at the largest; the exact gradient
+# is 0 but for near ties, which these seeds do not hold).
+@pytest.mark.parametrize("N,M", [(2, 4), (4, 8), (2, 8), (8, 16), (16, 32), (1, 4), (2, 3), (3, 5), (5, 12), (20, 24)])
+@pytest.mark.parametrize("tau", [1e-10, 1e-25])
+def test_tiny_temperatures(roi, N, M, tau):
+    W, phi, dWm, ph, Wb, dWb = make(3, 43 * M, "normal", data_seed=M + N)
+    got = gpu_run(roi, phi, W, dWm, N, M, tau, roi.NoiseState(7, 5, 2, 1.0, 3))
+    ref = O.mask_fwd(ph, Wb, N, M, tau, 7, 5, 2, 1.0, 3)
+    assert np.allclose(got["soft"], ref["soft"], atol=1e-5)
+    assert np.array_equal(got["hard_bits"], ref["hard_bits"])
+    assert np.abs(got["dlogits"]).max() <= 2.0**-24 * float((W.float() * dWm.float()).abs().max())
+
+
 # The warp-slice kernels' rule (tau = 0.1, tau lambda = 0.05); 41 rows are full tiles of
 # neither direction's shape and a ragged tail, 64 rows full tiles and a tail.
 @pytest.mark.parametrize("rows", [1, 41, 64])
