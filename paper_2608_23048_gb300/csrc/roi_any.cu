@@ -12,10 +12,13 @@ namespace roi {
 namespace {
 
 constexpr int kThreads = 128;
-// Padding members' keys (log2 units) and the magnitude up to which real keys take the fast
-// relaxation.
+// Padding members' keys (log2 units), the magnitude (squared) up to which real keys take the
+// fast relaxation, and the padding's largest offset from the second largest key over tau: 2^x
+// is 0 there whatever tau is, and second_of never picks it (a real key's offset lies above the
+// padding's by 2e18 / tau and by 1e30 - 2e18 / tau, of which one is 5e29 or more).
 constexpr float kPadKey = -3.0e18f;
 constexpr float kMaxKeySq = 1.0e36f;
+constexpr float kPadOffset = -1.0e30f;
 
 struct AnyArgs {
   const float* phi;
@@ -172,7 +175,10 @@ __device__ __forceinline__ uint32_t any_relax(const V (&kap)[MP], int N, int M, 
   V x[MP];
   V ref = second_of(kap);
 #pragma unroll
-  for (int l = 0; l < MP; ++l) x[l] = vmul(vsub(kap[l], ref), itau);
+  for (int l = 0; l < MP; ++l) {
+    x[l] = vmul(vsub(kap[l], ref), itau);
+    if (l >= MP / 2 && l >= M) x[l] = vmin(x[l], vconst<V>(kPadOffset));
+  }
 #pragma unroll 1
   for (int k = 0; k < N; ++k) {
     V c[MP], e[MP];

@@ -391,6 +391,18 @@ def test_tiny_temperatures(roi, N, M, tau):
     assert np.abs(got["dlogits"]).max() <= 2.0**-24 * float((W.float() * dWm.float()).abs().max())
 
 
+# Large temperatures (any finite tau is accepted): all weights of a group tend to 1 / M, and
+# the members that pad a group to 4, 8, 16 or 32 have none (a padding key that is divided by
+# tau like the others takes an eighth of 3:7's sum at tau = 1e20).
+@pytest.mark.parametrize("N,M", [(1, 2), (1, 3), (2, 3), (3, 7), (6, 7), (5, 12), (7, 24), (2, 4), (1, 4)])
+@pytest.mark.parametrize("tau", [1e3, 1e17, 1e20])
+def test_large_temperatures(roi, N, M, tau):
+    W, phi, dWm, ph, Wb, dWb = make(3, 43 * M, "normal", data_seed=M + N)
+    got = gpu_run(roi, phi, W, dWm, N, M, tau, roi.NoiseState(7, 5, 2, 1.0, 3))
+    check_against_oracle(got, ph, Wb, dWb, N, M, tau, 7, 5, 2, 1.0, 3)
+    assert np.allclose(got["soft"].reshape(-1, M).sum(1), N, atol=1e-5 * N)
+
+
 # The warp-slice kernels' rule (tau = 0.1, tau lambda = 0.05); 41 rows are full tiles of
 # neither direction's shape and a ragged tail, 64 rows full tiles and a tail.
 @pytest.mark.parametrize("rows", [1, 41, 64])
