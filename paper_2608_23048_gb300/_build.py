@@ -20,7 +20,7 @@ SOURCES = ["roi_api.cu", "roi_fwd.cu", "roi_bwd.cu", "roi_export.cu", "roi_noise
            "roi_any.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
-         "--expt-relaxed-constexpr", "-I", INCLUDE, "-I", CSRC]
+         "--expt-relaxed-constexpr", "-Xptxas", "-v", "-I", INCLUDE, "-I", CSRC]
 
 
 def nvcc() -> str:
@@ -30,12 +30,19 @@ def nvcc() -> str:
     raise RuntimeError("nvcc not found")
 
 
+def log_of(src: str) -> str:
+    """Path of what ptxas said of a source file (registers, stack, spills of each kernel)."""
+    return os.path.join(BUILD, src.replace(".cu", ".log"))
+
+
 def _compile(src: str, extra: list[str]) -> str:
     obj = os.path.join(BUILD, src.replace(".cu", ".o"))
     cmd = [nvcc(), "-c", os.path.join(CSRC, src), "-o", obj] + ARCH + FLAGS + extra
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         raise RuntimeError(f"nvcc failed for {src}:\n{' '.join(cmd)}\n{res.stdout}\n{res.stderr}")
+    with open(log_of(src), "w") as f:
+        f.write(res.stderr)
     return obj
 
 

@@ -4,17 +4,17 @@
 // 8, 16 or 32 members whose keys lie far below every real one: two groups in lockstep on
 // packed FP32 for MP <= 8, one for the wider ones.  The relaxation is FastGroup's WIDE one
 // (finite keys never leave its range) with the step loop rolled, and the backward keeps
-// the steps' weights in thread-local memory.  Non-finite keys, and every group at a
-// tau too small for WIDE (wide_holds), go to ExactGroup in place.
+// the steps' weights in thread-local memory.  Non-finite keys go to ExactGroup in place; at a
+// tau too small for WIDE (wide_holds) all groups go to kernels of ExactGroup alone.
 #include "roi_launch.h"
 
 namespace roi {
 namespace {
 
 constexpr int kThreads = 128;
-// Padding members' keys (log2 units), the magnitude (squared) up to which real keys take the
-// fast relaxation, and the padding's largest offset from the second largest key over tau: 2^x
-// is 0 there whatever tau is, and second_of never picks it (a real key's offset lies above the
+// Padding members' keys (log2 units), the magnitude (squared) up to which real keys take the fast
+// relaxation, and the padding's largest offset from the second largest key over tau: 2^x is 0
+// there whatever tau is, and second_of never picks it (a real key's offset lies above the
 // padding's by 2e18 / tau and by 1e30 - 2e18 / tau, of which one is 5e29 or more).
 constexpr float kPadKey = -3.0e18f;
 constexpr float kMaxKeySq = 1.0e36f;
@@ -39,7 +39,6 @@ struct AnyArgs {
   int N, M;
   float tau, inv_tau;
   NoiseParams np;
-  float max_sq;  // groups with a larger sum of squared keys go to ExactGroup (all if negative)
   bool wait;  // pdl_begin
 };
 
@@ -163,15 +162,15 @@ __device__ __forceinline__ V total_of(const V (&x)[MP]) {
 }
 
 // FastGroup's WIDE forward with N steps at run time; step(k, mu) sees every step's weights.
-// Returns the lanes' flags (a non-finite key, or keys beyond max_sq).
+// Returns the lanes' flags (a non-finite key, or keys beyond kMaxKeySq).
 template <int MP, class V, class Step>
-__device__ __forceinline__ uint32_t any_relax(const V (&kap)[MP], int N, int M, float inv_tau, float max_sq, Step&& step) {
+__device__ __forceinline__ uint32_t any_relax(const V (&kap)[MP], int N, int M, float inv_tau, Step&& step) {
   const V itau = vconst<V>(inv_tau);
   V sq = vmul(kap[0], kap[0]);
 #pragma unroll
   for (int l = 1; l < MP; ++l)
     if (l < M) sq = vfma(kap[l], kap[l], sq);
-  const uint32_t flag = vbelow(vsub(vconst<V>(max_sq), sq), 0.0f);
+  const uint32_t flag = vbelow(vsub(vconst<V>(kMaxKeySq), sq), 0.0f);
   V x[MP];
   V ref = second_of(kap);
 #pragma unroll
@@ -233,7 +232,7 @@ __global__ void __launch_bounds__(kThreads) roi_any_fwd_kernel(AnyArgs a, bool w
       any_keys<MP, V>(a, e0, kap);
 #pragma unroll
       for (int l = 0; l < MP; ++l) S[l] = vconst<V>(0.0f);
-      const uint32_t flag = any_relax<MP, V>(kap, a.N, a.M, a.inv_tau, a.max_sq, [&](int, const V (&mu)[MP]) {
+      const uint32_t flag = any_relax<MP, V>(kap, a.N, a.M, a.inv_tau, [&](int, const V (&mu)[MP]) {
 #pragma unroll
         for (int l = 0; l < MP; ++l) S[l] = vadd(S[l], mu[l]);
       });
@@ -325,10 +324,15 @@ __global__ void __launch_bounds__(kThreads) roi_any_bwd_kernel(AnyArgs a) {
   for (int64_t t = int64_t(blockIdx.x) * kThreads + threadIdx.x; t < lanes; t += stride) {
     int64_t e0[L];
     const int have = any_groups<L>(a, t, e0);
-    V hist[MP - 1][MP];  // mu of every step
+    // mu of every step; ExactGroup, which comes after the sweep, keeps its own in the same place
+    union {
+      V mu[MP - 1][MP];
+      ExactGroup<MP - 1, MP> exact;
+    } steps;
+    V(&hist)[MP - 1][MP] = steps.mu;
     V kap[MP], c[MP], b[MP];
     any_keys<MP, V>(a, e0, kap);
-    const uint32_t flag = any_relax<MP, V>(kap, a.N, a.M, a.inv_tau, a.max_sq, [&](int k, const V (&mu)[MP]) {
+    const uint32_t flag = any_relax<MP, V>(kap, a.N, a.M, a.inv_tau, [&](int k, const V (&mu)[MP]) {
 #pragma unroll
       for (int l = 0; l < MP; ++l) hist[k][l] = mu[l];
     });
@@ -385,9 +389,8 @@ __global__ void __launch_bounds__(kThreads) roi_any_bwd_kernel(AnyArgs a) {
         float kn[MP], cc[MP];
 #pragma unroll
         for (int l = 0; l < MP; ++l) kn[l] = lane_of(kap[l], h) * kLn2, cc[l] = lane_of(c[l], h);
-        ExactGroup<MP - 1, MP> ex;
-        ex.forward(kn, a.N, a.M, a.tau, s);
-        ex.backward(cc, a.N, a.M, a.tau, g);
+        steps.exact.forward(kn, a.N, a.M, a.tau, s);
+        steps.exact.backward(cc, a.N, a.M, a.tau, g);
 #pragma unroll
         for (int l = 0; l < MP; ++l) g[l] *= a.np.inv_lam;
       }
@@ -440,6 +443,83 @@ __global__ void __launch_bounds__(kThreads) roi_any_bwd_kernel(AnyArgs a) {
   }
 }
 
+// Every group by ExactGroup, one a thread, members in local memory (1536 x 1536, tau = 0.05,
+// forward / backward: 18:24 1341 / 3828 us in place behind a fast relaxation that was thrown
+// away, 941 / 2529 here; 20:32 1531 / 4906, 1272 / 4061).  What bounds these is the L1's
+// bandwidth for the members.  A warp's frame is 32 times a thread's: the keys' array is longer
+// than 32 so that the frame is 16 bytes times an odd number and the warps' frames start in
+// different sets of the L1 (20:32 with 4864 B a thread 1516 / 4887 us, with 4880 1272 / 4061).
+constexpr int kExactKeys = 36;
+__device__ __forceinline__ void exact_keys(const AnyArgs& a, int64_t e0, float* kap) {
+  uint4 block = {};
+  for (int l = 0; l < a.M; ++l) {
+    const uint64_t e = a.np.e_base + uint64_t(e0) + l;
+    const uint32_t w = uint32_t(e) & 3u;
+    if (w == 0u || l == 0) block = noise_block(a.np, e & ~uint64_t(3));
+    kap[l] = key_log2(a.phi[e0 + l], uniform_from_word(w == 0u ? block.x : w == 1u ? block.y : w == 2u ? block.z : block.w),
+                      a.np.l2e_inv_lam);
+  }
+}
+
+// hard words are zeroed beforehand
+__global__ void __launch_bounds__(kThreads) roi_any_exact_fwd_kernel(AnyArgs a) {
+  pdl_begin(a.wait);
+  const int64_t stride = int64_t(gridDim.x) * kThreads;
+  for (int64_t g = int64_t(blockIdx.x) * kThreads + threadIdx.x; g < a.groups; g += stride) {
+    const int64_t e0 = g * a.M;
+    float kap[kExactKeys], S[32];
+    exact_keys(a, e0, kap);
+    const uint32_t bits = a.hard != nullptr || a.st ? topn_bits_dyn(kap, a.N, a.M) : 0u;
+    for (int l = 0; l < a.M; ++l) kap[l] *= kLn2;  // natural-log keys
+    ExactGroup<31, 32> ex;
+    ex.forward(kap, a.N, a.M, a.tau, S);
+    for (int l = 0; l < a.M; ++l) {
+      const int64_t e = e0 + l;
+      a.Wm[e] = a.st ? (((bits >> l) & 1u) ? a.W[e] : uint16_t(0))
+                     : __bfloat16_as_ushort(__float2bfloat16_rn(__fmul_rn(bf16_bits_to_float(a.W[e]), S[l])));
+      if (a.soft != nullptr) a.soft[e] = S[l];
+    }
+    if (a.hard != nullptr) {
+      const uint64_t v = uint64_t(bits) << (e0 & 31);
+      if (uint32_t(v) != 0u) atomicOr(&a.hard[e0 >> 5], uint32_t(v));
+      if (uint32_t(v >> 32) != 0u) atomicOr(&a.hard[(e0 >> 5) + 1], uint32_t(v >> 32));
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) roi_any_exact_bwd_kernel(AnyArgs a) {
+  pdl_begin(a.wait);
+  const int64_t stride = int64_t(gridDim.x) * kThreads;
+  for (int64_t g = int64_t(blockIdx.x) * kThreads + threadIdx.x; g < a.groups; g += stride) {
+    const int64_t e0 = g * a.M;
+    float kap[kExactKeys], c[32], S[32], dk[32];
+    exact_keys(a, e0, kap);
+    for (int l = 0; l < a.M; ++l) {
+      kap[l] *= kLn2;  // natural-log keys
+      c[l] = __fmul_rn(bf16_bits_to_float(a.dWm[e0 + l]), bf16_bits_to_float(a.W[e0 + l]));
+    }
+    ExactGroup<31, 32> ex;
+    ex.forward(kap, a.N, a.M, a.tau, S);
+    ex.backward(c, a.N, a.M, a.tau, dk);
+    for (int l = 0; l < a.M; ++l) {
+      const int64_t e = e0 + l;
+      const float d = dk[l] * a.np.inv_lam;
+      if (a.dphi != nullptr) a.dphi[e] = d;
+      if (a.phi_out != nullptr) {
+        float ph = a.phi[e], m = a.m[e], v = a.v[e];
+        adamw_elem(ph, d, m, v, a.opt);
+        a.phi_out[e] = ph;
+        a.m[e] = m;
+        a.v[e] = v;
+      }
+      if (a.dW != nullptr)
+        a.dW[e] = a.hard_in != nullptr
+                      ? (((a.hard_in[e >> 5] >> (e & 31)) & 1u) ? a.dWm[e] : uint16_t(0))
+                      : __bfloat16_as_ushort(__float2bfloat16_rn(__fmul_rn(bf16_bits_to_float(a.dWm[e]), S[l])));
+    }
+  }
+}
+
 int any_grid(int64_t groups, int per_thread) {
   const int64_t blocks = (groups + int64_t(per_thread) * kThreads - 1) / (int64_t(per_thread) * kThreads);
   const int64_t cap = int64_t(sm_count()) * 32;
@@ -462,15 +542,15 @@ int launch_any_fwd(const FwdCall& c) {
   a.tau = c.tau;
   a.inv_tau = 1.0f / c.tau;
   a.np = c.np;
-  a.max_sq = wide_holds(c.N, c.tau) ? kMaxKeySq : -1.0f;
-  const bool words = 32 % c.M == 0;
-  if (c.hard != nullptr && !words) {
-    // groups straddle words: assembled with atomicOr
+  const bool words = 32 % c.M == 0, exact = !wide_holds(c.N, c.tau);
+  if (c.hard != nullptr && (!words || exact)) {
+    // assembled with atomicOr
     if (cudaMemsetAsync(c.hard, 0, size_t((c.E + 31) / 32) * 4, c.stream) != cudaSuccess) return -1;
   }
   a.wait = lone_pdl(c.stream);
   int r;
-  if (c.M <= 4) r = launch_maybe_pdl(roi_any_fwd_kernel<4>, any_grid(a.groups, 2), kThreads, 0, c.stream, a.wait, a, words);
+  if (exact) r = launch_maybe_pdl(roi_any_exact_fwd_kernel, any_grid(a.groups, 1), kThreads, 0, c.stream, a.wait, a);
+  else if (c.M <= 4) r = launch_maybe_pdl(roi_any_fwd_kernel<4>, any_grid(a.groups, 2), kThreads, 0, c.stream, a.wait, a, words);
   else if (c.M <= 8) r = launch_maybe_pdl(roi_any_fwd_kernel<8>, any_grid(a.groups, 2), kThreads, 0, c.stream, a.wait, a, words);
   else if (c.M <= 16) r = launch_maybe_pdl(roi_any_fwd_kernel<16>, any_grid(a.groups, 1), kThreads, 0, c.stream, a.wait, a, words);
   else r = launch_maybe_pdl(roi_any_fwd_kernel<32>, any_grid(a.groups, 1), kThreads, 0, c.stream, a.wait, a, words);
@@ -495,10 +575,11 @@ int launch_any_bwd(const BwdCall& c) {
   a.tau = c.tau;
   a.inv_tau = 1.0f / c.tau;
   a.np = c.np;
-  a.max_sq = wide_holds(c.N, c.tau) ? kMaxKeySq : -1.0f;
+  const bool exact = !wide_holds(c.N, c.tau);
   a.wait = lone_pdl(c.stream);
   int r;
-  if (c.M <= 4) r = launch_maybe_pdl(roi_any_bwd_kernel<4>, any_grid(a.groups, 2), kThreads, 0, c.stream, a.wait, a);
+  if (exact) r = launch_maybe_pdl(roi_any_exact_bwd_kernel, any_grid(a.groups, 1), kThreads, 0, c.stream, a.wait, a);
+  else if (c.M <= 4) r = launch_maybe_pdl(roi_any_bwd_kernel<4>, any_grid(a.groups, 2), kThreads, 0, c.stream, a.wait, a);
   else if (c.M <= 8) r = launch_maybe_pdl(roi_any_bwd_kernel<8>, any_grid(a.groups, 2), kThreads, 0, c.stream, a.wait, a);
   else if (c.M <= 16) r = launch_maybe_pdl(roi_any_bwd_kernel<16>, any_grid(a.groups, 1), kThreads, 0, c.stream, a.wait, a);
   else r = launch_maybe_pdl(roi_any_bwd_kernel<32>, any_grid(a.groups, 1), kThreads, 0, c.stream, a.wait, a);

@@ -377,6 +377,38 @@ def test_patterns_without_own_kernel(roi, rows, groups, N, M, tau, lam):
     check_against_oracle(got, ph, Wb, dWb, N, M, tau, 123456789, 5, 2, lam, 3)
 
 
+# Large groups at the schedule's late temperatures (N log2(1 / tau) > 76), whose groups all go
+# to the log-space kernels: every form of the call, M that divides a hard word and M that does
+# not, a group count that is no multiple of a CTA's.  The first two have logits a unit apart (a
+# random permutation of 0, 1, 2, ... per group): near ties that compete over 18 steps and more
+# grow by up to 1 + 2 / tau in each, beyond any bound linear in N (18:24 at tau = 0.05 on normal
+# logits: 8 of 3096 soft entries at up to 3.4 times it, in the oracle's own recursion).
+@pytest.mark.parametrize("N,M,tau,lam,spaced", [(18, 24, 0.05, 0.05, True), (20, 32, 0.06, 0.05, True),
+                                                (31, 32, 0.17, 1.0, False), (22, 23, 0.08, 1.0, False)])
+def test_patterns_below_the_wide_rule(roi, N, M, tau, lam, spaced):
+    import torch
+    W, phi, dWm, ph, Wb, dWb = make(3, 43 * M, "normal", data_seed=M + N)
+    if spaced:
+        order = torch.rand(3 * 43, M, generator=torch.Generator().manual_seed(N)).argsort(dim=1)
+        phi = order.float().view(3, 43 * M).contiguous()
+        ph = phi.numpy()
+    st = roi.NoiseState(123456789, 5, 2, lam, 3)
+    got = gpu_run(roi, phi, W, dWm, N, M, tau, st)
+    check_against_oracle(got, ph, Wb, dWb, N, M, tau, 123456789, 5, 2, lam, 3)
+    p, w, d = phi.cuda(), W.cuda(), dWm.cuda()
+    hard = torch.full((roi.hard_words(*p.shape),), -1, dtype=torch.int32, device="cuda")
+    Wm, dW, dphi, g, m, v = (torch.empty_like(x) for x in (w, w, p, p, p, p))
+    roi.roi_mask_fwd_st(p, w, N, M, tau, st, Wm, None, hard)
+    roi.roi_mask_bwd_st(p, w, st, N, M, d, hard, tau, dphi, dW)
+    m.zero_(), v.zero_()
+    roi.roi_mask_bwd_adamw(p, w, st, N, M, d, tau, m, v, roi.AdamW(1e-3, 0.5, 0.75, 1e-8, 0.05, 3), g)
+    keep = torch.from_numpy(O.unpack_bits(got["hard_bits"], W.numel()).astype(bool)).view(W.shape).cuda()
+    assert np.array_equal(_bits(hard), got["hard_bits"])
+    assert torch.equal(Wm, torch.where(keep, w, 0)) and torch.equal(dW, torch.where(keep, d, 0))
+    assert np.array_equal(dphi.cpu().numpy(), got["dlogits"]) and torch.equal(g, dphi)
+    assert torch.equal(m, 0.5 * g) and torch.equal(v, 0.25 * (g * g)) and not torch.equal(p, phi.cuda())
+
+
 # Tiny temperatures, where every group's weights saturate: no NaN, and no remainder of the
 # capped lead in the gradient (2^-24 of the incoming one at the largest; the exact gradient
 # is 0 but for near ties, which these seeds do not hold).
