@@ -119,8 +119,10 @@ __device__ __forceinline__ void issue_chunk(const CUtensorMap* tm_phi, const CUt
 }
 
 // Relax this thread's pair of chunk kc from the staged logits and write
-// bf16(W * S) into the chunk's A tile (core-matrix layout).
-template <int N, int M, bool TAU1, bool WIDE>
+// bf16(W * S) into the chunk's A tile (core-matrix layout).  EXACT: every group by ExactGroup,
+// from keys that are formed in scalar code, as the mask forward's kernels for a tau too small
+// for the WIDE relaxation (roi_any.cu) form them.
+template <int N, int M, bool TAU1, bool WIDE, bool EXACT>
 __device__ __forceinline__ void chunk_masked_weights(const LinArgs& a, uint8_t* smem, const LinSmem& L, int stage,
                                                      int64_t row0, int kc) {
   int r, gk;
@@ -139,66 +141,79 @@ __device__ __forceinline__ void chunk_masked_weights(const LinArgs& a, uint8_t* 
       ph[h][4 * s] = p.x, ph[h][4 * s + 1] = p.y, ph[h][4 * s + 2] = p.z, ph[h][4 * s + 3] = p.w;
     }
   }
-  // keys in log2 units, as the mask forward forms them
-  F2 kap[M];
-  {
-    uint32_t x[2][M];
-    // every counter of the call below 2^32: the counter's low word in 32-bit
-    // arithmetic and a zero high word (as the mask kernels; rows past the last may
-    // wrap, but their outputs are never stored)
-    if (a.np.narrow) {
-      const uint32_t qk = uint32_t(a.np.e_base >> 2) + uint32_t(k >> 2);
+  // the noise words
+  uint32_t x[2][M];
+  // every counter of the call below 2^32: the counter's low word in 32-bit
+  // arithmetic and a zero high word (as the mask kernels; rows past the last may
+  // wrap, but their outputs are never stored)
+  if (a.np.narrow) {
+    const uint32_t qk = uint32_t(a.np.e_base >> 2) + uint32_t(k >> 2);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const uint32_t q0 = qk + uint32_t(row0 + r + 64 * h) * uint32_t(a.cols >> 2);
+    for (int h = 0; h < 2; ++h) {
+      const uint32_t q0 = qk + uint32_t(row0 + r + 64 * h) * uint32_t(a.cols >> 2);
 #pragma unroll
-        for (int s = 0; s < M / 4; ++s) {
-          const uint4 w = noise_block_lo(a.np, q0 + s);
-          x[h][4 * s] = w.x, x[h][4 * s + 1] = w.y, x[h][4 * s + 2] = w.z, x[h][4 * s + 3] = w.w;
-        }
-      }
-    } else {
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const uint64_t q0 = (a.np.e_base + uint64_t(e0[h])) >> 2;
-#pragma unroll
-        for (int s = 0; s < M / 4; ++s) {
-          const uint4 w = noise_block_q(a.np, q0 + s);
-          x[h][4 * s] = w.x, x[h][4 * s + 1] = w.y, x[h][4 * s + 2] = w.z, x[h][4 * s + 3] = w.w;
-        }
+      for (int s = 0; s < M / 4; ++s) {
+        const uint4 w = noise_block_lo(a.np, q0 + s);
+        x[h][4 * s] = w.x, x[h][4 * s + 1] = w.y, x[h][4 * s + 2] = w.z, x[h][4 * s + 3] = w.w;
       }
     }
+  } else {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint64_t q0 = (a.np.e_base + uint64_t(e0[h])) >> 2;
+#pragma unroll
+      for (int s = 0; s < M / 4; ++s) {
+        const uint4 w = noise_block_q(a.np, q0 + s);
+        x[h][4 * s] = w.x, x[h][4 * s + 1] = w.y, x[h][4 * s + 2] = w.z, x[h][4 * s + 3] = w.w;
+      }
+    }
+  }
+  float S[2][M];
+  if constexpr (EXACT) {
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      float kn[M], sh[M];
+#pragma unroll
+      for (int l = 0; l < M; ++l)
+        kn[l] = __fmul_rn(key_log2(h == 0 ? ph[0][l] : ph[1][l], uniform_from_word(h == 0 ? x[0][l] : x[1][l]), a.np.l2e_inv_lam), kLn2);
+      ExactGroup<N, M> ex;
+      ex.forward(kn, N, M, a.tau, sh);
+#pragma unroll
+      for (int l = 0; l < M; ++l) (h == 0 ? S[0][l] : S[1][l]) = sh[l];
+    }
+  } else {
+    // keys in log2 units, as the mask forward forms them
+    F2 kap[M];
 #pragma unroll
     for (int l = 0; l < M; ++l) {
       const F2 one_plus = f2(one_plus_from_word(x[0][l]), one_plus_from_word(x[1][l]));
       const F2 u = vsub(one_plus, vconst<F2>(__uint_as_float(0x3f7fffffu)));
       kap[l] = key_log2(f2(ph[0][l], ph[1][l]), u, a.np.l2e_inv_lam);
     }
-  }
-  FastGroup<N, M, TAU1, false, F2, RegSteps<1, 1, F2>, WIDE> fg;
-  fg.forward(kap, a.inv_tau);
-  float S[2][M];
+    FastGroup<N, M, TAU1, false, F2, RegSteps<1, 1, F2>, WIDE> fg;
+    fg.forward(kap, a.inv_tau);
 #pragma unroll
-  for (int h = 0; h < 2; ++h)
+    for (int h = 0; h < 2; ++h)
 #pragma unroll
-    for (int l = 0; l < M; ++l) S[h][l] = lane_of(fg.S[l], h);
-  if (fg.flag != 0u) {
+      for (int l = 0; l < M; ++l) S[h][l] = lane_of(fg.S[l], h);
+    if (fg.flag != 0u) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if ((fg.flag >> h) & 1u) {
-        // the mask forward's fallback, so Wm stays its bit for bit
-        float k[M], kn[M];
+      for (int h = 0; h < 2; ++h) {
+        if ((fg.flag >> h) & 1u) {
+          // the mask forward's fallback, so Wm stays its bit for bit
+          float k[M], kn[M];
 #pragma unroll
-        for (int l = 0; l < M; ++l) {
-          k[l] = lane_of(kap[l], h);
-          kn[l] = k[l] * kLn2;  // natural-log keys
-        }
-        if (!TAU1 && !WIDE && all_finite(k)) {
-          RobustGroup<N, M> rg;
-          rg.forward(k, a.inv_tau, S[h]);
-        } else {
-          ExactGroup<N, M> ex;
-          ex.forward(kn, N, M, a.tau, S[h]);
+          for (int l = 0; l < M; ++l) {
+            k[l] = lane_of(kap[l], h);
+            kn[l] = k[l] * kLn2;  // natural-log keys
+          }
+          if (!TAU1 && !WIDE && all_finite(k)) {
+            RobustGroup<N, M> rg;
+            rg.forward(k, a.inv_tau, S[h]);
+          } else {
+            ExactGroup<N, M> ex;
+            ex.forward(kn, N, M, a.tau, S[h]);
+          }
         }
       }
     }
@@ -225,7 +240,7 @@ __device__ __forceinline__ void chunk_masked_weights(const LinArgs& a, uint8_t* 
   }
 }
 
-template <int N, int M, bool TAU1, bool WIDE>
+template <int N, int M, bool TAU1, bool WIDE, bool EXACT = false>
 __global__ void __launch_bounds__(LinCfg<M>::kThreads + 32, 1)
     roi_masked_linear_kernel(const __grid_constant__ CUtensorMap tm_phi, const __grid_constant__ CUtensorMap tm_w,
                              const __grid_constant__ CUtensorMap tm_x, LinArgs a) {
@@ -316,7 +331,7 @@ __global__ void __launch_bounds__(LinCfg<M>::kThreads + 32, 1)
     for (int c = 0; c < nc; ++c) {
       if (ok) ok = mbar_wait_ring(full + s, phase, lim);
       if (!ok) break;
-      chunk_masked_weights<N, M, TAU1, WIDE>(a, smem, L, s, row0, c_begin + c);
+      chunk_masked_weights<N, M, TAU1, WIDE, EXACT>(a, smem, L, s, row0, c_begin + c);
       fence_proxy_async_smem();
       mbar_arrive(ready + s);
       if (s == kStages - 1) {
@@ -455,9 +470,14 @@ int launch_nm(const LinearCall& c, const LinArgs& a) {
       variant = 2;
       kern = roi_masked_linear_kernel<N, M, false, false>;
     }
+  } else {
+    if (variant == 1 && !tile_pattern(N, M, a.tau)) {
+      variant = 3;
+      kern = roi_masked_linear_kernel<N, M, false, false, true>;
+    }
   }
   // the shared-memory limit is set once per device and kernel, to the largest size
-  static int set_to[3][64] = {{0}};
+  static int set_to[4][64] = {{0}};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
   int& cur = set_to[variant][dev];

@@ -161,6 +161,34 @@ def test_prologue_wm_is_the_mask_forward(roi):
         assert np.all(np.abs(Y - want) <= acc + 1e-30)
 
 
+@pytest.mark.parametrize("N,M", [(2, 4), (2, 8), (4, 8)])
+@pytest.mark.parametrize("tau", [4e-12, 3e-12, 1e-25, 1e-38])
+def test_tiny_temperatures_follow_the_mask_forward(roi, N, M, tau):
+    """Where the mask forward leaves the WIDE relaxation (2:4 and 2:8 below tau = 2^-38) the
+    prologue does too.  Logits that put every key within 3 of 0 (target minus the noise), so
+    that key / tau stays finite down to tau = 1e-38 while key differences over tau do not."""
+    import torch
+    rows, cols, T = 130, 96, 5
+    W, _, _ = WL.make_inputs(rows, cols, "normal", 61)
+    X = WL.make_tokens(T, cols, 61)
+    st = roi.NoiseState(5, 9, 1, 1.0, 0)
+    g = torch.empty(rows * cols, device="cuda")
+    roi.roi_gumbel_noise(st, rows, cols, g)
+    target = 3.0 - 6.0 * torch.rand(rows * cols, generator=torch.Generator().manual_seed(3))
+    phi = (target.cuda() - g).view(rows, cols)
+    Y = gpu_linear(roi, X, phi, W, N, M, tau, st)
+    Wm = torch.empty(rows, cols, dtype=torch.bfloat16, device="cuda")
+    roi.roi_mask_fwd_ex(phi, W.cuda(), N, M, tau, st, Wm)
+    wm_bits = _u16(Wm)
+    want = O.bf16_to_f32(WL.bf16_bits(X)).astype(np.float64) @ O.bf16_to_f32(wm_bits).astype(np.float64).T
+    _, acc = linear_tolerance(WL.bf16_bits(X), wm_bits, cols)
+    if N == 2:
+        assert np.all(np.isfinite(want))
+    assert np.array_equal(np.isnan(Y), np.isnan(want))
+    fin = np.isfinite(want)
+    assert np.all(np.abs(Y - want)[fin] <= (acc + 1e-30)[fin])
+
+
 def test_split_k_is_deterministic(roi):
     """Long K over one row block: the workspace lets K split across CTAs; two runs
     agree bit for bit, and the unsplit call (no workspace) agrees up to order."""
