@@ -957,10 +957,12 @@ int launch_persistent(Kern kern, LaunchCache& cache, size_t smem, SliceArgs a, c
     cache.per_sm[dev] = per_sm < 1 ? 1 : per_sm;
   }
   const int64_t cap = int64_t(sm_count()) * cache.per_sm[dev];
-  // A lone tensor of less than one tile per SM goes as one ragged tail, its warps spread evenly
-  // over the SMs: a lane's sixteen members take N steps one after the other, and the fewer
-  // warps share an SM the sooner they are through.
-  if (a.full_tiles < cap && !pdl) a.full_tiles = 0;
+  // A lone tensor's whole rounds over the SMs go as tiles and the rest, which is all of a small
+  // tensor, as its ragged tail, whose warps are spread evenly over the SMs: a lane's sixteen
+  // members take N steps one after the other, and the fewer warps share an SM the sooner they
+  // are through (8:16 at tau = 0.5 with AdamW, a few tiles more than one round: 24.0 us with
+  // those as tiles, 21.4 so; 16:32 straight-through forward of 1.3 M elements 23.0 -> 20.6).
+  if (!pdl) a.full_tiles -= a.full_tiles % cap;
   const int64_t warps = ((a.E - a.full_tiles * kTileOf<Shape>) / Shape::kP + 31) / 32;
   const int64_t want = a.full_tiles + warps;
   const int grid = int(want < 1 ? 1 : (want < cap ? want : cap));

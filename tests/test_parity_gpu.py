@@ -331,6 +331,45 @@ def test_small_tensors_equal_slices(roi, N, M, tau, rows):
                          max(0, rows - 2))
 
 
+def _sms():
+    import torch
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+def check_rows(whole, phi, W, dWm, rows, N, M, tau, st, check_dlogits=True):
+    """Some rows of a call's outputs (no hard words) against the oracle."""
+    for a, b in rows:
+        got = {k: v[a:b] for k, v in whole.items() if k != "hard_bits"}
+        check_against_oracle(got, phi[a:b].numpy(), WL.bf16_bits(W[a:b]), WL.bf16_bits(dWm[a:b]), N, M, tau, st.seed,
+                             st.step, st.tensor_id, st.lam, st.row_offset + a, check_dlogits=check_dlogits)
+
+
+# Tensors that take tiles in a single call whatever the GPU's size (2:4: more than five rounds
+# of one pair a thread; the slices: a tile per SM or more, where the backward of 16:32 has the
+# smallest tile, and then a few tiles that are no round), and a remainder of an odd group
+# count, in the plain and the WIDE relaxations, at tau = 1 and tau > 1.
+@pytest.mark.parametrize("N,M", [(2, 4), (4, 8), (2, 8), (8, 16), (16, 32)])
+@pytest.mark.parametrize("tau,lam", [(1.0, 1.0), (0.6, 0.9), (0.45, 0.1), (1.5, 1.0)])
+def test_tiles_and_remainder(roi, N, M, tau, lam):
+    cols = 32 * 33
+    E = _sms() * {4: 5 * 1024 * 4 + 8192, 8: 2 * 8192, 16: 8192 + 2048, 32: 8192 + 2048}[M]
+    rows = E // cols + 3 | 1
+    W, phi, dWm, *_ = make(rows, cols, "normal", data_seed=N + M)
+    st = roi.NoiseState(123456789, 5, 2, lam, 0)
+    whole = gpu_run(roi, phi, W, dWm, N, M, tau, st)
+    check_rows(whole, phi, W, dWm, [(0, 2), (rows // 2, rows // 2 + 2), (rows - 20, rows)], N, M, tau, st)
+    # the same rows in two calls, the second one small
+    cut = (rows - 9) // 8 * 8
+    parts = [gpu_run(roi, phi[a:b].contiguous(), W[a:b].contiguous(), dWm[a:b].contiguous(), N, M, tau,
+                     roi.NoiseState(123456789, 5, 2, lam, a)) for a, b in ((0, cut), (cut, rows))]
+    for key in whole:
+        a, b = whole[key].ravel(), np.concatenate([p[key].ravel() for p in parts])
+        if M == 8 and key in ("soft", "Wm", "dlogits", "dW"):
+            # the remainder of an M = 8 tensor is scalar code, which rounds differently
+            a, b = a[:E // 2], b[:E // 2]
+        assert np.array_equal(a, b), key
+
+
 # Outputs end where the tensor does: every buffer carries a margin whose contents must
 # survive, at sizes whose last chunk holds a few groups only (one to a hard word's worth and
 # one more) alone, behind whole chunks and behind whole tiles.
