@@ -312,6 +312,11 @@ __device__ __forceinline__ uint32_t bwd_groups(const float* const* phi_g, const 
     }
   }
   if constexpr (HIST) bwd_upstream<M, V>(W_g, dWm_g, c);
+  // The moments' copies are waited for where they are used, but in the plain 4:8 form, whose
+  // sweep keeps within its registers only behind the wait (18944 x 3584, tau = 0.86: 577 -> 522
+  // us; WIDE 115 -> 120 and tau = 1 464 -> 503 the other way round).
+  constexpr bool kWaitFirst = N == 4 && !TAU1 && !WIDE;
+  if constexpr (kStageMoments && kWaitFirst) cp_async_wait_all();
   fg.backward(c, a.inv_tau, dkv);
   // dL/dphi = dL/dkappa / lambda (at tau = 1, lambda = 1 nothing to scale, the same bits)
   if (!TAU1 || a.np.inv_lam != 1.0f) {
@@ -319,7 +324,7 @@ __device__ __forceinline__ uint32_t bwd_groups(const float* const* phi_g, const 
 #pragma unroll
     for (int l = 0; l < M; ++l) dkv[l] = vmul(dkv[l], scale);
   }
-  if constexpr (kStageMoments) cp_async_wait_all();
+  if constexpr (kStageMoments && !kWaitFirst) cp_async_wait_all();
 #pragma unroll
   for (int h = 0; h < L; ++h) {
     float dk[M];

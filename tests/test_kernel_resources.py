@@ -43,3 +43,10 @@ def test_exact_kernels(usage):
     exact = {n: u for n, u in usage["roi_any.cu"].items() if "exact" in n}
     assert len(exact) == 2
     assert all(regs <= 64 and stack % 32 == 16 for regs, stack, _ in exact.values()), exact
+
+
+def test_4of8_adamw_does_not_spill(usage):
+    """4:8 at tau != 1 with the fused optimizer: where the moments' copies are waited for decides
+    whether the tile loop keeps within 168 registers."""
+    kernels = {n: u for n, u in usage["roi_bwd.cu"].items() if "roi_bwd_kernelILi4ELi8ELb0ELb0ELb1E" in n}
+    assert len(kernels) == 2 and all(u[2] == 0 for u in kernels.values()), kernels
