@@ -645,7 +645,6 @@ __global__ void __launch_bounds__(Cfg<N, M, ST || OPT>::kThreads, Cfg<N, M, ST |
   int cur = -1, src_cur = -1;
   int64_t lo = 0, hi = 0, src_lo = 0, src_hi = 0;
   BwdArgs a;
-  BwdOptArgs o;
   const uint8_t* src_ptr[3] = {nullptr, nullptr, nullptr};
   pdl_begin(mm.wait);
   const bool ok = run_tiles_src<C::kThreads, C::kTile, C::kStages, 3>(
@@ -667,9 +666,12 @@ __global__ void __launch_bounds__(Cfg<N, M, ST || OPT>::kThreads, Cfg<N, M, ST |
           lo = tile0[cur];
           hi = tile0[cur + 1];
           a = multi_args<N, M, ST || OPT>(mm, cur);
-          o = multi_opt(mm, cur);
         }
-        bwd_tile<N, M, TAU1, ST, OPT, NARROW_ONLY, WIDE>(stage, t - lo, a, o, smem, dg, int64_t(cur) << 48, exact);
+        // the optimizer's arguments from the parameter block where they are used: in registers
+        // they made the 4:8 forms spill (twelve 1024 x 1024 tensors, tau = 0.5 / 0.1, 135.2 /
+        // 138.4 -> 115.4 / 119.8 us; 2:4 96.0 -> 92.8, 2:8 109.4 -> 107.8)
+        bwd_tile<N, M, TAU1, ST, OPT, NARROW_ONLY, WIDE>(stage, t - lo, a, multi_opt(mm, cur), smem, dg,
+                                                         int64_t(cur) << 48, exact);
         release();
       });
   if constexpr (C::kDefer) {

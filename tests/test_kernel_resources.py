@@ -46,7 +46,9 @@ def test_exact_kernels(usage):
 
 
 def test_4of8_adamw_does_not_spill(usage):
-    """4:8 at tau != 1 with the fused optimizer: where the moments' copies are waited for decides
-    whether the tile loop keeps within 168 registers."""
-    kernels = {n: u for n, u in usage["roi_bwd.cu"].items() if "roi_bwd_kernelILi4ELi8ELb0ELb0ELb1E" in n}
-    assert len(kernels) == 2 and all(u[2] == 0 for u in kernels.values()), kernels
+    """4:8 at tau != 1 with the fused optimizer: the order of the sweep's sums and where the
+    optimizer's arguments live decide whether the tile loops keep within 168 registers (they
+    spilled 8 B alone, 168 and 268 B in runs, which cost up to 15 %)."""
+    for name in ("roi_bwd_kernel", "roi_bwd_multi_kernel"):
+        kernels = {n: u for n, u in usage["roi_bwd.cu"].items() if name + "ILi4ELi8ELb0ELb0ELb1E" in n}
+        assert len(kernels) == 2 and all(u[2] == 0 for u in kernels.values()), kernels
