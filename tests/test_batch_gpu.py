@@ -101,6 +101,123 @@ def test_batch_equals_single_calls(roi, N, M, tau):
         assert_same(a, b)
 
 
+def run_kind(roi, kind, ts, outs, N, M, tau, batch, opt):
+    """The straight-through calls or the fused AdamW backward of every tensor; `outs` is filled
+    (AdamW: phi, m, v in place)."""
+    if kind == "adamw":
+        items = [(o["phi"], t["W"], t["st"], t["dWm"], o["m"], o["v"], o["dphi"], o["dW"]) for t, o in zip(ts, outs)]
+        if batch:
+            roi.roi_mask_bwd_adamw_batch(items, N, M, tau, opt)
+        else:
+            for p, W, s, d, m, v, dphi, dW in items:
+                roi.roi_mask_bwd_adamw(p, W, s, N, M, d, tau, m, v, opt, dphi, dW)
+    elif batch:
+        roi.roi_mask_fwd_st_batch([(t["phi"], t["W"], t["st"], o["Wm"], o["soft"], o["hard"]) for t, o in zip(ts, outs)],
+                                  N, M, tau)
+        roi.roi_mask_bwd_st_batch([(t["phi"], t["W"], t["st"], t["dWm"], o["hard"], o["dphi"], o["dW"])
+                                   for t, o in zip(ts, outs)], N, M, tau)
+    else:
+        for t, o in zip(ts, outs):
+            roi.roi_mask_fwd_st(t["phi"], t["W"], N, M, tau, t["st"], o["Wm"], o["soft"], o["hard"])
+            roi.roi_mask_bwd_st(t["phi"], t["W"], t["st"], N, M, t["dWm"], o["hard"], tau, o["dphi"], o["dW"])
+    roi.roi_device_status()
+
+
+def adamw_state(t):
+    import torch
+    return {"phi": t["phi"].clone(), "m": torch.full_like(t["phi"], 1e-5), "v": torch.full_like(t["phi"], 1e-9)}
+
+
+# 2:4 at tau = 1 with outlier logits (+-100 in one of eight): about four groups of ten leave the
+# relaxation's range and the backward queues them, in a launch of several tensors under the
+# tensor's number (bit 48 of the entry).  Ten tensors of several tiles with remainders, and of
+# whole tiles only, whose kernels have no code for remainders: the single calls, which handle
+# such groups in place, and the oracle give the same.
+@pytest.mark.parametrize("kind", ["soft", "st", "adamw"])
+@pytest.mark.parametrize("shapes", [[(37, 1000), (64, 3584), (129, 2048), (300, 520), (16, 24576)] * 2,
+                                    [(64, 3584), (8, 1024), (512, 256), (128, 2048), (16, 24576)] * 2])
+def test_deferred_queue_of_a_shared_launch(roi, kind, shapes):
+    import torch
+    N, M, tau = 2, 4, 1.0
+    ts = make_set(shapes, 31)
+    g = torch.Generator().manual_seed(6)
+    for t in ts:
+        out = torch.randint(0, 16, t["phi"].shape, generator=g).cuda()
+        t["phi"] = t["phi"] + 100.0 * (out == 0) - 100.0 * (out == 1)
+    flags = [(True, True, True)] * len(ts)
+    if kind == "soft":
+        single, batch = run_single(roi, ts, N, M, tau, flags), run_batch(roi, ts, N, M, tau, flags)
+    else:
+        opt = roi.AdamW(1e-3, 0.9, 0.95, 1e-8, 0.05, 3)
+        single, batch = ([dict(outputs(roi, t, *f), **(adamw_state(t) if kind == "adamw" else {}))
+                          for t, f in zip(ts, flags)] for _ in range(2))
+        for b, outs in ((False, single), (True, batch)):
+            run_kind(roi, kind, ts, outs, N, M, tau, b, opt)
+    for a, b in zip(single, batch):
+        skip = ("Wm", "soft", "hard") if kind == "adamw" else ()
+        assert_same({k: v for k, v in a.items() if k not in skip}, {k: v for k, v in b.items() if k not in skip})
+    for t, o in list(zip(ts, batch))[:3]:
+        seed, step, tid, lam, roff = t["st"]
+        ph, Wb, dWb = t["phi"].cpu().numpy(), _u16(t["W"]), _u16(t["dWm"])
+        kw = dict(tensor_id=tid, lam=lam, row_offset=roff)
+        keys = O.mask_fwd(ph, Wb, N, M, tau, seed, step, **kw)["keys"]
+        b64 = O.mask_bwd(ph, Wb, dWb, N, M, tau, seed, step, **kw)["dlogits"]
+        b32 = O.mask_bwd(ph, Wb, dWb, N, M, tau, seed, step, dtype=np.float32, **kw)["dlogits"]
+        c = (O.bf16_to_f32(dWb).astype(np.float64) * O.bf16_to_f32(Wb)).ravel()
+        n, worst = C.dlogit_violations(o["dphi"].cpu().numpy(), b64, c, keys, N, M, tau, lam,
+                                       extra=4.0 * np.abs(b32.astype(np.float64) - b64))
+        assert n == 0, worst
+
+
+# Tensors of whole tiles (no remainder in either direction): at tau = 1 and below, plain and
+# fused with AdamW, the 2:4 backward has kernels of its own for them.
+@pytest.mark.parametrize("N,M", [(2, 4), (4, 8), (2, 8)])
+@pytest.mark.parametrize("tau", [1.0, 0.4, 0.1])
+def test_whole_tiles_equal_single_calls(roi, N, M, tau):
+    ts = make_set([(96, 1024), (24, 1024), (48, 2048), (192, 512), (24, 8192)] * 2, 83)
+    for a, b in zip(run_single(roi, ts, N, M, tau, [(True, True, False)] * len(ts)),
+                    run_batch(roi, ts, N, M, tau, [(True, True, False)] * len(ts))):
+        assert_same(a, b)
+    opt = roi.AdamW(1e-3, 0.9, 0.95, 1e-8, 0.05, 3)
+    single, batch = ([dict(adamw_state(t), dphi=t["phi"].clone(), dW=None) for t in ts] for _ in range(2))
+    run_kind(roi, "adamw", ts, single, N, M, tau, False, opt)
+    run_kind(roi, "adamw", ts, batch, N, M, tau, True, opt)
+    for a, b in zip(single, batch):
+        assert_same(a, b)
+
+
+# Outputs of batched calls end where their tensors do: margins behind every buffer survive.
+# Three tensors are launched one after another (the plain backward shares), ten share.
+@pytest.mark.parametrize("N,M", [(2, 4), (4, 8), (2, 8), (8, 16), (16, 32)])
+@pytest.mark.parametrize("count", [3, 10])
+@pytest.mark.parametrize("kind", ["soft", "st", "adamw"])
+def test_batch_writes_nothing_past_its_tensors(roi, N, M, count, kind):
+    import torch
+    ts = make_set([((1 + 3 * k) * (1 + 40 * (k % 3)), 32 * (1 + 2 * k)) for k in range(count)], 19)
+    pad, tau, opt = 4096, 0.4, roi.AdamW(1e-3, 0.9, 0.95, 1e-8, 0.05, 3)
+    outs, whole = [], []
+    for t in ts:
+        E, shape = t["phi"].numel(), t["phi"].shape
+        words = roi.hard_words(*shape)
+        buf = {k: torch.full((E + pad,), 7.0, device="cuda") for k in ("soft", "dphi", "phi", "m", "v")}
+        buf.update({k: torch.full((E + pad,), 7.0, dtype=torch.bfloat16, device="cuda") for k in ("Wm", "dW")})
+        buf["hard"] = torch.full((words + pad,), 7, dtype=torch.int32, device="cuda")
+        whole.append((buf, E, words))
+        outs.append({k: v[:words] if k == "hard" else v[:E].view(shape) for k, v in buf.items()})
+        outs[-1]["phi"].copy_(t["phi"])
+    if kind == "soft":
+        roi.roi_mask_fwd_batch([(t["phi"], t["W"], t["st"], o["Wm"], o["soft"], o["hard"]) for t, o in zip(ts, outs)],
+                               N, M, tau)
+        roi.roi_mask_bwd_batch([(t["phi"], t["W"], t["st"], t["dWm"], o["dphi"], o["dW"]) for t, o in zip(ts, outs)],
+                               N, M, tau)
+        roi.roi_device_status()
+    else:
+        run_kind(roi, kind, ts, outs, N, M, tau, True, opt)
+    for buf, E, words in whole:
+        for k, v in buf.items():
+            assert torch.all(v[words if k == "hard" else E:] == 7), k
+
+
 # Runs of small tensors of the wide patterns share a launch: odd group counts, a tensor of
 # one group, outlier logits whose groups go to the exact routine (queue entries that name
 # their tensor), lambda on both sides of the relaxation's rule (tau lambda = 0.05).

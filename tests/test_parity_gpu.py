@@ -167,15 +167,14 @@ CASES = [
     (11, 1001, 3, 7, 0.9, "normal"),
     (5, 64, 31, 32, 1.0, "normal"),
     (3, 6, 1, 2, 2.0, "normal"),
-    # the final temperature of the paper's schedule: a few per cent of the groups
-    # leave the fast paths' range and take the exact routines (the warp-slice
-    # kernels' deferred queue); 16:32 at tau = 0.1 takes the deferring variant too
+    # the final temperature of the paper's schedule: WIDE relaxations, but 16:32 at
+    # tau = 0.1 and lambda = 1, the last temperature of its plain one
     (64, 1024, 2, 4, 0.05, "logw"),
     (64, 1024, 4, 8, 0.05, "logw"),
     pytest.param(32, 1024, 8, 16, 0.05, "logw", marks=_SLICE_SMALL_TAU),
     pytest.param(32, 1024, 16, 32, 0.05, "logw", marks=_SLICE_SMALL_TAU),
     (32, 1024, 16, 32, 0.1, "logw"),
-    # 1 / tau < 1: the exclusive sums are checked themselves
+    # 1 / tau < 1
     (29, 1024, 4, 8, 1.5, "normal"),
     (9, 1024, 8, 16, 2.0, "normal"),
 ]
@@ -280,13 +279,13 @@ def test_wide_key_gaps_take_exact_path(roi, N, M, tau):
 
 @pytest.mark.parametrize("N,M", [(2, 4), (4, 8), (8, 16), (16, 32)])
 def test_every_group_out_of_range(roi, N, M):
-    """Every group leaves the fast paths' range at tau = 0.05: the logits of a group
-    are 20 natural-log units apart (a random permutation of 0, 20, 40, ... per group),
-    so each step's top key leads the next by far more than the ~3.5 units the fast
-    path's float range allows, and each step takes one member cleanly (a well-
-    conditioned input, unlike spreads where consumed members come back).  The
-    per-warp queues of the exact routine then fill tile after tile (32 drained at a
-    time) over several tiles and a ragged tail; results match the oracle."""
+    """Every group leaves the plain relaxations' range at tau = 0.05: the logits of a
+    group are 20 natural-log units apart (a random permutation of 0, 20, 40, ... per
+    group), so each step's top key leads the next by far more than the ~3.5 units that
+    range allows, and each step takes one member cleanly (a well-conditioned input,
+    unlike spreads where consumed members come back).  The WIDE relaxations, which these
+    patterns take there, cap every lead; results match the oracle.  (The queues of the
+    exact routines: test_deferred_queue.)"""
     import torch
     rows, cols = 40, 4160
     W, _, dWm, *_ = make(rows, cols, "normal", data_seed=17)
@@ -300,8 +299,9 @@ def test_every_group_out_of_range(roi, N, M):
 
 # The spread of the keys over the range of the plain tau != 1 relaxation grows as
 # 1 / (tau lambda): the temperatures of the annealing schedule, on both sides of the rule
-# that picks the relaxation for 4:8 (tau = 0.2, tau lambda = 0.09), and tau > 1.  24600 or
-# 24576 + a ragged tail of elements: full tiles of every tile kernel and a remainder.
+# that picks the relaxation for 4:8 (tau = 0.2, tau lambda = 0.09), and tau > 1.  24600
+# elements: three or four tiles of the M = 8 kernels and a ragged tail, and 2:4's form without
+# tiles (test_tiles_and_remainder takes those).
 @pytest.mark.parametrize("N,M", [(2, 4), (4, 8), (2, 8)])
 @pytest.mark.parametrize("tau,lam", [(0.2236, 0.0447), (0.05, 0.002), (0.21, 0.43), (0.21, 0.42), (0.2, 1.0),
                                      (0.201, 1.0), (1.5, 0.01)])
@@ -370,9 +370,40 @@ def test_tiles_and_remainder(roi, N, M, tau, lam):
         assert np.array_equal(a, b), key
 
 
+def outliers(phi, seed):
+    """One logit in sixteen 100 up, one 100 down: gaps beyond the tau = 1 relaxation's range in
+    about four groups of ten at M = 4."""
+    import torch
+    shift = torch.randint(0, 16, phi.shape, generator=torch.Generator().manual_seed(seed))
+    return (phi + 100.0 * (shift == 0).float() - 100.0 * (shift == 1).float()).contiguous()
+
+
+# The queues of the exact routines (2:4 backward at tau = 1; 8:16 and 16:32 in both directions,
+# tau = 1 and plain), of tensors that take tiles: more groups than 32 a warp and tile, a
+# remainder behind them, and the fused AdamW step, which a queued group must take once.
+@pytest.mark.parametrize("N,M,tau", [(2, 4, 1.0), (8, 16, 1.0), (8, 16, 0.5), (16, 32, 1.0), (16, 32, 0.5)])
+def test_deferred_queue(roi, N, M, tau):
+    import torch
+    cols = 32 * 33
+    rows = _sms() * (5 * 1024 * 4 + 8192 if M == 4 else 8192 + 2048) // cols + 3 | 1
+    W, phi, dWm, *_ = make(rows, cols, "normal", data_seed=N + M)
+    phi = outliers(phi, 77)
+    st = roi.NoiseState(3, 0, 0, 1.0, 0)
+    whole = gpu_run(roi, phi, W, dWm, N, M, tau, st)
+    check_rows(whole, phi, W, dWm, [(0, 2), (rows // 2, rows // 2 + 2), (rows - 12, rows)], N, M, tau, st)
+    p, m, v, g = phi.cuda(), *(torch.zeros_like(phi, device="cuda") for _ in range(3))
+    roi.roi_mask_bwd_adamw(p, W.cuda(), st, N, M, dWm.cuda(), tau, m, v, roi.AdamW(1e-3, 0.5, 0.75, 1e-8, 0.05, 3), g)
+    gn, ref = g.cpu().numpy(), whole["dlogits"]
+    scale = np.abs(ref).reshape(-1, M).max(-1, keepdims=True).repeat(M, -1).reshape(ref.shape)
+    assert np.all(np.abs(gn - ref) <= 1e-6 * scale + 1e-30)
+    assert torch.equal(m, 0.5 * g) and torch.equal(v, 0.25 * (g * g))
+    phi1 = phi.cuda() * np.float32(1.0 - np.float32(1e-3) * np.float32(0.05))
+    assert torch.all((p - phi1).abs() <= 1e-3 * 1.2 + 1e-5 * phi1.abs())  # one step: |m_hat / sqrt(v_hat)| <= 1.2 here
+
+
 # Outputs end where the tensor does: every buffer carries a margin whose contents must
 # survive, at sizes whose last chunk holds a few groups only (one to a hard word's worth and
-# one more) alone, behind whole chunks and behind whole tiles.
+# one more) alone, behind whole chunks and, at M = 8, behind whole tiles.
 @pytest.mark.parametrize("N,M", [(2, 4), (4, 8), (2, 8), (8, 16), (16, 32), (1, 4), (3, 7)])
 @pytest.mark.parametrize("base", [0, 12288 * 3, 4096 * 5])
 @pytest.mark.parametrize("groups", [1, 3, 5, 7, 8, 9, 17])
@@ -474,8 +505,8 @@ def test_large_temperatures(roi, N, M, tau):
     assert np.allclose(got["soft"].reshape(-1, M).sum(1), N, atol=1e-5 * N)
 
 
-# The warp-slice kernels' rule (tau = 0.1, tau lambda = 0.05); 41 rows are full tiles of
-# neither direction's shape and a ragged tail, 64 rows full tiles and a tail.
+# The warp-slice kernels' rule (tau = 0.1, tau lambda = 0.05), on tensors that go as one ragged
+# tail (test_tiles_and_remainder takes tiles).
 @pytest.mark.parametrize("rows", [1, 41, 64])
 @pytest.mark.parametrize("N,M", [(8, 16), (16, 32)])
 @pytest.mark.parametrize("tau,lam", [(0.6, 0.07), (0.35, 0.141), (0.35, 0.145), (1.5, 0.02), (1.5, 0.2)])

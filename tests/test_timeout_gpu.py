@@ -141,3 +141,37 @@ def test_masked_linear_times_out_drains_then_recovers(roi):
     roi.roi_device_status()
     assert torch.all(torch.isfinite(after))
     assert torch.equal(before.view(torch.int32), after.view(torch.int32))
+
+
+def test_exports_time_out_then_recover(roi):
+    """The exports of M = 4 and 8 (bits alone, with pruned weights, the compressed form) walk the
+    same ring; the next calls give the earlier ones' bits."""
+    import torch
+    dev = torch.device("cuda")
+    rows, cols = 2048, 4096  # several tiles per SM
+    W, phi, _ = WL.make_inputs(rows, cols, "normal", 57, device=dev)
+
+    def run(which):
+        bits = torch.zeros(roi.hard_words(rows, cols), dtype=torch.int32, device=dev)
+        Wp = torch.zeros_like(W)
+        vals = torch.zeros(rows, cols // 2, dtype=torch.bfloat16, device=dev)
+        if which == "bits4":
+            roi.roi_hard_mask_export(phi, 2, 4, bits)
+        elif which == "bits8":
+            roi.roi_hard_mask_export(phi, 4, 8, bits)
+        elif which == "pruned4":
+            roi.roi_hard_mask_export(phi, 2, 4, bits, W, Wp)
+        elif which == "pruned8":
+            roi.roi_hard_mask_export(phi, 4, 8, bits, W, Wp)
+        else:
+            roi.roi_export_compressed_2of4(phi, W, vals, bits)
+        return bits, Wp, vals
+
+    for which in ("bits4", "bits8", "pruned4", "pruned8", "compressed"):
+        before = run(which)
+        roi.roi_device_status()
+        _expect_timeout(roi, lambda: run(which))
+        after = run(which)
+        roi.roi_device_status()
+        assert torch.equal(before[0], after[0])
+        assert all(torch.equal(a.view(torch.int16), b.view(torch.int16)) for a, b in zip(before[1:], after[1:]))
