@@ -855,7 +855,7 @@ def run_variant(args):
         achieved = E * EXPORT_2OF4_BYTES * args.steps / a_t / 1e9
         per, step_bytes = EXPORT_2OF4_BYTES, EXPORT_2OF4_BYTES
         extra = {"ms_per_step": round(1e3 * a_t / args.steps, 3)}
-        kernel = "roi_export_2of4_kernel"
+        kernel = "roi_export_tiles_kernel"
         metric = "compressed 2:4 export groups/s and HBM GB/s, 1 GPU"
     step_gbs = E * step_bytes * args.steps / elapsed / 1e9
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",

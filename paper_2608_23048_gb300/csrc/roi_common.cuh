@@ -28,9 +28,8 @@ constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kTinyExcl = 7.888609052210118e-31f;  // 2^-100
 
 // FastGroup's WIDE relaxation: the largest lead of a group's first member over its second,
-// in log2 units, and the patterns that always take it.  With one correction (N = 2) the
-// second maximum costs what the range checks it replaces did; at N = 4 it is formed three
-// times, and wide_range() in roi_launch.h decides.
+// in log2 units, and the patterns that always take it.  With one correction (N = 2) there is
+// one second maximum to form; at N = 4 there are three, and wide_range() in roi_launch.h decides.
 constexpr float kLeadCap = 100.0f;
 // Range of the plain tau != 1 relaxations (see FastGroup's forward).
 constexpr float kLeastRange = -98.0f;
@@ -405,8 +404,9 @@ __device__ __forceinline__ uint32_t topn_bits_dyn(const float* kap, int N, int M
 // Follows the recursion literally: z = alpha / tau, mu = exp(z - LSE z),
 // log(1 - mu_l) = LSE_{i != l} z_i - LSE z (no clamp).  The backward uses the
 // bounded form d l_i / d z_l = [l != i] exp(z_l - LSE_{j != i} z_j) - mu_l.
-// Used for groups the fast path flags, for ragged tails and for N:M patterns
-// without a specialised kernel.  NMAX x MMAX bounds the (runtime) N x M.
+// Used for groups with non-finite keys, for finite ones out of the tau = 1 kernels' range, and
+// for whole calls of the patterns at a tau too small for the WIDE relaxation (roi_any.cu).
+// NMAX x MMAX bounds the (runtime) N x M.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float lse_excluding(const float* z, int M, int skip) {
   float m = -INFINITY;
@@ -869,14 +869,6 @@ __device__ __forceinline__ V max_of(const V (&x)[M]) {
   V m = x[0];
 #pragma unroll
   for (int l = 1; l < M; ++l) m = vmax(m, x[l]);
-  return m;
-}
-
-template <int M, class V>
-__device__ __forceinline__ V min_of(const V (&x)[M]) {
-  V m = x[0];
-#pragma unroll
-  for (int l = 1; l < M; ++l) m = vmin(m, x[l]);
   return m;
 }
 

@@ -97,9 +97,7 @@ __device__ __forceinline__ float lane_of(V v, int h) {
   }
 }
 
-// L groups (one per lane of V) processed in lockstep by one thread; writes their
-// outputs and returns each group's hard bits in bits[h].
-// The keys of L groups from their staged logits (first half of fwd_groups).
+// The keys of L groups (one per lane of V) from their staged logits.
 template <int M, class V, bool NARROW = false>
 __device__ __forceinline__ void fwd_keys(const float* const* phi_g, const int64_t* e0, const uint32_t* q0,
                                          const FwdArgs& a, V (&kap)[M]) {
@@ -116,7 +114,8 @@ __device__ __forceinline__ void fwd_keys(const float* const* phi_g, const int64_
   group_keys<M, V, NARROW>(ph, e0, q0, a.np, kap);
 }
 
-// Relaxation, hard bits and outputs of L groups whose keys are `kap`.
+// Relaxation, hard bits (bits[h]) and outputs of L groups whose keys are `kap`, in lockstep by
+// one thread.
 template <int N, int M, bool TAU1, class V, bool ST, bool WIDE>
 __device__ __forceinline__ void fwd_finish(const V (&kap)[M], const uint16_t* const* W_g, const int64_t* e0,
                                                const FwdArgs& a, uint32_t* bits) {

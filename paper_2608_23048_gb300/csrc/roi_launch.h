@@ -16,15 +16,19 @@ inline bool counters_narrow(const NoiseParams& np, int64_t E) {
   return np.e_base <= lim && uint64_t(E) <= lim - np.e_base;
 }
 
-// The relaxation of a tau != 1 tile kernel (FastGroup, M = 4, 8).  WIDE always where it
-// costs nothing (kAlwaysWide; 0.5B-shaped 2:4 step at tau = 0.1 1848 -> 1813 us).  4:8 at
-// tau = 0.5 pays 2.7 % for it (one 1.5B-shaped block, forward and backward, 335 -> 344 us)
-// and takes the plain one unless groups are likely to leave that one's range, which are
-// then relaxed by a slow routine.  The range is ~69 tau in natural-log units of the keys:
-// the Gumbel noise alone exceeds it below tau = 0.2 (same block, plain / WIDE: 347 / 343 us
-// at tau = 0.2, 519 / 344 at 0.1, 1338 / 344 at 0.06), logits of unit spread do where
-// 69 tau is a few times 1 / lambda (986 / 349 us at tau = 0.22, lambda = 0.045, while
-// tau lambda = 0.1 still measured 336 plain).
+// The relaxation of a tau != 1 tile kernel (FastGroup, M = 4, 8).  The plain one leaves groups
+// beyond its range, ~69 tau in natural-log units of the keys, to a slow routine; WIDE has no
+// range and costs more where no group leaves the plain one's:
+// - N = 2 takes WIDE always (kAlwaysWide).  Early in the schedule, on logits of unit spread, it
+//   costs the 2:4 forward 3 % and the masked linear 5 % on large tensors (18944 x 3584, tau =
+//   0.74: 142 -> 147 us, 149 -> 157; the backwards nothing); from tau lambda = 0.046 on, or
+//   0.086 at twice that spread, it takes 2 to 34 % less.
+// - 4:8 takes it where groups are likely to leave.  The Gumbel noise alone does below tau = 0.2
+//   (one 1.5B-shaped block, forward and backward, plain / WIDE: 347 / 343 us at tau = 0.2, 519 /
+//   344 at 0.1, 1338 / 344 at 0.06), logits where their spread is a few times 69 tau lambda
+//   (8960 x 1536, forward, unit spread: 42.9 / 45.8 us at tau lambda = 0.063, 58.3 / 45.7 at
+//   0.046; twice that spread 43.0 / 45.6 at 0.117, 73.3 / 45.9 at 0.086).  The line keeps twice
+//   the unit spread on the WIDE side; unit spread pays 7 % between 0.09 and 0.055 for it.
 constexpr float kWideTau = 0.2f;
 // WIDE holds the weights of a group behind its leader's capped lead at 2^-100 or more where
 // they should vanish, and the backward multiplies such a remainder by 1 / tau once a step:

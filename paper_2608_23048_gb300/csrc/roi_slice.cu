@@ -20,8 +20,8 @@ namespace roi {
 namespace {
 
 // Launch shapes: threads per CTA (one CTA per SM in either direction), ring stages.
-// The backward keeps steps 0 .. N-3 of the relaxation in shared memory behind the ring
-// (4 P bytes a thread and step) and the last two in registers.
+// The backward keeps the last kRegSteps steps of the relaxation in registers and the others in
+// shared memory behind the ring (4 P bytes a thread and step).
 template <int M>
 struct FwdShape {
   static constexpr int kP = 16;  // members of a group per lane
@@ -99,37 +99,23 @@ __device__ __forceinline__ F2 sum_pk(const F2 (&x)[H]) {
 // the other half's sums.
 template <int SL, int H>
 __device__ __forceinline__ float exclusive(const F2 (&x)[H], F2 (&ex)[H]) {
-  static_assert(H == 4 || H == 8, "8 or 16 members a lane");
-  if constexpr (H == 4) {
-    const F2 p = x[0] + x[1], q = x[2] + x[3];
-    const F2 t = p + q;
-    const float own = __fadd_rn(lo(t), hi(t));
-    const float oth = sum_others<SL>(own);
-    const F2 beyond = SL == 1 ? swap(t) : swap(t) + f2(oth);
-    const F2 p1 = p + beyond, q1 = q + beyond;
-    ex[0] = x[1] + q1;
-    ex[1] = x[0] + q1;
-    ex[2] = x[3] + p1;
-    ex[3] = x[2] + p1;
-    return SL == 1 ? own : __fadd_rn(own, oth);
-  } else {
-    F2 p[4];
+  static_assert(H == 8, "16 members a lane");
+  F2 p[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) p[i] = x[2 * i] + x[2 * i + 1];
-    const F2 q0 = p[0] + p[1], q1 = p[2] + p[3];
-    const F2 t = q0 + q1;
-    const float own = __fadd_rn(lo(t), hi(t));
-    const float oth = sum_others<SL>(own);
-    const F2 beyond = SL == 1 ? swap(t) : swap(t) + f2(oth);
-    const F2 r0 = q0 + beyond, r1 = q1 + beyond;
-    const F2 e[4] = {p[1] + r1, p[0] + r1, p[3] + r0, p[2] + r0};
+  for (int i = 0; i < 4; ++i) p[i] = x[2 * i] + x[2 * i + 1];
+  const F2 q0 = p[0] + p[1], q1 = p[2] + p[3];
+  const F2 t = q0 + q1;
+  const float own = __fadd_rn(lo(t), hi(t));
+  const float oth = sum_others<SL>(own);
+  const F2 beyond = SL == 1 ? swap(t) : swap(t) + f2(oth);
+  const F2 r0 = q0 + beyond, r1 = q1 + beyond;
+  const F2 e[4] = {p[1] + r1, p[0] + r1, p[3] + r0, p[2] + r0};
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      ex[2 * i] = x[2 * i + 1] + e[i];
-      ex[2 * i + 1] = x[2 * i] + e[i];
-    }
-    return SL == 1 ? own : __fadd_rn(own, oth);
+  for (int i = 0; i < 4; ++i) {
+    ex[2 * i] = x[2 * i + 1] + e[i];
+    ex[2 * i + 1] = x[2 * i] + e[i];
   }
+  return SL == 1 ? own : __fadd_rn(own, oth);
 }
 template <int SL, int H>
 __device__ __forceinline__ float group_max(const F2 (&x)[H]) {
@@ -961,7 +947,7 @@ int launch_persistent(Kern kern, LaunchCache& cache, size_t smem, SliceArgs a, c
   // tensor, as its ragged tail, whose warps are spread evenly over the SMs: a lane's sixteen
   // members take N steps one after the other, and the fewer warps share an SM the sooner they
   // are through (8:16 at tau = 0.5 with AdamW, a few tiles more than one round: 24.0 us with
-  // those as tiles, 21.4 so; 16:32 straight-through forward of 1.3 M elements 23.0 -> 20.6).
+  // those as tiles, 21.4 so; 16:32 straight-through forward of 1.3 M elements 23.2 -> 17.7).
   if (!pdl) a.full_tiles -= a.full_tiles % cap;
   const int64_t warps = ((a.E - a.full_tiles * kTileOf<Shape>) / Shape::kP + 31) / 32;
   const int64_t want = a.full_tiles + warps;
