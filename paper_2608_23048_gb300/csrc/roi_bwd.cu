@@ -839,7 +839,7 @@ int launch_multi(const BwdCall* calls, int count, bool pdl) {
 }  // namespace
 
 namespace {
-int launch_bwd_impl(const BwdCall& c, bool pdl) {
+int launch_bwd_impl(const BwdCall& c, bool pdl, bool alone) {
   BwdArgs a;
   a.phi = c.phi;
   a.W = c.W;
@@ -859,7 +859,7 @@ int launch_bwd_impl(const BwdCall& c, bool pdl) {
   a.np = c.np;
   a.np.narrow = counters_narrow(c.np, c.E);
   a.status = c.status;
-  if (slice_supported(c.N, c.M)) return launch_slice_bwd(c, pdl);
+  if (slice_supported(c.N, c.M)) return launch_slice_bwd(c, pdl, alone);
   if (!tile_pattern(c.N, c.M, c.tau)) return launch_any_bwd(c);
   if (c.N == 2 && c.M == 4) return launch_nm<2, 4>(a, o, c.stream, pdl);
   if (c.N == 4 && c.M == 8) return launch_nm<4, 8>(a, o, c.stream, pdl);
@@ -867,7 +867,7 @@ int launch_bwd_impl(const BwdCall& c, bool pdl) {
 }
 }  // namespace
 
-int launch_bwd(const BwdCall& c) { return launch_bwd_impl(c, false); }
+int launch_bwd(const BwdCall& c) { return launch_bwd_impl(c, false, true); }
 
 // As launch_fwd_batch: the tensors are independent, so from the second launch on
 // the tile kernels (plain or fused with AdamW) are launched with programmatic
@@ -915,7 +915,7 @@ int launch_bwd_batch(const BwdCall* calls, int count) {
       }
     }
     const bool tiled = tile_pattern(c.N, c.M, c.tau) || slice_supported(c.N, c.M);
-    const int r = launch_bwd_impl(c, tiled && prev_tiled);
+    const int r = launch_bwd_impl(c, tiled && prev_tiled, count == 1);
     if (r < 0) return -1;
     launched += r;
     prev_tiled = tiled && r > 0;

@@ -614,7 +614,7 @@ int launch_multi(const FwdCall* calls, int count, bool pdl) {
 }  // namespace
 
 namespace {
-int launch_fwd_impl(const FwdCall& c, bool pdl) {
+int launch_fwd_impl(const FwdCall& c, bool pdl, bool alone) {
   FwdArgs a;
   a.phi = c.phi;
   a.W = c.W;
@@ -629,7 +629,7 @@ int launch_fwd_impl(const FwdCall& c, bool pdl) {
   a.np = c.np;
   a.np.narrow = counters_narrow(c.np, c.E);
   a.status = c.status;
-  if (slice_supported(c.N, c.M)) return launch_slice_fwd(c, pdl);
+  if (slice_supported(c.N, c.M)) return launch_slice_fwd(c, pdl, alone);
   if (!tile_pattern(c.N, c.M, c.tau)) return launch_any_fwd(c);
   if (c.N == 2 && c.M == 4) return launch_nm<2, 4>(a, c.stream, pdl);
   if (c.N == 4 && c.M == 8) return launch_nm<4, 8>(a, c.stream, pdl);
@@ -637,7 +637,7 @@ int launch_fwd_impl(const FwdCall& c, bool pdl) {
 }
 }  // namespace
 
-int launch_fwd(const FwdCall& c) { return launch_fwd_impl(c, false); }
+int launch_fwd(const FwdCall& c) { return launch_fwd_impl(c, false, true); }
 
 // The tensors of a batch are independent (the caller checked that no output
 // overlaps another range), so from the second launch on the tile kernels are
@@ -681,7 +681,7 @@ int launch_fwd_batch(const FwdCall* calls, int count) {
       }
     }
     const bool tiled = tile_pattern(c.N, c.M, c.tau) || slice_supported(c.N, c.M);
-    const int r = launch_fwd_impl(c, tiled && prev_tiled);
+    const int r = launch_fwd_impl(c, tiled && prev_tiled, count == 1);
     if (r < 0) return -1;
     launched += r;
     prev_tiled = tiled && r > 0;

@@ -135,8 +135,9 @@ int launch_export(const ExportCall& c);
 int launch_export_compressed_2of4(const CompressCall& c);
 // Warp-slice kernels for M = 16, 32 (roi_slice.cu).
 bool slice_supported(int N, int M);
-int launch_slice_fwd(const FwdCall& c, bool pdl = false);
-int launch_slice_bwd(const BwdCall& c, bool pdl = false);
+// (`alone`: no launch is chained behind)
+int launch_slice_fwd(const FwdCall& c, bool pdl, bool alone);
+int launch_slice_bwd(const BwdCall& c, bool pdl, bool alone);
 // A batch's runs of small tensors, one launch each.
 int slice_fwd_run(const FwdCall* calls, int count);
 int slice_bwd_run(const BwdCall* calls, int count);

@@ -930,7 +930,7 @@ struct LaunchCache {
 };
 
 template <class Shape, class Kern>
-int launch_persistent(Kern kern, LaunchCache& cache, size_t smem, SliceArgs a, cudaStream_t stream, bool pdl) {
+int launch_persistent(Kern kern, LaunchCache& cache, size_t smem, SliceArgs a, cudaStream_t stream, bool pdl, bool alone) {
   a.full_tiles = a.E / kTileOf<Shape>;
   a.wait = !pdl && lone_pdl(stream);
   int dev = 0;
@@ -946,9 +946,14 @@ int launch_persistent(Kern kern, LaunchCache& cache, size_t smem, SliceArgs a, c
   // A lone tensor's whole rounds over the SMs go as tiles and the rest, which is all of a small
   // tensor, as its ragged tail, whose warps are spread evenly over the SMs: a lane's sixteen
   // members take N steps one after the other, and the fewer warps share an SM the sooner they
-  // are through (8:16 at tau = 0.5 with AdamW, a few tiles more than one round: 24.0 us with
-  // those as tiles, 21.4 so; 16:32 straight-through forward of 1.3 M elements 23.2 -> 17.7).
-  if (!pdl) a.full_tiles -= a.full_tiles % cap;
+  // are through (8:16 at tau = 0.5 with AdamW, a few tiles more than one round: 24.5 us with
+  // those as tiles, 21.5 so; 16:32 straight-through forward of 1.3 M elements 23.2 -> 17.7).
+  // A last round that is more than half full stays as tiles, whose loads are staged (8:16
+  // forward of 3.7 M elements 19.9 against 20.2 us), but for AdamW's, whose own loads are not
+  // (1.8 M elements 30.2 against 26.8).  Where a launch is chained behind, it fills the SMs that
+  // the last round leaves (the first tensor of a 3B-shaped set cut: its step 1677 -> 1694 us).
+  const int64_t last = a.full_tiles % cap;
+  if ((a.full_tiles < cap && !pdl) || (alone && (last <= cap / 2 || a.phi_out != nullptr))) a.full_tiles -= last;
   const int64_t warps = ((a.E - a.full_tiles * kTileOf<Shape>) / Shape::kP + 31) / 32;
   const int64_t want = a.full_tiles + warps;
   const int grid = int(want < 1 ? 1 : (want < cap ? want : cap));
@@ -956,29 +961,29 @@ int launch_persistent(Kern kern, LaunchCache& cache, size_t smem, SliceArgs a, c
 }
 
 template <int N, int M, bool TAU1, bool WIDE>
-int slice_fwd(const SliceArgs& a, cudaStream_t stream, bool pdl) {
+int slice_fwd(const SliceArgs& a, cudaStream_t stream, bool pdl, bool alone) {
   static LaunchCache cache;
   constexpr size_t smem = kFwdDeferOffset<M> + kDeferBytes<M, FwdShape<M>>;
   static_assert(smem <= 232448, "shared memory per CTA");
-  return launch_persistent<FwdShape<M>>(roi_slice_fwd_kernel<N, M, TAU1, WIDE>, cache, smem, a, stream, pdl);
+  return launch_persistent<FwdShape<M>>(roi_slice_fwd_kernel<N, M, TAU1, WIDE>, cache, smem, a, stream, pdl, alone);
 }
 template <int N, int M, bool TAU1, bool WIDE>
-int slice_bwd(const SliceArgs& a, cudaStream_t stream, bool pdl) {
+int slice_bwd(const SliceArgs& a, cudaStream_t stream, bool pdl, bool alone) {
   static LaunchCache cache;
   constexpr size_t smem = kBwdDeferOffset<N, M> + kDeferBytes<M, BwdShape<M>>;
   static_assert(smem <= 232448, "shared memory per CTA");
-  return launch_persistent<BwdShape<M>>(roi_slice_bwd_kernel<N, M, TAU1, WIDE>, cache, smem, a, stream, pdl);
+  return launch_persistent<BwdShape<M>>(roi_slice_bwd_kernel<N, M, TAU1, WIDE>, cache, smem, a, stream, pdl, alone);
 }
 
 template <int N, int M>
-int slice_fwd_nm(const SliceArgs& a, cudaStream_t stream, bool pdl) {
-  if (a.tau == 1.0f) return slice_fwd<N, M, true, false>(a, stream, pdl);
-  return slice_wide(N, a.tau, a.np) ? slice_fwd<N, M, false, true>(a, stream, pdl) : slice_fwd<N, M, false, false>(a, stream, pdl);
+int slice_fwd_nm(const SliceArgs& a, cudaStream_t stream, bool pdl, bool alone) {
+  if (a.tau == 1.0f) return slice_fwd<N, M, true, false>(a, stream, pdl, alone);
+  return slice_wide(N, a.tau, a.np) ? slice_fwd<N, M, false, true>(a, stream, pdl, alone) : slice_fwd<N, M, false, false>(a, stream, pdl, alone);
 }
 template <int N, int M>
-int slice_bwd_nm(const SliceArgs& a, cudaStream_t stream, bool pdl) {
-  if (a.tau == 1.0f) return slice_bwd<N, M, true, false>(a, stream, pdl);
-  return slice_wide(N, a.tau, a.np) ? slice_bwd<N, M, false, true>(a, stream, pdl) : slice_bwd<N, M, false, false>(a, stream, pdl);
+int slice_bwd_nm(const SliceArgs& a, cudaStream_t stream, bool pdl, bool alone) {
+  if (a.tau == 1.0f) return slice_bwd<N, M, true, false>(a, stream, pdl, alone);
+  return slice_wide(N, a.tau, a.np) ? slice_bwd<N, M, false, true>(a, stream, pdl, alone) : slice_bwd<N, M, false, false>(a, stream, pdl, alone);
 }
 
 template <int N, int M, bool TAU1, bool WIDE, bool BWD>
@@ -1084,7 +1089,7 @@ int slice_bwd_run(const BwdCall* calls, int count) {
 int launch_slice_fwd_multi(const FwdCall* calls, int count, bool pdl) { return launch_slice_multi<false>(calls, count, pdl); }
 int launch_slice_bwd_multi(const BwdCall* calls, int count, bool pdl) { return launch_slice_multi<true>(calls, count, pdl); }
 
-int launch_slice_fwd(const FwdCall& c, bool pdl) {
+int launch_slice_fwd(const FwdCall& c, bool pdl, bool alone) {
   SliceArgs a{};
   a.phi = c.phi;
   a.W = c.W;
@@ -1097,12 +1102,12 @@ int launch_slice_fwd(const FwdCall& c, bool pdl) {
   a.inv_tau = 1.0f / c.tau;
   a.np = c.np;
   a.status = c.status;
-  if (c.N == 8 && c.M == 16) return slice_fwd_nm<8, 16>(a, c.stream, pdl);
-  if (c.N == 16 && c.M == 32) return slice_fwd_nm<16, 32>(a, c.stream, pdl);
+  if (c.N == 8 && c.M == 16) return slice_fwd_nm<8, 16>(a, c.stream, pdl, alone);
+  if (c.N == 16 && c.M == 32) return slice_fwd_nm<16, 32>(a, c.stream, pdl, alone);
   return -1;
 }
 
-int launch_slice_bwd(const BwdCall& c, bool pdl) {
+int launch_slice_bwd(const BwdCall& c, bool pdl, bool alone) {
   SliceArgs a{};
   a.phi = c.phi;
   a.W = c.W;
@@ -1119,8 +1124,8 @@ int launch_slice_bwd(const BwdCall& c, bool pdl) {
   a.inv_tau = 1.0f / c.tau;
   a.np = c.np;
   a.status = c.status;
-  if (c.N == 8 && c.M == 16) return slice_bwd_nm<8, 16>(a, c.stream, pdl);
-  if (c.N == 16 && c.M == 32) return slice_bwd_nm<16, 32>(a, c.stream, pdl);
+  if (c.N == 8 && c.M == 16) return slice_bwd_nm<8, 16>(a, c.stream, pdl, alone);
+  if (c.N == 16 && c.M == 32) return slice_bwd_nm<16, 32>(a, c.stream, pdl, alone);
   return -1;
 }
 
