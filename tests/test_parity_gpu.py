@@ -142,7 +142,7 @@ def test_tiny_config_full_parity(roi):
 
 # Known limit: at tau = 0.05 the warp-slice kernels' float32 recursion (linear-domain
 # weights, exclusive sums, hardware exp2 / log2) lands outside the derived logit-gradient
-# bound on one or two groups of these inputs (by 2.7x at 8:16, 1.8x at 16:32), where
+# bound on one or two groups of these inputs (by 1.8x in either pattern), where
 # near-tied members keep competing over eight or sixteen steps; the soft mask, the
 # masked weights and the hard mask are within their rules.
 _SLICE_SMALL_TAU = pytest.mark.xfail(strict=True, raises=AssertionError,
