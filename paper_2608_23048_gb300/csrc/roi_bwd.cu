@@ -25,6 +25,12 @@ struct Cfg {
   static constexpr int kStages = M == 4 ? 3 : 2;  // 192 KB (M = 4), 96 KB + 72 KB step history (M = 8)
   static constexpr int kMinBlocks = 1;
   static constexpr int kTile = 2 * kPairs * kThreads * M;  // elements
+  // Tiles cover whole units.  The forms of 2:8 have tiles of 6144 and 8192 elements, and their
+  // gradients are the same bit for bit: the ragged tail, whose scalar code rounds apart from the
+  // tiles', starts at the same element in all of them.
+  static constexpr int kUnit = N == 2 && M == 8 ? 24576 : kTile;
+  static_assert(kUnit % kTile == 0, "whole tiles");
+  static constexpr __host__ __device__ int64_t tiles(int64_t E) { return E / kUnit * (kUnit / kTile); }
   // rounds of one pair a thread up to which a lone tensor takes no tiles (tile_grid): 2:4
   // 0.5 M elements 3.1 against 4.6 us, 2.5 M 8.6 against 9.5, 3.5 M 10.0 against 9.9.  A
   // tile at M = 8 is one pair a thread as it is.
@@ -592,7 +598,7 @@ __device__ __forceinline__ BwdArgs multi_args(const BwdMulti& mm, int i) {
   a.dW = x.dW;
   a.hard_in = x.hard_in;
   a.E = x.E;
-  a.full_tiles = x.E / Cfg<N, M, AUX>::kTile;
+  a.full_tiles = Cfg<N, M, AUX>::tiles(x.E);
   a.tau = mm.tau;
   a.inv_tau = mm.inv_tau;
   a.np = x.np;
@@ -708,7 +714,7 @@ int launch_tiles(const BwdArgs& a, const BwdOptArgs& o, cudaStream_t stream, boo
   }
   const int64_t cap = int64_t(sm_count()) * cache.per_sm[dev];
   BwdArgs b = a;
-  b.full_tiles = a.E / C::kTile;
+  b.full_tiles = C::tiles(a.E);
   b.wait = !pdl && lone_pdl(stream);
   const int grid = tile_grid(b.full_tiles, a.E, M, C::kTailChunk, C::kTile, cap, pdl ? 0 : C::kTailRounds);
   return launch_maybe_pdl(kern, grid, C::kThreads, smem, stream, pdl || b.wait, b, o);
@@ -787,6 +793,7 @@ template <int N, int M>
 int launch_multi(const BwdCall* calls, int count, bool pdl) {
   const int kind = bwd_kind(calls[0]);
   const int64_t tile = kind != 0 ? Cfg<N, M, true>::kTile : Cfg<N, M, false>::kTile;
+  const auto tiles_of = [kind](int64_t E) { return kind != 0 ? Cfg<N, M, true>::tiles(E) : Cfg<N, M, false>::tiles(E); };
   const int64_t chunk = kind != 0 ? Cfg<N, M, true>::kTailChunk : Cfg<N, M, false>::kTailChunk;
   static thread_local BwdMulti mm;
   mm.count = count;
@@ -811,9 +818,9 @@ int launch_multi(const BwdCall* calls, int count, bool pdl) {
     x.tile0 = tiles;
     x.np = c.np;
     x.np.narrow = counters_narrow(c.np, c.E);
-    tiles += c.E / tile;
+    tiles += tiles_of(c.E);
     x.tail0 = tails;
-    tails += (c.E % tile / M + chunk - 1) / chunk;
+    tails += ((c.E - tiles_of(c.E) * tile) / M + chunk - 1) / chunk;
   }
   mm.total_tiles = tiles;
   mm.total_tails = tails;

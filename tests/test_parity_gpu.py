@@ -779,6 +779,29 @@ def test_compressed_2of4_export_bit_exact(roi, rows, cols):
     assert np.array_equal(_bits(meta), ref["meta"])
 
 
+# The forms of a pattern's backward have the same gradients whatever their launch shapes (2:8
+# has larger tiles with the straight-through dW and with AdamW): sizes on either side of whole
+# tiles of each.
+@pytest.mark.parametrize("N,M,tau", [(2, 8, 0.3), (2, 8, 1.0), (2, 4, 0.3), (4, 8, 0.5), (4, 8, 0.1), (8, 16, 0.2),
+                                     (16, 32, 0.2), (3, 4, 0.5)])
+@pytest.mark.parametrize("E", [6144 * 3, 8192 * 5, 24576 * 2 + 32 * 5, 24576 * 2 - 32 * 3, 6144 * 21 + 32])
+def test_forms_have_one_gradient(roi, N, M, tau, E):
+    import torch
+    W, phi, dWm, *_ = make(1, E, "normal", data_seed=E % 1000)
+    phi, W, dWm = phi.cuda(), W.cuda(), dWm.cuda()
+    st = roi.NoiseState(77, 4, 5, 0.5, 0)
+    hard = torch.zeros(roi.hard_words(1, E), dtype=torch.int32, device="cuda")
+    dW, plain, through, fused, m, v = (torch.zeros_like(x) for x in (W, phi, phi, phi, phi, phi))
+    roi.roi_mask_bwd(phi, W, st, N, M, dWm, tau, plain, None)
+    roi.roi_mask_bwd_st(phi, W, st, N, M, dWm, hard, tau, through, dW)
+    roi.roi_mask_bwd_adamw(phi.clone(), W, st, N, M, dWm, tau, m, v, roi.AdamW(1e-3, 0.9, 0.95, 1e-8, 0.05, 4), fused)
+    roi.roi_device_status()
+    assert torch.equal(plain, through)
+    # the fused form's is compiled apart: within 1e-6 of the group's largest
+    scale = plain.view(-1, M).abs().amax(1, keepdim=True)
+    assert torch.all((fused - plain).view(-1, M).abs() <= 1e-6 * scale + 1e-30)
+
+
 ADAMW_CASES = [
     (37, 1000, 2, 4, 1.0, "logw"),
     (29, 1536, 4, 8, 1.0, "normal"),
