@@ -12,6 +12,12 @@ namespace roi {
 namespace {
 
 constexpr int kThreads = 128;
+// CTAs per SM that the register budget is sized for: the padded group without a spill, and no
+// more registers than that (left to itself ptxas spills at MP = 4, forward and backward, and in
+// the backward at 8: 3:4 at 1536 x 1536 backward 15.8 us, 12.2 here; with 6 CTAs at MP = 4 the
+// forward takes 11.5 us, with 8 11.2).
+template <int MP>
+constexpr int kMinBlocks = MP == 4 ? 8 : MP <= 16 ? 4 : 2;
 // Padding members' keys (log2 units), the magnitude (squared) up to which real keys take the fast
 // relaxation, and the padding's largest offset from the second largest key over tau: 2^x is 0
 // there whatever tau is, and second_of never picks it (a real key's offset lies above the
@@ -140,6 +146,19 @@ __device__ __forceinline__ void any_keys(const AnyArgs& a, const int64_t* e0, V 
   }
 }
 
+// The keys of one group for ExactGroup, in natural-log units: phi / lambda stays finite up to the
+// type's largest value, where log2 units overflow (the lowest one masks a member out).
+__device__ __forceinline__ void exact_keys(const AnyArgs& a, int64_t e0, float* kap) {
+  uint4 block = {};
+  for (int l = 0; l < a.M; ++l) {
+    const uint64_t e = a.np.e_base + uint64_t(e0) + l;
+    const uint32_t w = uint32_t(e) & 3u;
+    if (w == 0u || l == 0) block = noise_block(a.np, e & ~uint64_t(3));
+    kap[l] = __fmaf_rn(a.phi[e0 + l], a.np.inv_lam,
+                       gumbel_from_word(w == 0u ? block.x : w == 1u ? block.y : w == 2u ? block.z : block.w));
+  }
+}
+
 // Sum over the other members, of which the padding's are 0.
 template <int MP, class V>
 __device__ __forceinline__ void others_of(const V (&x)[MP], V (&ex)[MP]) {
@@ -217,7 +236,7 @@ __device__ __forceinline__ int any_groups(const AnyArgs& a, int64_t t, int64_t (
 }
 
 template <int MP>
-__global__ void __launch_bounds__(kThreads) roi_any_fwd_kernel(AnyArgs a, bool words) {
+__global__ void __launch_bounds__(kThreads, kMinBlocks<MP>) roi_any_fwd_kernel(AnyArgs a, bool words) {
   using V = typename Lanes<MP>::V;
   constexpr int L = vlanes<V>();
   pdl_begin(a.wait);
@@ -247,11 +266,10 @@ __global__ void __launch_bounds__(kThreads) roi_any_fwd_kernel(AnyArgs a, bool w
         const bool rank = a.hard != nullptr || a.st;
         if ((flag >> h) & 1u) {
           float kn[MP];
-#pragma unroll
-          for (int l = 0; l < MP; ++l) kn[l] = k[l] * kLn2;  // natural-log keys
+          exact_keys(a, e0[h], kn);
           ExactGroup<MP - 1, MP> ex;
           ex.forward(kn, a.N, a.M, a.tau, s);
-          if (rank) bits[h] = topn_bits_dyn(k, a.N, a.M);
+          if (rank) bits[h] = topn_bits_dyn(kn, a.N, a.M);
         } else if (rank) {
           if constexpr (MP == 4) {
             bits[h] = topn_bits4(k, a.N);
@@ -314,7 +332,7 @@ __global__ void __launch_bounds__(kThreads) roi_any_fwd_kernel(AnyArgs a, bool w
 }
 
 template <int MP>
-__global__ void __launch_bounds__(kThreads) roi_any_bwd_kernel(AnyArgs a) {
+__global__ void __launch_bounds__(kThreads, kMinBlocks<MP>) roi_any_bwd_kernel(AnyArgs a) {
   using V = typename Lanes<MP>::V;
   constexpr int L = vlanes<V>();
   pdl_begin(a.wait);
@@ -388,7 +406,8 @@ __global__ void __launch_bounds__(kThreads) roi_any_bwd_kernel(AnyArgs a) {
       if ((flag >> h) & 1u) {
         float kn[MP], cc[MP];
 #pragma unroll
-        for (int l = 0; l < MP; ++l) kn[l] = lane_of(kap[l], h) * kLn2, cc[l] = lane_of(c[l], h);
+        for (int l = 0; l < MP; ++l) cc[l] = lane_of(c[l], h);
+        exact_keys(a, e0[h], kn);
         steps.exact.forward(kn, a.N, a.M, a.tau, s);
         steps.exact.backward(cc, a.N, a.M, a.tau, g);
 #pragma unroll
@@ -450,17 +469,6 @@ __global__ void __launch_bounds__(kThreads) roi_any_bwd_kernel(AnyArgs a) {
 // than 32 so that the frame is 16 bytes times an odd number and the warps' frames start in
 // different sets of the L1 (20:32 with 4864 B a thread 1516 / 4887 us, with 4880 1272 / 4061).
 constexpr int kExactKeys = 36;
-__device__ __forceinline__ void exact_keys(const AnyArgs& a, int64_t e0, float* kap) {
-  uint4 block = {};
-  for (int l = 0; l < a.M; ++l) {
-    const uint64_t e = a.np.e_base + uint64_t(e0) + l;
-    const uint32_t w = uint32_t(e) & 3u;
-    if (w == 0u || l == 0) block = noise_block(a.np, e & ~uint64_t(3));
-    kap[l] = key_log2(a.phi[e0 + l], uniform_from_word(w == 0u ? block.x : w == 1u ? block.y : w == 2u ? block.z : block.w),
-                      a.np.l2e_inv_lam);
-  }
-}
-
 // hard words are zeroed beforehand
 __global__ void __launch_bounds__(kThreads) roi_any_exact_fwd_kernel(AnyArgs a) {
   pdl_begin(a.wait);
@@ -470,7 +478,6 @@ __global__ void __launch_bounds__(kThreads) roi_any_exact_fwd_kernel(AnyArgs a) 
     float kap[kExactKeys], S[32];
     exact_keys(a, e0, kap);
     const uint32_t bits = a.hard != nullptr || a.st ? topn_bits_dyn(kap, a.N, a.M) : 0u;
-    for (int l = 0; l < a.M; ++l) kap[l] *= kLn2;  // natural-log keys
     ExactGroup<31, 32> ex;
     ex.forward(kap, a.N, a.M, a.tau, S);
     for (int l = 0; l < a.M; ++l) {
@@ -494,10 +501,7 @@ __global__ void __launch_bounds__(kThreads) roi_any_exact_bwd_kernel(AnyArgs a) 
     const int64_t e0 = g * a.M;
     float kap[kExactKeys], c[32], S[32], dk[32];
     exact_keys(a, e0, kap);
-    for (int l = 0; l < a.M; ++l) {
-      kap[l] *= kLn2;  // natural-log keys
-      c[l] = __fmul_rn(bf16_bits_to_float(a.dWm[e0 + l]), bf16_bits_to_float(a.W[e0 + l]));
-    }
+    for (int l = 0; l < a.M; ++l) c[l] = __fmul_rn(bf16_bits_to_float(a.dWm[e0 + l]), bf16_bits_to_float(a.W[e0 + l]));
     ExactGroup<31, 32> ex;
     ex.forward(kap, a.N, a.M, a.tau, S);
     ex.backward(c, a.N, a.M, a.tau, dk);

@@ -120,8 +120,8 @@ __device__ __forceinline__ void issue_chunk(const CUtensorMap* tm_phi, const CUt
 
 // Relax this thread's pair of chunk kc from the staged logits and write
 // bf16(W * S) into the chunk's A tile (core-matrix layout).  EXACT: every group by ExactGroup,
-// from keys that are formed in scalar code, as the mask forward's kernels for a tau too small
-// for the WIDE relaxation (roi_any.cu) form them.
+// on the keys that the mask forward's kernels for a tau too small for the WIDE relaxation
+// (exact_keys in roi_any.cu) form.
 template <int N, int M, bool TAU1, bool WIDE, bool EXACT>
 __device__ __forceinline__ void chunk_masked_weights(const LinArgs& a, uint8_t* smem, const LinSmem& L, int stage,
                                                      int64_t row0, int kc) {
@@ -175,7 +175,7 @@ __device__ __forceinline__ void chunk_masked_weights(const LinArgs& a, uint8_t* 
       float kn[M], sh[M];
 #pragma unroll
       for (int l = 0; l < M; ++l)
-        kn[l] = __fmul_rn(key_log2(h == 0 ? ph[0][l] : ph[1][l], uniform_from_word(h == 0 ? x[0][l] : x[1][l]), a.np.l2e_inv_lam), kLn2);
+        kn[l] = __fmaf_rn(h == 0 ? ph[0][l] : ph[1][l], a.np.inv_lam, gumbel_from_word(h == 0 ? x[0][l] : x[1][l]));
       ExactGroup<N, M> ex;
       ex.forward(kn, N, M, a.tau, sh);
 #pragma unroll

@@ -493,6 +493,44 @@ def test_tiny_temperatures(roi, N, M, tau):
     assert np.abs(got["dlogits"]).max() <= 2.0**-24 * float((W.float() * dWm.float()).abs().max())
 
 
+# The type's lowest value as a mask, and its largest as a pin: such a member has no weight (and
+# ranks above -inf), or comes first; the others are as without it.  Patterns without a kernel of
+# their own, whose keys stay finite there.
+# (At tau = 1 and N > 1 a member that leads by 3e38 comes back at its runner-up's level, the
+# difference of two such numbers, which neither precision holds.)
+@pytest.mark.parametrize("N,M,tau", [(1, 2, 1.5), (3, 4, 1.5), (1, 4, 1.0), (2, 3, 1.5), (3, 7, 1.5), (1, 8, 1.0),
+                                     (5, 12, 1.5), (4, 16, 1.5), (18, 24, 1.5)])
+def test_logits_at_the_ends_of_the_type(roi, N, M, tau):
+    import torch
+    rows, groups = 6, 43
+    W, phi, dWm, ph, Wb, dWb = make(rows, groups * M, "normal", data_seed=M + N)
+    low, high = torch.finfo(torch.float32).min, 3.0e38
+    phi = phi.clone().view(rows, groups, M)
+    phi[0, :, 0] = low
+    phi[1, :, M - 1] = high
+    phi[2, :, :M - N] = low
+    phi[3, :, 0], phi[3, :, M - 1] = float("-inf"), low
+    phi[4, ::3, :] = low
+    phi = phi.view(rows, groups * M).contiguous()
+    got = gpu_run(roi, phi, W, dWm, N, M, tau, roi.NoiseState(5, 6, 7, 1.0, 0))
+    with np.errstate(all="ignore"):
+        ref = O.mask_fwd(phi.numpy(), Wb, N, M, tau, 5, 6, tensor_id=7)
+        refb = O.mask_bwd(phi.numpy(), Wb, dWb, N, M, tau, 5, 6, tensor_id=7, dtype=np.float32)
+    keep = lambda r: O.unpack_bits(r["hard_bits"], phi.numel()).reshape(rows, groups, M)  # noqa: E731
+    # a group of equal keys at the lowest value (its noise lost) is ranked by index, as its
+    # float64 keys, which the noise still separates, are not
+    whole = np.ones((rows, groups), bool)
+    whole[4, ::3] = False
+    whole[2] = N == 1
+    assert np.array_equal(keep(got)[whole], keep(ref)[whole])
+    assert np.array_equal(np.isnan(got["soft"]), np.isnan(ref["soft"]))
+    ok = ~np.isnan(ref["soft"]).reshape(rows, groups, M) & whole[:, :, None]
+    assert np.allclose(got["soft"].reshape(rows, groups, M)[ok], ref["soft"].reshape(rows, groups, M)[ok], atol=2e-5)
+    g, h = got["dlogits"].reshape(rows, groups, M)[:3], refb["dlogits"].reshape(rows, groups, M)[:3]
+    fin = np.isfinite(h) & whole[:3, :, None]
+    assert np.all(np.isfinite(g[fin])) and np.allclose(g[fin], h[fin], atol=1e-4 * np.abs(h[fin]).max())
+
+
 # Large temperatures (any finite tau is accepted): all weights of a group tend to 1 / M, and
 # the members that pad a group to 4, 8, 16 or 32 have none (a padding key that is divided by
 # tau like the others takes an eighth of 3:7's sum at tau = 1e20).
