@@ -251,8 +251,10 @@ roi_status roi_export_compressed_2of4(const float* logits, const roi_bf16* W, in
 /* Masked linear forward: the layer's product with the masked weights (Eq. 5),
  *     Y[t, r] = sum_c X[t, c] Wm[r, c],   Wm = bf16_rne(float(W) * S),
  * where S is the relaxed mask of roi_mask_fwd_ex for the same (logits, W, N, M,
- * tau, st), bit for bit, formed in the prologue of a tensor-core GEMM: Wm is
- * never written to memory and the logits and W are read once.  The sum runs in
+ * tau, st), formed in the prologue of a tensor-core GEMM: Wm is never written
+ * to memory and the logits and W are read once.  Wm is the mask forward's bit for
+ * bit, except in the last rows*cols % 8192 elements of an M = 8 tensor, which the
+ * mask forward rounds in another order (S apart by last bits).  The sum runs in
  * float32 on the tensor cores (products of bf16 exact, accumulation order the
  * hardware's), Y is float32.  If a kernel of the call gives up a wait
  * (roi_device_status then returns ROI_ERR_TIMEOUT), out_Y is undefined: the

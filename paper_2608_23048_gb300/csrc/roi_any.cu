@@ -464,10 +464,10 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks<MP>) roi_any_bwd_kernel(A
 
 // Every group by ExactGroup, one a thread, members in local memory (1536 x 1536, tau = 0.05,
 // forward / backward: 18:24 1341 / 3828 us in place behind a fast relaxation that was thrown
-// away, 941 / 2529 here; 20:32 1531 / 4906, 1272 / 4061).  What bounds these is the L1's
+// away, 941 / 2529 here; 20:32 1531 / 4906, 1297 / 4070).  What bounds these is the L1's
 // bandwidth for the members.  A warp's frame is 32 times a thread's: the keys' array is longer
 // than 32 so that the frame is 16 bytes times an odd number and the warps' frames start in
-// different sets of the L1 (20:32 with 4864 B a thread 1516 / 4887 us, with 4880 1272 / 4061).
+// different sets of the L1 (20:32 with 4864 B a thread 1516 / 4887 us, with 4880 1297 / 4070).
 constexpr int kExactKeys = 36;
 // hard words are zeroed beforehand
 __global__ void __launch_bounds__(kThreads) roi_any_exact_fwd_kernel(AnyArgs a) {

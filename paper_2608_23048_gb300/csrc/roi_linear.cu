@@ -14,7 +14,8 @@
 // to the stage's `mma` mbarrier and refills the stage when they are done.  The
 // compute warps never wait for each other: each thread relaxes one pair of
 // groups per chunk from shared memory (the same keys, noise and rounding as
-// roi_mask_fwd, so Wm is bit-identical to its output), writes their bf16
+// the tiles of roi_mask_fwd, so Wm is bit-identical to its output; the ragged tail
+// of its M = 8 forward alone is scalar code and rounds apart), writes their bf16
 // products into the chunk's A tile and arrives.  Layers with few row blocks
 // split K across CTAs, which write fp32 partials; a second launch, dependent on
 // the first (programmatic dependent launch: it is scheduled while the GEMM drains
